@@ -7,16 +7,26 @@
 //   slots[n_bins * B]  uint64  key << 32 | value; all-ones = empty
 //   meta[n_bins]       uint32  per-bin metadata word:
 //       two-choice: bits 0-7 claim flags (Sec. 8), 8-15 duplicate marks
-//       (Sec. 4), 16-19 spawn count (Sec. 5), 20-27 hit counter (Sec. 6),
-//       28-31 version;  d-ary: bit 0 claim flag, bits 8-15 rattle counter of
+//       (Sec. 4), 16-19 spawn count (Sec. 5), 20-27 hit counter (Sec. 6)
+//       less the bin's occupied slots (below), 28-31 version;  d-ary: bit 0 claim flag, bits 8-15 rattle counter of
 //       the resident key (Sec. 7), 28-31 version.
+//
+// Queue-kicking's hit counter h counts every placement into its bin.  The
+// word holds h minus the number of occupied slots, modulo 256: a placement
+// into a free slot moves both by one, so it leaves the word alone, and a new
+// key that finds room (most of a fill) writes only its slot.  A kick-out or
+// an overwritten duplicate adds one (h moves, the occupancy does not), a
+// delete adds one (the occupancy falls, h stays).  h itself is needed only
+// of full bins, where it is the field plus B, and in exported words, where
+// the occupied slots are added (k_convert_hits).  The add that used to
+// advance h was a random read-modify-write of a 64 MiB array per new key.
 //
 // Every write to an occupied slot happens while its claim flag is held.  A
 // claim is a compare-and-swap of the whole metadata word from the value read
 // when the bin was viewed, so a successful claim also shows that nothing in
 // the bin changed since the view -- every release adds one to the version
 // field (the release also folds in the duplicate/rattle update of the slot),
-// and the hit counter of queue-kicking moves on every insertion -- unless
+// and the hit counter of queue-kicking moves on every kick-out -- unless
 // the word came back to the value seen (the 4-bit version wraps after 16
 // releases).  The writes themselves are therefore 64-bit compare-and-swaps
 // from the records the plan saw, undone if one fails, which closes that
@@ -384,7 +394,9 @@ __device__ __forceinline__ int nth_bit(uint32_t mask, uint32_t i) {
 }
 
 __device__ __forceinline__ uint32_t spawn_of(uint32_t m) { return (m >> SPAWN_SHIFT) & 15u; }
-__device__ __forceinline__ uint32_t hit_of(uint32_t m) { return (m >> HIT_SHIFT) & 255u; }
+// the hit counter of a full bin of B slots (the field holds it less B)
+template <int B>
+__device__ __forceinline__ uint32_t hit_of_full(uint32_t m) { return ((m >> HIT_SHIFT) + B) & 255u; }
 __device__ __forceinline__ uint32_t rattle_of(uint32_t m) { return (m >> RATTLE_SHIFT) & 255u; }
 
 }  // namespace ck

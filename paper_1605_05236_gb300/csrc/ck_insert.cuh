@@ -165,7 +165,8 @@ __device__ __forceinline__ int plan_room(const DevTable& t, Ctx& c) {
 }
 
 // Claim slot s of `bin` by CAS from the viewed metadata word m (hit: the
-// claim also advances queue-kicking's hit counter) and append the entry.
+// claim also advances queue-kicking's hit counter, for a slot that is
+// occupied) and append the entry.
 __device__ __forceinline__ bool claim(const DevTable& t, Ctx& c, uint32_t bin, uint32_t m, int s, uint8_t kind,
                                       bool hit, uint64_t content, uint32_t old_r = 0, uint32_t new_r = 0) {
   uint32_t desired = m + (hit ? HIT_ONE : 0u) + (1u << s);
@@ -223,19 +224,17 @@ __device__ __forceinline__ bool claim_again(const DevTable& t, Ctx& c, uint32_t 
 }
 
 // A new key straight into free slot s of `bin` (tables without ghosts):
-// one 64-bit compare-and-swap of the slot from empty to the record, and for
-// queue-kicking a relaxed add that advances the bin's hit counter (Sec. 6:
-// every placement into a bin counts).  No claim is taken and the version
-// does not move: the key moves nothing, so no reader that proves a miss and
+// one 64-bit compare-and-swap of the slot from empty to the record.  (For
+// queue-kicking the bin's hit counter advances with its occupancy, which
+// the metadata word need not show.)  No claim is taken and the version does
+// not move: the key moves nothing, so no reader that proves a miss and
 // no planner's claim depends on it (a chain that had claimed this slot as
 // its terminal finds it taken when its compare-and-swap commits, and starts
 // again).  With one insertion in flight the slot and the policy's metadata
 // end exactly as a claim and its release would leave them.
 template <int B>
-__device__ __forceinline__ bool place_direct(const DevTable& t, Ctx& c, uint32_t bin, int s, bool hit) {
-  if (!cas_slot(t.slots + (uint64_t)bin * B + s, EMPTY, c.krec)) return false;
-  if (hit) red_relaxed(t.meta + bin, HIT_ONE);
-  return true;
+__device__ __forceinline__ bool place_direct(const DevTable& t, Ctx& c, uint32_t bin, int s) {
+  return cas_slot(t.slots + (uint64_t)bin * B + s, EMPTY, c.krec);
 }
 
 // Abandon the plan: drop every claim (and hit increment).  Nothing was
@@ -367,13 +366,13 @@ __device__ __forceinline__ int dead_end(Ctx& c) {
 // otherwise each claim its first bin, fail on the other's, release, and
 // meet again on every retry.
 __device__ __forceinline__ bool claim_ghost_pair(const DevTable& t, Ctx& c, uint32_t b0, uint32_t m0, int s0,
-                                                 uint32_t b1, uint32_t m1, int s1, bool hit) {
+                                                 uint32_t b1, uint32_t m1, int s1) {
   if (b1 < b0) {
-    if (!claim(t, c, b1, m1, s1, K_GHOST, hit, EMPTY)) return false;
-    return claim(t, c, b0, m0, s0, K_GHOST, hit, EMPTY);
+    if (!claim(t, c, b1, m1, s1, K_GHOST, false, EMPTY)) return false;
+    return claim(t, c, b0, m0, s0, K_GHOST, false, EMPTY);
   }
-  if (!claim(t, c, b0, m0, s0, K_GHOST, hit, EMPTY)) return false;
-  return claim(t, c, b1, m1, s1, K_GHOST, hit, EMPTY);
+  if (!claim(t, c, b0, m0, s0, K_GHOST, false, EMPTY)) return false;
+  return claim(t, c, b1, m1, s1, K_GHOST, false, EMPTY);
 }
 
 __device__ __forceinline__ bool plan_has_bin(const Ctx& c, uint32_t bin) {
@@ -484,11 +483,11 @@ __device__ int insert_random2(const DevTable& t, Ctx& c) {
     load_view_fast<B>(t, b0, v0);
     c.viewed++;
     int s = lowest(free_mask<B>(v0));
-    if (s >= 0) return place_direct<B>(t, c, b0, s, false) ? (int)ST_OK : (int)ST_CONFLICT;
+    if (s >= 0) return place_direct<B>(t, c, b0, s) ? (int)ST_OK : (int)ST_CONFLICT;
     load_view_fast<B>(t, b1, v1);
     c.viewed++;
     s = lowest(free_mask<B>(v1));
-    if (s >= 0) return place_direct<B>(t, c, b1, s, false) ? (int)ST_OK : (int)ST_CONFLICT;
+    if (s >= 0) return place_direct<B>(t, c, b1, s) ? (int)ST_OK : (int)ST_CONFLICT;
     // both full: the views as read serve the walk (unordered metadata and
     // slots are fine: every move is re-validated after its claim)
   } else {
@@ -496,7 +495,7 @@ __device__ int insert_random2(const DevTable& t, Ctx& c) {
     c.viewed += 2;
     uint32_t f0 = free_mask<B>(v0), f1 = free_mask<B>(v1);
     if (f0 && f1) {
-      if (!claim_ghost_pair(t, c, b0, v0.m, lowest(f0), b1, v1.m, lowest(f1), false)) return ST_CONFLICT;
+      if (!claim_ghost_pair(t, c, b0, v0.m, lowest(f0), b1, v1.m, lowest(f1))) return ST_CONFLICT;
       c.ghosts_made++;
       return ST_OK;
     }
@@ -572,7 +571,8 @@ __device__ int insert_random2(const DevTable& t, Ctx& c) {
 // ------------------------------------------------------------------
 // Every placement into a bin takes its hit counter h and increments it (the
 // claim of a kicked slot and the increment are one compare-and-swap, the GPU
-// form of the paper's fetch-and-add scheduling).  A record goes to the
+// form of the paper's fetch-and-add scheduling; a placement into a free slot
+// increments it by filling the slot).  A record goes to the
 // lowest free slot (in insert-only tables the bin fills in slot order, so
 // this is slot h mod B); a full bin gives up the record at h mod B, the one
 // that has been there longest -- also when this chain placed it there on an
@@ -596,7 +596,7 @@ __device__ int insert_queue(const DevTable& t, Ctx& c) {
       bool first = __popc(g0) >= __popc(g1);
       uint32_t x = first ? b0 : b1;
       int s = lowest(first ? g0 : g1);
-      return place_direct<B>(t, c, x, s, true) ? (int)ST_OK : (int)ST_CONFLICT;
+      return place_direct<B>(t, c, x, s) ? (int)ST_OK : (int)ST_CONFLICT;
     }
     // both full: the metadata words, with the slots as read (unordered is
     // fine: every move is re-validated after its claim)
@@ -611,7 +611,7 @@ __device__ int insert_queue(const DevTable& t, Ctx& c) {
   if (GHOST && f0 > 0 && f1 > 0) {
     int s0 = lowest(fm0);
     int s1 = lowest(fm1);
-    if (!claim_ghost_pair(t, c, b0, v0.m, s0, b1, v1.m, s1, true)) return ST_CONFLICT;
+    if (!claim_ghost_pair(t, c, b0, v0.m, s0, b1, v1.m, s1)) return ST_CONFLICT;
     c.ghosts_made++;
     return ST_OK;
   }
@@ -626,7 +626,7 @@ __device__ int insert_queue(const DevTable& t, Ctx& c) {
     x = first ? b0 : b1;
     vx = first ? v0 : v1;
   } else {
-    bool first = hit_of(v0.m) <= hit_of(v1.m);
+    bool first = hit_of_full<B>(v0.m) <= hit_of_full<B>(v1.m);
     x = first ? b0 : b1;
     vx = first ? v0 : v1;
   }
@@ -639,11 +639,11 @@ __device__ int insert_queue(const DevTable& t, Ctx& c) {
   for (;;) {
     int tries = 0;
     for (;;) {  // one step at bin x: free slot, duplicate, or victim from hit mod B
-      uint32_t h = hit_of(vx.m) % B;
+      uint32_t h = hit_of_full<B>(vx.m) % B;  // used when no slot is free
       uint32_t fm = free_mask<B>(vx);
       const uint64_t chk = pend ? ld_slot(pend) : 0;
       if (fm) {
-        if (claim(t, c, x, vx.m, lowest(fm), K_MOVE, true, EMPTY))
+        if (claim(t, c, x, vx.m, lowest(fm), K_MOVE, false, EMPTY))
           return (pend && chk != pend_v) ? (int)ST_CONFLICT : (int)ST_OK;
       } else if (GHOST && dup_mask<B>(vx)) {
         const int r = take_dup<B>(t, c, x, vx, first_from<B>(dup_mask<B>(vx), h), true);

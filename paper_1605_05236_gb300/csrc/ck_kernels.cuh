@@ -225,6 +225,7 @@ __device__ __forceinline__ int delete_one(const DevTable& t, uint32_t key, DelPl
     }
     for (int i = 0; i < p.n; i++) {
       uint32_t delta = VER_ONE - (1u << p.slot[i]);
+      if (B > 1 && t.policy == P_QUEUE) delta += HIT_ONE;               // one slot fewer, the same hits
       if (B == 1) delta -= (uint32_t)p.old_r[i] << RATTLE_SHIFT;        // the bin forgets r(x)
       else if (p.old_r[i]) delta -= 1u << (DUP_SHIFT + p.slot[i]);       // duplicate mark goes too
       add_release(t.meta + p.bin[i], delta);
@@ -577,6 +578,50 @@ static __global__ void __launch_bounds__(256) k_lookup_dary(DevTable t, const ui
     if (hits_sh) atomicAdd(t.counters + C_LOOKUP_HITS, hits_sh);
     if (cnt_sh) atomicAdd(t.counters + C_LOOKUPS, cnt_sh);
   }
+}
+
+// The hit field of every metadata word, for an export (sign 1: the bin's
+// occupied slots added, which makes it queue-kicking's hit counter) and back
+// (sign -1).  B is 4 or 8.
+static __global__ void __launch_bounds__(256) k_convert_hits(const uint64_t* slots, uint32_t* meta, uint64_t n_bins,
+                                                             uint32_t B, int sign) {
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; b < n_bins; b += stride) {
+    uint32_t occupied = 0;
+    for (uint32_t s = 0; s < B; s++) occupied += slots[b * B + s] != EMPTY;
+    const uint32_t m = meta[b];
+    const uint32_t h = ((m >> HIT_SHIFT) + (uint32_t)sign * occupied) & 255u;
+    meta[b] = (m & ~(255u << HIT_SHIFT)) | (h << HIT_SHIFT);
+  }
+}
+
+// Metadata words to host memory in the exported form (hit counters of
+// queue-kicking tables), the device's words as they were afterwards.  On the
+// legacy default stream, with no other work on the table.
+inline cudaError_t copy_meta_out(const DevTable& t, uint32_t* h_meta) {
+  const bool convert = t.policy == P_QUEUE && t.B > 1;
+  const unsigned grid = (unsigned)(t.n_bins < 256 * 4096 ? (t.n_bins + 255) / 256 : 4096);
+  if (convert) {
+    k_convert_hits<<<grid, 256>>>(t.slots, t.meta, t.n_bins, t.B, 1);
+    const cudaError_t e1 = cudaGetLastError();
+    if (e1 != cudaSuccess) return e1;
+  }
+  cudaError_t e = cudaMemcpy(h_meta, t.meta, t.n_bins * sizeof(uint32_t), cudaMemcpyDeviceToHost);
+  if (convert) {
+    k_convert_hits<<<grid, 256>>>(t.slots, t.meta, t.n_bins, t.B, -1);
+    const cudaError_t e2 = cudaStreamSynchronize(nullptr);  // callers may go on on another stream
+    if (e == cudaSuccess) e = e2;
+  }
+  return e;
+}
+
+// Words as exported, back into the device's form (the slots are in place).
+inline cudaError_t convert_meta_in(const DevTable& t) {
+  if (t.policy != P_QUEUE || t.B == 1) return cudaSuccess;
+  const unsigned grid = (unsigned)(t.n_bins < 256 * 4096 ? (t.n_bins + 255) / 256 : 4096);
+  k_convert_hits<<<grid, 256>>>(t.slots, t.meta, t.n_bins, t.B, -1);
+  const cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? cudaStreamSynchronize(nullptr) : e;
 }
 
 template <int B>

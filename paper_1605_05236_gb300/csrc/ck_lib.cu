@@ -473,9 +473,7 @@ int ck_export(ck_table* t, uint64_t* h_slots, uint32_t* h_meta) {
   if (h_slots && cudaMemcpy(h_slots, t->dt.slots, t->dt.total_slots * sizeof(uint64_t), cudaMemcpyDeviceToHost) !=
                      cudaSuccess)
     return CK_ECUDA;
-  if (h_meta &&
-      cudaMemcpy(h_meta, t->dt.meta, t->dt.n_bins * sizeof(uint32_t), cudaMemcpyDeviceToHost) != cudaSuccess)
-    return CK_ECUDA;
+  if (h_meta && copy_meta_out(t->dt, h_meta) != cudaSuccess) return CK_ECUDA;
   return CK_OK;
 }
 
@@ -508,7 +506,8 @@ int ck_import(ck_table* t, const uint64_t* h_slots, const uint32_t* h_meta) {
   if (cudaMemcpy(t->dt.slots, h_slots, t->dt.total_slots * sizeof(uint64_t), cudaMemcpyHostToDevice) !=
           cudaSuccess ||
       cudaMemcpy(t->dt.meta, h_meta, nb * sizeof(uint32_t), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemset(t->dt.counters, 0, COUNTER_WORDS * sizeof(uint64_t)) != cudaSuccess)
+      cudaMemset(t->dt.counters, 0, COUNTER_WORDS * sizeof(uint64_t)) != cudaSuccess ||
+      convert_meta_in(t->dt) != cudaSuccess)
     return CK_ECUDA;
   // a ghost pair is one key stored twice, both copies marked
   const unsigned long long size_ghosts[2] = {occupied - dups / 2, dups / 2};

@@ -551,8 +551,7 @@ int ck_multi_export(ck_multi* m, uint32_t table, uint64_t* h_slots, uint32_t* h_
   const DevTable& t = m->host_tables[table];
   if (h_slots && cudaMemcpy(h_slots, t.slots, t.total_slots * sizeof(uint64_t), cudaMemcpyDeviceToHost) != cudaSuccess)
     return CK_ECUDA;
-  if (h_meta && cudaMemcpy(h_meta, t.meta, t.n_bins * sizeof(uint32_t), cudaMemcpyDeviceToHost) != cudaSuccess)
-    return CK_ECUDA;
+  if (h_meta && copy_meta_out(t, h_meta) != cudaSuccess) return CK_ECUDA;
   return CK_OK;
 }
 

@@ -268,8 +268,8 @@ __device__ int insert_search(const DevTable& t, Ctx& c, uint8_t* region) {
     load_view_fast<B>(t, b1, v1);
     c.viewed += 2;
     uint32_t g0 = free_mask<B>(v0), g1 = free_mask<B>(v1);
-    if (g0) return place_direct<B>(t, c, b0, lowest(g0), false) ? (int)ST_OK : (int)ST_CONFLICT;
-    if (g1) return place_direct<B>(t, c, b1, lowest(g1), false) ? (int)ST_OK : (int)ST_CONFLICT;
+    if (g0) return place_direct<B>(t, c, b0, lowest(g0)) ? (int)ST_OK : (int)ST_CONFLICT;
+    if (g1) return place_direct<B>(t, c, b1, lowest(g1)) ? (int)ST_OK : (int)ST_CONFLICT;
     fence_acquire();
     load_slots<B>(t, b0, v0);
     load_slots<B>(t, b1, v1);
@@ -280,7 +280,7 @@ __device__ int insert_search(const DevTable& t, Ctx& c, uint8_t* region) {
   uint32_t f0 = free_mask<B>(v0), f1 = free_mask<B>(v1);
   if (GHOST) {
     if (f0 && f1) {
-      if (!claim_ghost_pair(t, c, b0, v0.m, lowest(f0), b1, v1.m, lowest(f1), false)) return ST_CONFLICT;
+      if (!claim_ghost_pair(t, c, b0, v0.m, lowest(f0), b1, v1.m, lowest(f1))) return ST_CONFLICT;
       c.ghosts_made++;
       return ST_OK;
     }

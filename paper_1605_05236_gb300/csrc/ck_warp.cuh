@@ -314,9 +314,9 @@ __global__ void __launch_bounds__(WARP_BLOCK, 8) k_insert_warp(DevTable t, const
         c.viewed += 2;
         const uint32_t g0 = free_mask<B>(v0), g1 = free_mask<B>(v1);
         if (g0) {
-          at = place_direct<B>(t, c, b0, lowest(g0), false) ? (int)ST_OK : (int)ST_CONFLICT;
+          at = place_direct<B>(t, c, b0, lowest(g0)) ? (int)ST_OK : (int)ST_CONFLICT;
         } else if (g1) {
-          at = place_direct<B>(t, c, b1, lowest(g1), false) ? (int)ST_OK : (int)ST_CONFLICT;
+          at = place_direct<B>(t, c, b1, lowest(g1)) ? (int)ST_OK : (int)ST_CONFLICT;
         } else {
           fence_acquire();
           load_slots<B>(t, b0, v0);
