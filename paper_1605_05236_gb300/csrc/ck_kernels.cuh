@@ -2,7 +2,7 @@
 // (every policy), lookup and delete (Kuszmaul, arXiv:1605.05236, Sec. 1,
 // Sec. 3-8), plus their per-batch counters.
 #pragma once
-#include "ck_search.cuh"
+#include "ck_look.cuh"
 
 namespace ck {
 
@@ -170,6 +170,15 @@ __device__ __forceinline__ bool swap_copies(const DevTable& t, const DelPlan& p,
 // (status 2).
 constexpr int DELETE_ATTEMPTS = 1024;
 
+// The metadata words of a key's bins, all read before any of the bins'
+// slots: a record that moves between the key's bins moves under its source's
+// claim, whose release changes that bin's word, but the free slot it moves to
+// need not be claimed (ck_walk.cuh), so both words have to be from before.
+__device__ __forceinline__ void read_words(const DevTable& t, const uint32_t* b, uint32_t nb, uint32_t* seen) {
+  for (uint32_t j = 0; j < nb; j++) seen[j] = ld_relaxed(t.meta + b[j]);
+  fence_acquire();
+}
+
 template <int B>
 __device__ __forceinline__ int delete_one(const DevTable& t, uint32_t key, DelPlan& p, uint32_t& ghost_removed) {
   uint32_t b[4];
@@ -181,11 +190,11 @@ __device__ __forceinline__ int delete_one(const DevTable& t, uint32_t key, DelPl
     bool conflict = false, any = false;
     int dup_copies = 0;
     uint32_t seen[4];
+    read_words(t, b, nb, seen);
     for (uint32_t j = 0; j < nb && !conflict; j++) {
       View<B> v;
-      load_view<B>(t, b[j], v);
-      uint32_t m = v.m;
-      seen[j] = m;
+      load_slots<B>(t, b[j], v);
+      const uint32_t m = seen[j];
       uint32_t add = 0;
 #pragma unroll
       for (int s = 0; s < B; s++) {
@@ -251,11 +260,11 @@ __device__ __forceinline__ int update_one(const DevTable& t, uint32_t key, uint6
     p.n = 0;
     bool conflict = false, any = false;
     uint32_t seen[4];
+    read_words(t, b, nb, seen);
     for (uint32_t j = 0; j < nb && !conflict; j++) {
       View<B> v;
-      load_view<B>(t, b[j], v);
-      uint32_t m = v.m;
-      seen[j] = m;
+      load_slots<B>(t, b[j], v);
+      const uint32_t m = seen[j];
       uint32_t add = 0;
 #pragma unroll
       for (int s = 0; s < B; s++) {
@@ -327,20 +336,22 @@ __global__ void __launch_bounds__(256, insert_blocks_per_sm<B, POL>()) k_insert(
                                                 uint32_t* __restrict__ viewed_out, uint64_t load_base,
                                                 uint32_t upsert) {
   asm volatile("griddepcontrol.launch_dependents;");
-  __shared__ unsigned int h_views[HIST_BUCKETS];
-  __shared__ unsigned int h_cnt[HIST_BUCKETS];
-  __shared__ unsigned int h_chain[CHAIN_BUCKETS];
-  __shared__ unsigned long long bc[C_N];
+  __shared__ BlockTally bt;
   __shared__ unsigned long long s_next;  // next key of this block's range
   __shared__ int s_slab[SLABS_PER_BLOCK], s_long;
-  for (int i = threadIdx.x; i < HIST_BUCKETS; i += blockDim.x) h_views[i] = h_cnt[i] = 0;
-  for (int i = threadIdx.x; i < CHAIN_BUCKETS; i += blockDim.x) h_chain[i] = 0;
-  for (int i = threadIdx.x; i < C_N; i += blockDim.x) bc[i] = 0;
+  // searches on two-choice tables take their keys through a first look
+  // (ck_look.cuh); the other kernels built from this template are for ghosts,
+  // upserts and single-slot bins, whose keys need claims from the start
+  constexpr bool LOOK = B > 1 && !GHOST && !SERIAL && (POL == P_BFS || POL == P_SORTED || POL == P_HYBRID);
+  __shared__ LookMaybe<LOOK> ls;
+  const bool look = LOOK && !upsert;
+  bt.clear();
   // each block owns a contiguous range of the batch; its threads pull keys
   // from it one at a time, so a thread held up by a long chain does not
   // hold up the others
   const uint64_t per = (n + gridDim.x - 1) / gridDim.x;
   const uint64_t lo = min(n, (uint64_t)blockIdx.x * per), hi = min(n, lo + per);
+  if constexpr (LOOK) ls.begin(t, lo, load_base);
   if (threadIdx.x == 0) {
     s_next = lo;
     const int need = (int)((blockDim.x + SLAB - 1) / SLAB);
@@ -365,7 +376,6 @@ __global__ void __launch_bounds__(256, insert_blocks_per_sm<B, POL>()) k_insert(
                                                    SEARCH_REGION
                                    : nullptr;
   if (t.scratch && !region) usable = false;
-  const unsigned long long size_base = load_base;
 
   // per-thread tallies of the counts every key adds to (32-bit: a thread
   // handles far fewer than 2^32 keys or bin views in one launch), flushed
@@ -373,14 +383,12 @@ __global__ void __launch_bounds__(256, insert_blocks_per_sm<B, POL>()) k_insert(
   // block's counters as they happen, which keeps them out of registers for
   // the whole loop
   uint32_t ok = 0, viewed = 0, viewed_all = 0;
-  for (;;) {
-    uint64_t i = atomicAdd(&s_next, 1ull);
-    if (i >= hi) break;
+  auto insert = [&](uint64_t i) {
     uint32_t key = keys[i];
     if (key == RESERVED_KEY) {
       if (status) status[i] = ST_INVALID;
       if (viewed_out) viewed_out[i] = 0;
-      continue;
+      return;
     }
     Ctx c;
     c.key = key;
@@ -389,13 +397,13 @@ __global__ void __launch_bounds__(256, insert_blocks_per_sm<B, POL>()) k_insert(
       DelPlan up;
       int r = update_one<B>(t, key, c.krec, up);
       if (r != 0) {
-        atomicAdd(&bc[r == 1 ? C_UPDATES : C_INS_ABORTED], 1ull);
+        atomicAdd(&bt.bc[r == 1 ? C_UPDATES : C_INS_ABORTED], 1ull);
         if (status) status[i] = (uint8_t)(r == 1 ? ST_UPDATED : ST_ABORTED);
         if (viewed_out) viewed_out[i] = 0;
-        continue;
+        return;
       }
     }
-    c.viewed = 0;
+    c.viewed = c.viewed0 = 0;
     c.reviews = 0;
     uint32_t aborts = 0;
     // concurrent mode retries a failed attempt (up to three times): other
@@ -403,20 +411,6 @@ __global__ void __launch_bounds__(256, insert_blocks_per_sm<B, POL>()) k_insert(
     // the serial replay never retries
     int st = usable ? insert_one<B, POL, GHOST>(t, c, region, aborts, local_e, local_cap, !SERIAL)
                     : (int)ST_ABORTED;
-    if (st == ST_OK) {
-      ok++;
-      if (c.kicks) {
-        atomicAdd(&bc[C_KICKS], (unsigned long long)c.kicks);
-        atomicMax(&bc[C_CHAIN_MAX], (unsigned long long)c.kicks);
-      }
-      atomicAdd(&h_chain[chain_bucket(c.kicks)], 1u);
-      if (c.ghosts_made) atomicAdd(&bc[C_GHOSTS_MADE], (unsigned long long)c.ghosts_made);
-      if (c.dup_evict) atomicAdd(&bc[C_DUP_EVICT], (unsigned long long)c.dup_evict);
-    } else {
-      atomicAdd(&bc[st == ST_FAILED ? C_INS_FAILED : C_INS_ABORTED], 1ull);
-    }
-    if (aborts) atomicAdd(&bc[C_ABORTS], (unsigned long long)aborts);
-    if (c.reviews) atomicAdd(&bc[C_REVIEWS], (unsigned long long)c.reviews);
     // bins viewed by the attempt that was applied (or failed), and by all
     // attempts including those abandoned after claim conflicts
     uint32_t v_final = c.viewed - c.viewed0;
@@ -424,35 +418,29 @@ __global__ void __launch_bounds__(256, insert_blocks_per_sm<B, POL>()) k_insert(
     viewed_all += c.viewed;
     if (status) status[i] = (uint8_t)st;
     if (viewed_out) viewed_out[i] = v_final;
-    uint64_t bucket = ((size_base + i) * HIST_BUCKETS) / t.total_slots;
-    if (bucket >= HIST_BUCKETS) bucket = HIST_BUCKETS - 1;
-    atomicAdd(&h_views[bucket], v_final);
-    atomicAdd(&h_cnt[bucket], 1u);
+    ok += st == ST_OK;
+    bt.key_done(c, st, aborts, v_final, load_bucket(load_base + i, t.total_slots));
+  };
+  for (;;) {
+    uint64_t i = hi;
+    if constexpr (LOOK) {
+      if (look) {
+        const bool more = ls.template take<B, POL>(t, keys, vals, status, viewed_out, hi, load_base, 0xFFFFFFFFu, bt, i);
+        if (i < hi) insert(i);
+        __syncwarp();
+        if (!more) break;
+        continue;
+      }
+    }
+    i = atomicAdd(&s_next, 1ull);
+    if (i >= hi) break;
+    insert(i);
   }
-  flush_counter(&bc[C_INS_OK], ok);
-  flush_counter(&bc[C_VIEWED], viewed);
-  flush_counter(&bc[C_VIEWED_ALL], viewed_all);
+  flush_counter(&bt.bc[C_INS_OK], ok);
+  flush_counter(&bt.bc[C_VIEWED], viewed);
+  flush_counter(&bt.bc[C_VIEWED_ALL], viewed_all);
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int k = 0; k < C_N; k++) {
-      if (!bc[k]) continue;
-      if (k == C_CHAIN_MAX) atomicMax(t.counters + k, bc[k]);
-      else atomicAdd(t.counters + k, bc[k]);
-    }
-    // size and live ghosts follow from the counts above
-    if (bc[C_INS_OK]) atomicAdd(t.counters + C_SIZE, bc[C_INS_OK]);
-    long long dg = (long long)bc[C_GHOSTS_MADE] - (long long)bc[C_DUP_EVICT];
-    if (dg) atomicAdd(t.counters + C_LIVE_GHOSTS, (unsigned long long)dg);
-  }
-  unsigned long long* hist = t.counters + C_N;
-  for (int i = threadIdx.x; i < HIST_BUCKETS; i += blockDim.x) {
-    if (h_cnt[i]) {
-      atomicAdd(hist + i, (unsigned long long)h_views[i]);
-      atomicAdd(hist + HIST_BUCKETS + i, (unsigned long long)h_cnt[i]);
-    }
-  }
-  for (int i = threadIdx.x; i < CHAIN_BUCKETS; i += blockDim.x)
-    if (h_chain[i]) atomicAdd(t.counters + CHAIN_HIST + i, (unsigned long long)h_chain[i]);
+  bt.flush(t);
   if (threadIdx.x == 0) {
     if (s_slab[0] >= 0) {
       __threadfence();

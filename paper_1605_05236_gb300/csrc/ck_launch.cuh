@@ -6,6 +6,7 @@
 
 #include "ck.h"
 #include "ck_kernels.cuh"
+#include "ck_walk.cuh"
 #include "ck_warp.cuh"
 
 namespace ck {
@@ -40,19 +41,26 @@ cudaError_t launch_insert(const InsertLaunch& l, const uint32_t* keys, const uin
     return cudaGetLastError();
   }
   const uint32_t block = l.block;
+  // two-choice walks without ghosts run a step per lane (ck_walk.cuh), except
+  // upserts, which first look for the key under claims
+  constexpr bool WALKS = B > 1 && !GHOST && (POL == P_QUEUE || POL == P_RANDOM);
+  const bool walk = WALKS && !upsert;
   // persistent launch: at most the blocks that fit on the GPU at once
-  static int cached_block = 0, cached_per_sm = 0;
-  if (cached_block != (int)block) {
+  static int cached_block[2] = {0, 0}, cached_per_sm[2] = {0, 0};
+  if (cached_block[walk] != (int)block) {
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_insert<B, POL, GHOST, false>, block, 0) !=
-            cudaSuccess ||
-        per_sm < 1)
-      per_sm = 1;
-    cached_per_sm = per_sm;
-    cached_block = (int)block;
+    cudaError_t e;
+    if constexpr (WALKS)
+      e = walk ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_insert_walk<B, POL>, block, 0)
+               : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_insert<B, POL, GHOST, false>, block, 0);
+    else
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_insert<B, POL, GHOST, false>, block, 0);
+    if (e != cudaSuccess || per_sm < 1) per_sm = 1;
+    cached_per_sm[walk] = per_sm;
+    cached_block[walk] = (int)block;
   }
   uint64_t grid = (n + block - 1) / block;
-  uint64_t resident = (uint64_t)cached_per_sm * l.sm_count;
+  uint64_t resident = (uint64_t)cached_per_sm[walk] * l.sm_count;
   // Walks whose launches overlap leave part of the GPU to the next launch:
   // its blocks start while this launch's longest walks finish.  Measured
   // (whole fills, one GB300): two-choice queue-kicking 10.18 ms against
@@ -86,6 +94,8 @@ cudaError_t launch_insert(const InsertLaunch& l, const uint32_t* keys, const uin
   attr[0].val.programmaticStreamSerializationAllowed = l.overlap ? 1 : 0;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  if constexpr (WALKS)
+    if (walk) return cudaLaunchKernelEx(&cfg, k_insert_walk<B, POL>, dt, keys, vals, n, st, viewed, load_base);
   return cudaLaunchKernelEx(&cfg, k_insert<B, POL, GHOST, false>, dt, keys, vals, n, st, viewed, load_base, upsert);
 }
 

@@ -1,0 +1,222 @@
+// ck_look.cuh -- the first look at a batch's keys (two-choice tables without
+// ghosts) and a block's counts, shared by the concurrent insert kernels.
+//
+// Most keys of a fill find a free slot in one of their bins.  A warp takes
+// its keys 32 at a time, so that the loads of keys and the stores of statuses
+// are coalesced, reads the slots of their bins -- no metadata word -- and
+// places what it can by one compare-and-swap a key (place_direct).  The keys
+// that found no room, or lost their slot to another thread, are kept by index
+// in shared memory for the whole insertion, which a warp then enters with
+// full lanes instead of the few of each 32 that need it.  Bound by the
+// memory system: two random 128-byte lines a key (a random 32-byte miss
+// moves its whole line) and the line written back.  Measured on one GB300,
+// 2^20 keys a launch into an empty 2^24 x 4 table: 74 us against 90 with one
+// key a thread through the whole insertion; two keys a lane in flight: 79.
+#pragma once
+#include "ck_search.cuh"
+
+namespace ck {
+
+__device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31u; }
+
+// The bins-viewed histogram's bucket of a load of `at` keys.
+__device__ __forceinline__ uint32_t load_bucket(uint64_t at, uint64_t total) {
+  const uint64_t x = at * HIST_BUCKETS / total;
+  return x < HIST_BUCKETS ? (uint32_t)x : HIST_BUCKETS - 1;
+}
+
+// A block's counts, in shared memory.
+struct BlockTally {
+  unsigned int views[HIST_BUCKETS], cnt[HIST_BUCKETS];  // bins viewed and keys, by load
+  unsigned int chain[CHAIN_BUCKETS];
+  unsigned long long bc[C_N];
+
+  __device__ __forceinline__ void clear() {
+    for (int i = threadIdx.x; i < HIST_BUCKETS; i += blockDim.x) views[i] = cnt[i] = 0;
+    for (int i = threadIdx.x; i < CHAIN_BUCKETS; i += blockDim.x) chain[i] = 0;
+    for (int i = threadIdx.x; i < C_N; i += blockDim.x) bc[i] = 0;
+  }
+  // a key's insertion ended with st, v bins viewed by its last attempt; what
+  // every key adds to (insertions, bins viewed) the caller tallies
+  __device__ __forceinline__ void key_done(const Ctx& c, int st, uint32_t aborts, uint32_t v, uint32_t bucket) {
+    if (st == ST_OK) {
+      if (c.kicks) {
+        atomicAdd(&bc[C_KICKS], (unsigned long long)c.kicks);
+        atomicMax(&bc[C_CHAIN_MAX], (unsigned long long)c.kicks);
+      }
+      atomicAdd(&chain[chain_bucket(c.kicks)], 1u);
+      if (c.ghosts_made) atomicAdd(&bc[C_GHOSTS_MADE], (unsigned long long)c.ghosts_made);
+      if (c.dup_evict) atomicAdd(&bc[C_DUP_EVICT], (unsigned long long)c.dup_evict);
+    } else {
+      atomicAdd(&bc[st == ST_FAILED ? C_INS_FAILED : C_INS_ABORTED], 1ull);
+    }
+    if (aborts) atomicAdd(&bc[C_ABORTS], (unsigned long long)aborts);
+    if (c.reviews) atomicAdd(&bc[C_REVIEWS], (unsigned long long)c.reviews);
+    atomicAdd(&views[bucket], v);
+    atomicAdd(&cnt[bucket], 1u);
+  }
+  // after a barrier, by the whole block: into the table's counters
+  __device__ __forceinline__ void flush(const DevTable& t) {
+    if (threadIdx.x == 0) {
+      for (int k = 0; k < C_N; k++) {
+        if (!bc[k]) continue;
+        if (k == C_CHAIN_MAX) atomicMax(t.counters + k, bc[k]);
+        else atomicAdd(t.counters + k, bc[k]);
+      }
+      // size and live ghosts follow from the counts above
+      if (bc[C_INS_OK]) atomicAdd(t.counters + C_SIZE, bc[C_INS_OK]);
+      long long dg = (long long)bc[C_GHOSTS_MADE] - (long long)bc[C_DUP_EVICT];
+      if (dg) atomicAdd(t.counters + C_LIVE_GHOSTS, (unsigned long long)dg);
+    }
+    unsigned long long* hist = t.counters + C_N;
+    for (int i = threadIdx.x; i < HIST_BUCKETS; i += blockDim.x) {
+      if (cnt[i]) {
+        atomicAdd(hist + i, (unsigned long long)views[i]);
+        atomicAdd(hist + HIST_BUCKETS + i, (unsigned long long)cnt[i]);
+      }
+    }
+    for (int i = threadIdx.x; i < CHAIN_BUCKETS; i += blockDim.x)
+      if (chain[i]) atomicAdd(t.counters + CHAIN_HIST + i, (unsigned long long)chain[i]);
+  }
+};
+
+// A block's keys: the next index of its range, and per warp the keys looked
+// at that found no room.
+struct LookState {
+  unsigned long long next;
+  uint64_t left[8][64];
+  uint32_t n_left[8];
+  uint32_t bucket;       // the histogram bucket of the block's first keys ...
+  uint64_t bucket_end;   // ... up to this index
+
+  __device__ __forceinline__ void begin(const DevTable& t, uint64_t lo, uint64_t load_base) {
+    if (threadIdx.x < 8) n_left[threadIdx.x] = 0;
+    if (threadIdx.x == 0) {
+      next = lo;
+      bucket = load_bucket(load_base + lo, t.total_slots);
+      const uint64_t end = ((uint64_t)(bucket + 1) * t.total_slots + HIST_BUCKETS - 1) / HIST_BUCKETS;
+      bucket_end = bucket == HIST_BUCKETS - 1 ? ~0ull : end - load_base;
+    }
+  }
+
+  // One look at 32 new keys from `base` (those below hi), by a whole warp.
+  // Queue-kicking reads both bins and takes the less full one (b0 on ties);
+  // the other policies take b0's first free slot, else b1's, and fetch b1
+  // only where b0 has none.  The searches count both bins as viewed either
+  // way, as their definition does.
+  template <int B, int POL>
+  __device__ __forceinline__ uint32_t look(const DevTable& t, const uint32_t* __restrict__ keys,
+                                           const uint32_t* __restrict__ vals, uint8_t* status, uint32_t* viewed_out,
+                                           uint64_t base, uint64_t hi, uint64_t load_base, uint32_t nl,
+                                           BlockTally& bt) {
+    const uint64_t j = base + lane_id();
+    const bool on = j < hi;
+    const uint32_t key = on ? __ldcs(keys + j) : RESERVED_KEY;
+    const uint32_t val = on ? __ldcs(vals + j) : 0u;
+    uint64_t* p = nullptr;
+    uint32_t views = 2;
+    if (key != RESERVED_KEY) {
+      uint32_t b0, b1;
+      bins2(t, key, b0, b1);
+      View<B> v;
+      load_slots<B>(t, b0, v);
+      uint32_t g0, g1 = 0;
+      if (POL == P_QUEUE) {
+        View<B> v1;
+        load_slots<B>(t, b1, v1);
+        g0 = empty_mask<B>(v);
+        g1 = empty_mask<B>(v1);
+        if (__popc(g0) >= __popc(g1)) g1 = 0;
+        else g0 = 0;
+      } else {
+        g0 = empty_mask<B>(v);
+        if (!g0) {
+          load_slots<B>(t, b1, v);
+          g1 = empty_mask<B>(v);
+        } else if (POL == P_RANDOM) {
+          views = 1;
+        }
+      }
+      if (g0 | g1) p = t.slots + (uint64_t)(g0 ? b0 : b1) * B + lowest(g0 ? g0 : g1);
+    }
+    const bool placed = p && cas_slot(p, EMPTY, ((uint64_t)key << 32) | val);
+    const bool invalid = on && key == RESERVED_KEY;
+    if (placed || invalid) {
+      if (status) status[j] = (uint8_t)(invalid ? ST_INVALID : ST_OK);
+      if (viewed_out) viewed_out[j] = invalid ? 0u : views;
+    }
+    const unsigned pm = __ballot_sync(0xFFFFFFFFu, placed), lm = __ballot_sync(0xFFFFFFFFu, p && !placed);
+    if (pm) {
+      const uint32_t n = __popc(pm);
+      const uint32_t sum = POL == P_RANDOM ? __reduce_add_sync(0xFFFFFFFFu, placed ? views : 0u) : 2 * n;
+      const bool one = base + 32 <= bucket_end;  // the block's first bucket: one add for the warp
+      if (lane_id() == 0) {
+        atomicAdd(&bt.bc[C_INS_OK], (unsigned long long)n);
+        atomicAdd(&bt.bc[C_VIEWED], (unsigned long long)sum);
+        atomicAdd(&bt.bc[C_VIEWED_ALL], (unsigned long long)sum);
+        atomicAdd(&bt.chain[0], n);
+        if (one) {
+          atomicAdd(&bt.views[bucket], sum);
+          atomicAdd(&bt.cnt[bucket], n);
+        }
+      }
+      if (!one && placed) {
+        const uint32_t b = load_bucket(load_base + j, t.total_slots);
+        atomicAdd(&bt.views[b], views);
+        atomicAdd(&bt.cnt[b], 1u);
+      }
+    }
+    if (lm) {  // attempts given up on a conflict
+      const uint32_t sum = __reduce_add_sync(0xFFFFFFFFu, p && !placed ? views : 0u);
+      if (lane_id() == 0) {
+        atomicAdd(&bt.bc[C_ABORTS], (unsigned long long)__popc(lm));
+        atomicAdd(&bt.bc[C_VIEWED_ALL], (unsigned long long)sum);
+      }
+    }
+    const bool rest = on && !placed && !invalid;
+    const unsigned rm = __ballot_sync(0xFFFFFFFFu, rest);
+    if (rest) left[threadIdx.x >> 5][nl + __popc(rm & ((1u << lane_id()) - 1))] = j;
+    return nl + __popc(rm);
+  }
+
+  // Keys for the lanes of `idle` (called by the whole warp): `got` is set to
+  // the key's index, where one is left that needs the whole insertion.
+  // False: the block's range is done, and so is the warp's list.
+  template <int B, int POL>
+  __device__ __forceinline__ bool take(const DevTable& t, const uint32_t* __restrict__ keys,
+                                       const uint32_t* __restrict__ vals, uint8_t* status, uint32_t* viewed_out,
+                                       uint64_t hi, uint64_t load_base, unsigned idle, BlockTally& bt,
+                                       uint64_t& got) {
+    const uint32_t wp = threadIdx.x >> 5, lane = lane_id(), want = __popc(idle);
+    uint32_t nl = n_left[wp];
+    bool more = true;
+    while (nl < want) {
+      unsigned long long base = 0;
+      if (lane == 0) base = atomicAdd(&next, 32ull);
+      base = __shfl_sync(0xFFFFFFFFu, base, 0);
+      if (base >= hi) {
+        more = false;
+        break;
+      }
+      nl = look<B, POL>(t, keys, vals, status, viewed_out, base, hi, load_base, nl, bt);
+    }
+    __syncwarp();
+    const uint32_t give = nl < want ? nl : want, r = __popc(idle & ((1u << lane) - 1));
+    if (((idle >> lane) & 1u) && r < give) got = left[wp][nl - give + r];
+    __syncwarp();
+    if (lane == 0) n_left[wp] = nl - give;
+    __syncwarp();
+    return more || nl > give;
+  }
+};
+
+// LookState, or nothing for kernels that take no look.
+struct NoLook {};
+template <bool LOOK>
+struct LookMaybeT { using type = LookState; };
+template <>
+struct LookMaybeT<false> { using type = NoLook; };
+template <bool LOOK>
+using LookMaybe = typename LookMaybeT<LOOK>::type;
+
+}  // namespace ck

@@ -66,10 +66,10 @@ __global__ void __launch_bounds__(256) k_lookup_validated(DevTable t, const uint
         uint32_t seen[4];
         bool hit = false;
         uint32_t v = 0;
+        read_words(t, b, nb, seen);
         for (uint32_t j = 0; j < nb; j++) {
           View<B> vw;
-          load_view<B>(t, b[j], vw);
-          seen[j] = vw.m;
+          load_slots<B>(t, b[j], vw);
 #pragma unroll
           for (int q = 0; q < B; q++)
             if (!hit && vw.s[q] != EMPTY && key_of(vw.s[q]) == key) { hit = true; v = (uint32_t)vw.s[q]; }

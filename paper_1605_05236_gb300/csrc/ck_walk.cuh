@@ -1,0 +1,322 @@
+// ck_walk.cuh -- concurrent insertion by kick-out walks (queue-kicking and
+// random kicking, two-choice tables without ghosts; Kuszmaul,
+// arXiv:1605.05236, Sec. 1, Sec. 6, Sec. 8) with every lane of a warp at its
+// own point of its own walk.
+//
+// What bounds the insertions of a nearly full table is chains of dependent
+// round trips, and walks are uneven: near load 0.95 a key kicks five records
+// on average and the longest of 32 keys about forty, so a warp that waits
+// for its longest walk before it takes new keys keeps a fifth of its lanes
+// busy.  Here a walk is a state (Walk) that advances one kick a step; a lane
+// whose walk ends applies it and takes the next key while the others go on.
+// The parts that end and begin walks cost several round trips and all lanes
+// pass through them, so they run when most lanes wait for them (WAITERS), not
+// for each.  Fill of 2^24 x 4 to 0.95 in 2^20-key batches: 6.33 ms against
+// 9.27 with one insertion a lane from view to commit (k_insert) and 8.34 with
+// the first look alone; its last launch (load 0.94) 0.88 ms against 1.45.
+//
+// The claims, the re-validation of moves and the order of writes are
+// ck_insert.cuh's, with one difference: the free slot a chain ends in is not
+// claimed.  Nothing moves out of it, so no reader's proof of a miss and no
+// other plan rests on its claim, and the write that takes it is a
+// compare-and-swap from empty anyway; the claim and its release were two
+// more atomics on a metadata line the chain otherwise only reads.  The
+// compare-and-swap is the chain's first write, made once the last claimed
+// slot was read again and found as planned; if it fails, the walk views the
+// bin again with nothing written.
+#pragma once
+#include "ck_look.cuh"
+
+namespace ck {
+
+constexpr int WALK = -1;  // the walk goes on
+
+// A walk at a bin it has viewed, with the record c.held in hand.
+template <int B>
+struct Walk {
+  uint32_t x;            // the bin
+  int s;                 // random kicking: the slot to kick (-1: not drawn yet)
+  uint32_t tries;        // views of x beyond the first
+  View<B> v;             // x as viewed
+  const uint64_t* pend;  // the slot claimed by the last kick, not read again yet (reread), or null
+};
+
+// The two bins of a new key: placed if there is room (ST_OK), else the walk's
+// first bin is chosen.
+template <int B, int POL>
+__device__ __forceinline__ int walk_begin(const DevTable& t, Ctx& c, Walk<B>& w) {
+  constexpr uint32_t FULL = (1u << B) - 1;
+  uint32_t b0, b1;
+  bins2(t, c.key, b0, b1);
+  View<B> v0, v1;
+  load_view2_fast<B>(t, b0, b1, v0, v1);
+  c.held = c.krec;
+  w.pend = nullptr;
+  w.tries = 0;
+  w.s = -1;
+  const uint32_t g0 = empty_mask<B>(v0), g1 = empty_mask<B>(v1);
+  c.viewed += (POL == P_RANDOM && g0) ? 1 : 2;
+  if (g0 | g1) {
+    const bool first = POL == P_QUEUE ? __popc(g0) >= __popc(g1) : g0 != 0;
+    return place_direct<B>(t, c, first ? b0 : b1, lowest(first ? g0 : g1)) ? (int)ST_OK : (int)ST_CONFLICT;
+  }
+  bool first;
+  if (POL == P_QUEUE) {
+    first = hit_of_full<B>(v0.m) <= hit_of_full<B>(v1.m);
+  } else {  // first victim: uniform over the usable slots of b0 then b1
+    const uint32_t e0 = FULL & ~claimed_mask<B>(v0), e1 = FULL & ~claimed_mask<B>(v1);
+    const uint32_t n0 = __popc(e0), ne = n0 + __popc(e1);
+    if (ne == 0) return ST_CONFLICT;
+    const uint32_t idx = (uint32_t)(draw(t, c.key, c.draws++, c.attempt) % ne);
+    first = idx < n0;
+    w.s = first ? nth_bit(e0, idx) : nth_bit(e1, idx - n0);
+  }
+  w.x = first ? b0 : b1;
+  w.v.m = first ? v0.m : v1.m;
+#pragma unroll
+  for (int q = 0; q < B; q++) w.v.s[q] = first ? v0.s[q] : v1.s[q];
+  return WALK;
+}
+
+// One step at w.x: the free slot that ends the chain (ST_OK, and it is
+// written), or one kick -- the claim of the victim, the view of the bin it
+// moves to and the re-read of the slot the kick before claimed, in one round
+// trip -- or another view of the bin after a lost race (WALK).
+template <int B, int POL>
+__device__ __forceinline__ int walk_step(const DevTable& t, Ctx& c, Walk<B>& w) {
+  constexpr uint32_t FULL = (1u << B) - 1;
+  const uint64_t chk = w.pend ? ld_slot(w.pend) : c.held;
+  const uint32_t fm = empty_mask<B>(w.v);
+  bool again = true;
+  if (fm) {
+    if (chk != c.held) return ST_CONFLICT;
+    w.pend = nullptr;  // read again and as planned
+    uint64_t* p = t.slots + (uint64_t)w.x * B + lowest(fm);
+    if (cas_slot(p, EMPTY, c.held)) return ST_OK;
+  } else {
+    const uint32_t claimed = claimed_mask<B>(w.v);
+    int s = w.s, jprev = -1;
+    bool rev = false;
+    if (POL == P_QUEUE) {
+      // the record at slot h mod B, skipping slots another insertion holds;
+      // a slot this chain already wrote is taken again, with the record the
+      // chain put there
+      const uint32_t own = claimed ? own_slots(c, w.x) : 0u;
+      const uint32_t foreign = claimed & ~own;
+      if (foreign) c.foreign = 1;
+      s = first_from<B>(FULL & ~foreign, hit_of_full<B>(w.v.m) % B);
+      if (s < 0) return dead_end(c);
+      if (c.kicks == t.cap) return out_of_cap(c);
+      rev = (own >> s) & 1u;
+      if (rev) jprev = last_entry_for(c, w.x, (uint32_t)s);
+    } else {
+      if (c.kicks == t.cap) return ST_FAILED;
+      if (s < 0) {  // uniform over the slots no chain holds
+        const uint32_t e = FULL & ~claimed;
+        if (!e) return claims_all_ours<B>(c, w.x, claimed) ? (int)ST_FAILED : (int)ST_CONFLICT;
+        s = nth_bit(e, (uint32_t)(draw(t, c.key, c.draws++, c.attempt) % __popc(e)));
+        w.s = s;
+      } else if ((claimed >> s) & 1u) {  // taken while the claim was tried
+        return ST_CONFLICT;
+      }
+    }
+    if (int r0 = plan_room(t, c)) return r0;
+    const uint64_t victim = rev ? content_at(c, jprev) : slot_of<B>(w.v, s);
+    const uint32_t xn = other_bin2(t, victim, w.x);
+    View<B> vn;
+    load_view_fast<B>(t, xn, vn);
+    // (an entry of this kernel's plans holds the record its slot receives)
+    if (rev ? claim_again(t, c, w.x, w.v.m, s, jprev, c.held)
+            : claim(t, c, w.x, w.v.m, s, K_MOVE, POL == P_QUEUE, c.held)) {
+      if (chk != c.held) return ST_CONFLICT;
+      c.kicks++;
+      // a slot the chain holds already carries the plan's record: no re-read
+      w.pend = rev ? nullptr : t.slots + (uint64_t)w.x * B + s;
+      c.held = victim;
+      w.x = xn;
+      w.v = vn;
+      w.s = -1;
+      w.tries = 0;
+      c.viewed++;
+      again = false;
+    }
+  }
+  if (again) {  // the bin changed since its view
+    if (++w.tries == 4) return ST_CONFLICT;
+    load_view_fast<B>(t, w.x, w.v);
+    c.viewed++;
+    c.reviews++;
+  }
+  return WALK;
+}
+
+// Entries first .. first + 3 of the plan (those below n; the others repeat
+// the last), loaded together.
+__device__ __forceinline__ void load_entries(const Ctx& c, int first, int n, ulonglong2 (&e)[4]) {
+#pragma unroll
+  for (int u = 0; u < 4; u++) {
+    const int i = min(first + u, n - 1);
+    if (i < REG_ENTRIES) e[u] = make_ulonglong2(c.r0d, c.r0c);
+    else e[u] = *reinterpret_cast<const ulonglong2*>(c.pe + 2 * i);
+  }
+}
+
+// The chain's last record is in its free slot: the others' writes, last slot
+// first, then the releases (as commit, ck_insert.cuh).  An entry's content is
+// the record its slot receives.
+template <int B>
+__device__ __forceinline__ void walk_commit(const DevTable& t, Ctx& c) {
+  const int n = c.pn;
+  if (n == 0) return;
+  ulonglong2 e[4];
+  for (int first = (n - 1) & ~3; first >= 0; first -= 4) {
+    load_entries(c, first, n, e);
+#pragma unroll
+    for (int u = 3; u >= 0; u--) {
+      if (first + u >= n || e_sup(e[u].x)) continue;  // a later revisit of the slot writes it
+      if (t.ordered_writes) fence_release();          // the copy lands before its source is overwritten
+      st_slot(slot_at<B>(t, e[u].x), e[u].y);
+    }
+  }
+  fence_release();
+  for (int first = 0; first < n; first += 4) {
+    load_entries(c, first, n, e);
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      if (first + u >= n) continue;
+      red_relaxed(t.meta + e_bin(e[u].x), VER_ONE - (e_rev(e[u].x) ? 0u : 1u << e_slot(e[u].x)));
+    }
+  }
+}
+
+// The lanes whose walk ended, or that wait for a key, are served once they
+// are WAITERS times the lanes still walking.  Measured, fill of 2^24 x 4 to
+// 0.95 with queue-kicking (each against the next, same GPU): served as soon
+// as one lane waits 7.80 ms, from 1/8, 1/4 and 1/2 of the walking lanes on
+// 7.59, 7.37 and 7.16 (commits loading one entry at a time: 6.86 for 1/2 with
+// four at a time), from as many on 6.44, from twice as many on 6.33.
+//
+// 80 registers (3 blocks of 256 threads on an SM): 6.43 ms against 6.61 at
+// 64, which spill more.  One block waits for the launch before, which is
+// enough to keep this one from completing first: blocks that are done make
+// room for the next launch's (6.43 against 6.46 with every block waiting).
+constexpr int WAITERS = 2;
+
+template <int B, int POL>
+__global__ void __launch_bounds__(256, 3) k_insert_walk(DevTable t, const uint32_t* __restrict__ keys,
+                                                        const uint32_t* __restrict__ vals, uint64_t n,
+                                                        uint8_t* __restrict__ status,
+                                                        uint32_t* __restrict__ viewed_out, uint64_t load_base) {
+  asm volatile("griddepcontrol.launch_dependents;");
+  __shared__ BlockTally bt;
+  __shared__ LookState ls;
+  const uint64_t per = (n + gridDim.x - 1) / gridDim.x;
+  const uint64_t lo = min(n, (uint64_t)blockIdx.x * per), hi = min(n, lo + per);
+  bt.clear();
+  ls.begin(t, lo, load_base);
+  __syncthreads();
+
+  PlanStore<MAX_CHAIN> store;
+  // a lane has no key; has one whose next attempt begins; walks; has an
+  // attempt that ended with st; waits before its next attempt
+  enum Mode { IDLE, READY, WALKING, ENDED, WAITING };
+  int mode = IDLE, st = ST_OK;
+  Ctx c;
+  c.ghosts_made = c.dup_evict = 0;
+  Walk<B> w;
+  uint64_t i = 0;
+  uint32_t fails = 0, aborts = 0, wake = 0;
+  uint32_t ok = 0, viewed = 0, viewed_all = 0;
+  bool more = true;  // keys are left in the block's range (or in the warp's list)
+  for (;;) {
+    const unsigned walking = __ballot_sync(0xFFFFFFFFu, mode == WALKING);
+    if (mode == WAITING && (int)((uint32_t)clock() - wake) >= 0) mode = READY;
+    const unsigned waiting = __ballot_sync(0xFFFFFFFFu, mode == WAITING);
+    const unsigned need = __ballot_sync(0xFFFFFFFFu, mode == ENDED || mode == READY || (mode == IDLE && more));
+    if (!(walking | waiting | need)) break;
+    if (need && (__popc(need) >= WAITERS * __popc(walking))) {
+      if (mode == ENDED) {  // as insert_one ends an attempt
+        if (st == ST_OK) {
+          walk_commit<B>(t, c);
+        } else {
+          release_all(t, c);
+          const bool ran_out = st == ST_FAILED || c.capped;
+          bool over = false;
+          if (ran_out) {
+            over = ++fails > (st == ST_FAILED ? 6u : 32u);
+            if (over) st = ST_FAILED;
+          } else {
+            aborts++;
+          }
+          if (!over && ++c.attempt >= t.max_retries) {
+            st = ST_ABORTED;
+            over = true;
+          }
+          if (!over) {
+            const uint32_t a = ran_out ? 6 + 2 * fails : c.attempt;
+            const uint32_t ns = 64u << (a < 9 ? a : 9);
+            wake = (uint32_t)clock() + 2 * (ns + (fmix32(c.key ^ a) & (ns - 1)));
+            mode = WAITING;
+          }
+        }
+        if (mode == ENDED) {
+          if (c.long_id >= 0) release_long(t, c.long_id);
+          if (status) status[i] = (uint8_t)st;
+          if (viewed_out) viewed_out[i] = c.viewed - c.viewed0;
+          bt.key_done(c, st, aborts, c.viewed - c.viewed0, load_bucket(load_base + i, t.total_slots));
+          ok += st == ST_OK;
+          viewed += c.viewed - c.viewed0;
+          viewed_all += c.viewed;
+          mode = IDLE;
+        }
+      }
+      // keys for the idle lanes
+      const unsigned idle = __ballot_sync(0xFFFFFFFFu, mode == IDLE);
+      if (idle && more) {
+        uint64_t got = hi;
+        more = ls.template take<B, POL>(t, keys, vals, status, viewed_out, hi, load_base, idle, bt, got);
+        if (got < hi) {
+          i = got;
+          c.key = __ldcs(keys + i);
+          c.krec = ((uint64_t)c.key << 32) | __ldcs(vals + i);
+          c.attempt = 0;
+          c.viewed = 0;
+          c.reviews = 0;
+          c.long_id = -1;
+          fails = 0;
+          aborts = 0;
+          mode = READY;
+        }
+      }
+      if (mode == READY) {
+        c.kicks = 0;
+        c.draws = 0;
+        c.viewed0 = c.viewed;
+        c.foreign = 0;
+        c.capped = 0;
+        if (c.long_id < 0) {
+          c.pe = store.e;
+          c.pcap = MAX_CHAIN;
+        }
+        c.pn = 0;
+        st = walk_begin<B, POL>(t, c, w);
+        mode = st == WALK ? WALKING : ENDED;
+      }
+    }
+    if (mode == WALKING) {
+      st = walk_step<B, POL>(t, c, w);
+      if (st != WALK) mode = ENDED;
+    } else if (!walking && !need) {
+      __nanosleep(100);
+    }
+    __syncwarp();
+  }
+  if (ok) atomicAdd(&bt.bc[C_INS_OK], (unsigned long long)ok);
+  if (viewed) atomicAdd(&bt.bc[C_VIEWED], (unsigned long long)viewed);
+  if (viewed_all) atomicAdd(&bt.bc[C_VIEWED_ALL], (unsigned long long)viewed_all);
+  __syncthreads();
+  bt.flush(t);
+  if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");  // see WAITERS
+}
+
+}  // namespace ck
