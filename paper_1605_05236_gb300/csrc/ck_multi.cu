@@ -31,7 +31,7 @@ int ck_internal_launch_insert(const DevTable& dt, uint32_t block, int sm_count, 
 namespace {
 
 constexpr size_t ALIGN = 256;
-size_t align_up(size_t x) { return (x + ALIGN - 1) / ALIGN * ALIGN; }
+__host__ __device__ constexpr size_t align_up(size_t x) { return (x + ALIGN - 1) / ALIGN * ALIGN; }
 
 struct Tile {
   uint32_t table;
@@ -40,6 +40,9 @@ struct Tile {
 };
 
 constexpr uint32_t MULTI_LONG_PLANS = 1024;
+// Tables filled together.  Measured on 4096 tables (9.3 GB, 1.07e9 keys): 8
+// and 16 MiB 90.0 ms, 32 MiB 90.4, 64 MiB 90.8, all tables at once 107.1.
+constexpr size_t WINDOW_BYTES = 16u << 20;
 
 }  // namespace
 
@@ -271,30 +274,35 @@ int occupancy_blocks(uint32_t policy, uint32_t block) {
   return per_sm;
 }
 
-// Build the tile list for the current tile size and upload it.  Tiles are
-// interleaved round-robin over the tables (tile r of every table, then tile
-// r+1, ...): the GPU works on many tables at once and each table keeps only
-// a few tiles in flight, so its load grows in order and its insertions
-// rarely meet each other's claims.
-int build_tiles(ck_multi* m, cudaStream_t s) {
+// Build the tile list for the current tile size and upload it.  The tables
+// are taken in groups of about WINDOW_BYTES, in order, and the tiles of a
+// group round-robin over its tables (tile r of each, then tile r + 1): the
+// tables being filled stay in L2 from their first tile to their last, and
+// each keeps only a part of its tiles in flight, so its load grows in order.
+std::vector<Tile> make_tiles(const ck_multi_desc* desc, uint32_t n_tables, uint32_t tile) {
   std::vector<Tile> tiles;
-  tiles.reserve(count_tiles(m->desc.data(), m->n_tables, m->tile));
-  for (uint64_t r = 0;; r++) {
-    bool any = false;
-    for (uint32_t i = 0; i < m->n_tables; i++) {
-      const ck_multi_desc& d = m->desc[i];
-      uint64_t lo = r * m->tile;
-      if (lo >= d.n_keys) continue;
-      any = true;
-      Tile t;
-      t.table = i;
-      t.pad = 0;
-      t.lo = d.key_offset + lo;
-      t.hi = d.key_offset + (lo + m->tile < d.n_keys ? lo + m->tile : d.n_keys);
-      tiles.push_back(t);
+  tiles.reserve(count_tiles(desc, n_tables, tile));
+  for (uint32_t first = 0, last; first < n_tables; first = last) {
+    size_t bytes = 0;
+    for (last = first; last < n_tables && (last == first || bytes + table_bytes(desc[last]) <= WINDOW_BYTES); last++)
+      bytes += table_bytes(desc[last]);
+    bool any = true;
+    for (uint64_t r = 0; any; r++) {
+      any = false;
+      for (uint32_t i = first; i < last; i++) {
+        const ck_multi_desc& d = desc[i];
+        const uint64_t lo = r * tile;
+        if (lo >= d.n_keys) continue;
+        any = true;
+        tiles.push_back({i, 0, d.key_offset + lo, d.key_offset + (lo + tile < d.n_keys ? lo + tile : d.n_keys)});
+      }
     }
-    if (!any) break;
   }
+  return tiles;
+}
+
+int build_tiles(ck_multi* m, cudaStream_t s) {
+  const std::vector<Tile> tiles = make_tiles(m->desc.data(), m->n_tables, m->tile);
   m->n_tiles = (uint32_t)tiles.size();
   if (cudaMemcpyAsync(m->d_tiles, tiles.data(), tiles.size() * sizeof(Tile), cudaMemcpyHostToDevice, s) !=
       cudaSuccess)
@@ -302,16 +310,30 @@ int build_tiles(ck_multi* m, cudaStream_t s) {
   return cudaStreamSynchronize(s) == cudaSuccess ? CK_OK : CK_ECUDA;
 }
 
+// Empty every table and zero its counters, in one launch: block (i, y) takes
+// every gridDim.y-th piece of table i.  A write pass over the tables (bound by
+// DRAM).  Three memsets a table took 19 ms more on 4096 tables, replayed from
+// a graph (126.2 ms for clear and fill against 107.1).
+constexpr unsigned CLEAR_PARTS = 16;
+
+__device__ __forceinline__ void fill16(void* p, uint64_t bytes, uint32_t v) {  // p and bytes: multiples of 16
+  uint4* q = static_cast<uint4*>(p);
+  const uint4 x = make_uint4(v, v, v, v);
+  for (uint64_t i = (uint64_t)blockIdx.y * blockDim.x + threadIdx.x; i < bytes / 16; i += CLEAR_PARTS * blockDim.x) q[i] = x;
+}
+
+__global__ void __launch_bounds__(256) k_multi_clear(const DevTable* __restrict__ tables) {
+  const DevTable& t = tables[blockIdx.x];
+  // each part is followed by padding up to a multiple of 256 bytes
+  fill16(t.slots, align_up(t.total_slots * sizeof(uint64_t)), 0xFFFFFFFFu);
+  fill16(t.meta, align_up(t.n_bins * sizeof(uint32_t)), 0u);
+  fill16(t.counters, align_up(COUNTER_WORDS * sizeof(uint64_t)), 0u);
+}
+
 int clear_tables(ck_multi* m, cudaStream_t s) {
-  for (uint32_t i = 0; i < m->n_tables; i++) {
-    const DevTable& t = m->host_tables[i];
-    if (cudaMemsetAsync(t.slots, 0xFF, t.total_slots * sizeof(uint64_t), s) != cudaSuccess) return CK_ECUDA;
-    if (cudaMemsetAsync(t.meta, 0, t.n_bins * sizeof(uint32_t), s) != cudaSuccess) return CK_ECUDA;
-    if (cudaMemsetAsync(t.counters, 0, COUNTER_WORDS * sizeof(uint64_t), s) != cudaSuccess)
-      return CK_ECUDA;
-  }
+  k_multi_clear<<<dim3(m->n_tables, CLEAR_PARTS), 256, 0, s>>>(m->d_tables);
   m->last = s;
-  return CK_OK;
+  return cudaGetLastError() == cudaSuccess ? CK_OK : CK_ECUDA;
 }
 
 }  // namespace
