@@ -15,17 +15,6 @@ __device__ __forceinline__ void flush_counter(unsigned long long* shared_slot, u
   if (x) atomicAdd(shared_slot, x);
 }
 
-// Randomised exponential backoff after a conflict: [w, 2w) ns with w =
-// 64 << attempt, up to 32-64 us, so that long walks that keep meeting each
-// other (small tables with most keys in flight) drift apart.  Measured on
-// the 2^14 x 4 table with all 62,259 keys in flight at once (1.3 claim
-// conflicts per key): capping w at 32 us rather than 1 ms fills it about 9%
-// faster; the large fills do not change.
-__device__ __forceinline__ void backoff(uint32_t attempt, uint32_t key) {
-  uint32_t w = 64u << (attempt < 9 ? attempt : 9);
-  __nanosleep(w + (fmix32(key ^ attempt) & (w - 1)));
-}
-
 template <int B, int POL, bool GHOST>
 __device__ __forceinline__ int attempt_insert(const DevTable& t, Ctx& c, uint8_t* region) {
   if constexpr (B == 1) {

@@ -19,10 +19,56 @@ namespace ck {
 
 __device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31u; }
 
+// Randomised exponential backoff after a conflict: [w, 2w) ns with w =
+// 64 << attempt, up to 32-64 us, so that long walks that keep meeting each
+// other (small tables with most keys in flight) drift apart.  Measured on
+// the 2^14 x 4 table with all 62,259 keys in flight at once (1.3 claim
+// conflicts per key): capping w at 32 us rather than 1 ms fills it about 9%
+// faster; the large fills do not change.
+__device__ __forceinline__ uint32_t backoff_ns(uint32_t attempt, uint32_t key) {
+  uint32_t w = 64u << (attempt < 9 ? attempt : 9);
+  return w + (fmix32(key ^ attempt) & (w - 1));
+}
+
+__device__ __forceinline__ void backoff(uint32_t attempt, uint32_t key) { __nanosleep(backoff_ns(attempt, key)); }
+
 // The bins-viewed histogram's bucket of a load of `at` keys.
 __device__ __forceinline__ uint32_t load_bucket(uint64_t at, uint64_t total) {
   const uint64_t x = at * HIST_BUCKETS / total;
   return x < HIST_BUCKETS ? (uint32_t)x : HIST_BUCKETS - 1;
+}
+
+// What the insertions that ended in the lanes of `over` with st add up to (the
+// whole warp calls; every lane gets the sums).
+struct KeySums {
+  uint32_t ok, failed, aborted, kicks, chain_max, viewed, viewed_all, aborts, reviews;
+};
+__device__ __forceinline__ KeySums sum_keys(bool over, const Ctx& c, int st, uint32_t aborts) {
+  constexpr unsigned ALL = 0xFFFFFFFFu;
+  KeySums s;
+  const uint32_t k = over && st == ST_OK ? c.kicks : 0u;
+  s.ok = __popc(__ballot_sync(ALL, over && st == ST_OK));
+  s.failed = __popc(__ballot_sync(ALL, over && st == ST_FAILED));
+  s.aborted = __popc(__ballot_sync(ALL, over)) - s.ok - s.failed;
+  s.kicks = __reduce_add_sync(ALL, k);
+  s.chain_max = __reduce_max_sync(ALL, k);
+  s.viewed = __reduce_add_sync(ALL, over ? c.viewed - c.viewed0 : 0u);
+  s.viewed_all = __reduce_add_sync(ALL, over ? c.viewed : 0u);
+  s.aborts = __reduce_add_sync(ALL, over ? aborts : 0u);
+  s.reviews = __reduce_add_sync(ALL, over ? c.reviews : 0u);
+  return s;
+}
+// ... into counters (a block's or a table's), by one lane
+__device__ __forceinline__ void add_sums(unsigned long long* bc, const KeySums& s) {
+  if (s.ok) atomicAdd(bc + C_INS_OK, (unsigned long long)s.ok);
+  if (s.failed) atomicAdd(bc + C_INS_FAILED, (unsigned long long)s.failed);
+  if (s.aborted) atomicAdd(bc + C_INS_ABORTED, (unsigned long long)s.aborted);
+  if (s.kicks) atomicAdd(bc + C_KICKS, (unsigned long long)s.kicks);
+  if (s.chain_max) atomicMax(bc + C_CHAIN_MAX, (unsigned long long)s.chain_max);
+  if (s.viewed) atomicAdd(bc + C_VIEWED, (unsigned long long)s.viewed);
+  if (s.viewed_all) atomicAdd(bc + C_VIEWED_ALL, (unsigned long long)s.viewed_all);
+  if (s.aborts) atomicAdd(bc + C_ABORTS, (unsigned long long)s.aborts);
+  if (s.reviews) atomicAdd(bc + C_REVIEWS, (unsigned long long)s.reviews);
 }
 
 // A block's counts, in shared memory.
@@ -80,6 +126,45 @@ struct BlockTally {
   }
 };
 
+// One lane's look at a key: placed (true) in a free slot it sees, or not;
+// `views`: the bins viewed, `lost`: the slot was taken meanwhile (an attempt
+// given up on a conflict).  Queue-kicking reads both bins and takes the less
+// full one (b0 on ties); the other policies take b0's first free slot, else
+// b1's, and fetch b1 only where b0 has none.  The searches count both bins as
+// viewed either way, as their definition does.
+template <int B, int POL>
+__device__ __forceinline__ bool look_place(const DevTable& t, uint32_t key, uint32_t val, uint32_t& views,
+                                           bool& lost) {
+  uint32_t b0, b1;
+  bins2(t, key, b0, b1);
+  View<B> v;
+  load_slots<B>(t, b0, v);
+  uint32_t g0, g1 = 0;
+  views = 2;
+  lost = false;
+  if (POL == P_QUEUE) {
+    View<B> v1;
+    load_slots<B>(t, b1, v1);
+    g0 = empty_mask<B>(v);
+    g1 = empty_mask<B>(v1);
+    if (__popc(g0) >= __popc(g1)) g1 = 0;
+    else g0 = 0;
+  } else {
+    g0 = empty_mask<B>(v);
+    if (!g0) {
+      load_slots<B>(t, b1, v);
+      g1 = empty_mask<B>(v);
+    } else if (POL == P_RANDOM) {
+      views = 1;
+    }
+  }
+  if (!(g0 | g1)) return false;
+  const bool placed = cas_slot(t.slots + (uint64_t)(g0 ? b0 : b1) * B + lowest(g0 ? g0 : g1), EMPTY,
+                               ((uint64_t)key << 32) | val);
+  lost = !placed;
+  return placed;
+}
+
 // A block's keys: the next index of its range, and per warp the keys looked
 // at that found no room.
 struct LookState {
@@ -100,10 +185,6 @@ struct LookState {
   }
 
   // One look at 32 new keys from `base` (those below hi), by a whole warp.
-  // Queue-kicking reads both bins and takes the less full one (b0 on ties);
-  // the other policies take b0's first free slot, else b1's, and fetch b1
-  // only where b0 has none.  The searches count both bins as viewed either
-  // way, as their definition does.
   template <int B, int POL>
   __device__ __forceinline__ uint32_t look(const DevTable& t, const uint32_t* __restrict__ keys,
                                            const uint32_t* __restrict__ vals, uint8_t* status, uint32_t* viewed_out,
@@ -113,39 +194,15 @@ struct LookState {
     const bool on = j < hi;
     const uint32_t key = on ? __ldcs(keys + j) : RESERVED_KEY;
     const uint32_t val = on ? __ldcs(vals + j) : 0u;
-    uint64_t* p = nullptr;
-    uint32_t views = 2;
-    if (key != RESERVED_KEY) {
-      uint32_t b0, b1;
-      bins2(t, key, b0, b1);
-      View<B> v;
-      load_slots<B>(t, b0, v);
-      uint32_t g0, g1 = 0;
-      if (POL == P_QUEUE) {
-        View<B> v1;
-        load_slots<B>(t, b1, v1);
-        g0 = empty_mask<B>(v);
-        g1 = empty_mask<B>(v1);
-        if (__popc(g0) >= __popc(g1)) g1 = 0;
-        else g0 = 0;
-      } else {
-        g0 = empty_mask<B>(v);
-        if (!g0) {
-          load_slots<B>(t, b1, v);
-          g1 = empty_mask<B>(v);
-        } else if (POL == P_RANDOM) {
-          views = 1;
-        }
-      }
-      if (g0 | g1) p = t.slots + (uint64_t)(g0 ? b0 : b1) * B + lowest(g0 ? g0 : g1);
-    }
-    const bool placed = p && cas_slot(p, EMPTY, ((uint64_t)key << 32) | val);
+    uint32_t views = 0;
+    bool lost = false;
+    const bool placed = key != RESERVED_KEY && look_place<B, POL>(t, key, val, views, lost);
     const bool invalid = on && key == RESERVED_KEY;
     if (placed || invalid) {
       if (status) status[j] = (uint8_t)(invalid ? ST_INVALID : ST_OK);
       if (viewed_out) viewed_out[j] = invalid ? 0u : views;
     }
-    const unsigned pm = __ballot_sync(0xFFFFFFFFu, placed), lm = __ballot_sync(0xFFFFFFFFu, p && !placed);
+    const unsigned pm = __ballot_sync(0xFFFFFFFFu, placed), lm = __ballot_sync(0xFFFFFFFFu, lost);
     if (pm) {
       const uint32_t n = __popc(pm);
       const uint32_t sum = POL == P_RANDOM ? __reduce_add_sync(0xFFFFFFFFu, placed ? views : 0u) : 2 * n;
@@ -166,8 +223,8 @@ struct LookState {
         atomicAdd(&bt.cnt[b], 1u);
       }
     }
-    if (lm) {  // attempts given up on a conflict
-      const uint32_t sum = __reduce_add_sync(0xFFFFFFFFu, p && !placed ? views : 0u);
+    if (lm) {
+      const uint32_t sum = __reduce_add_sync(0xFFFFFFFFu, lost ? views : 0u);
       if (lane_id() == 0) {
         atomicAdd(&bt.bc[C_ABORTS], (unsigned long long)__popc(lm));
         atomicAdd(&bt.bc[C_VIEWED_ALL], (unsigned long long)sum);

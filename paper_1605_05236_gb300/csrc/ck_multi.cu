@@ -20,6 +20,7 @@
 
 #include "ck.h"
 #include "ck_kernels.cuh"
+#include "ck_walk.cuh"
 
 using namespace ck;
 
@@ -56,7 +57,7 @@ struct ck_multi {
   unsigned long long* d_tile_ctr;
   uint8_t* buf;
   size_t bytes;
-  uint32_t n_tiles;
+  uint32_t n_tiles, n_tiles4;  // all, and those of 4-slot tables (first in the list)
   uint32_t tile;
   uint32_t block;
   uint32_t blocks_per_sm;  // 0: as many as fit
@@ -123,7 +124,8 @@ MultiLayout multi_layout(const ck_multi_desc* d, uint32_t n) {
   return L;
 }
 
-// Persistent batched insert: blocks pull tiles, threads pull keys.
+// Persistent batched insert (ghost policies): blocks pull tiles, threads pull
+// keys.
 template <int POL, bool GHOST>
 __global__ void __launch_bounds__(256, 4) k_multi_insert(const DevTable* __restrict__ tables,
                                                       const Tile* __restrict__ tiles, uint32_t n_tiles,
@@ -208,6 +210,210 @@ __global__ void __launch_bounds__(256, 4) k_multi_insert(const DevTable* __restr
   }
 }
 
+// ------------------------------------------------------------------
+// walks (tables without ghosts): lanes of a warp in tables of their own
+// ------------------------------------------------------------------
+// A warp takes pieces of SUB_TILE keys from the queue and gives its lanes the
+// keys that found no room (ck_look.cuh); a lane goes on to the next piece's
+// keys, in whichever table they are, when its walk ends, so no lane waits for
+// a tile's longest walk and a piece can be small, which keeps the tables in
+// work few enough for L2.  A warp keeps the counts of the tables it works on
+// in shared memory and adds them to a table's counters when another takes
+// the place.  4- and 8-slot tables have a launch each.
+//
+// Bound by latency (L2 round trips of looks and kicks), not by L2 or DRAM
+// rates.  Measured, clear and fill of 4096 tables (9.3 GB, 1.07e9 keys) from a
+// graph: 61 ms against 90 with a block a tile and an insertion a thread; 151
+// with the counts added to the tables' counters per 32 keys (a few lines that
+// every warp adds to); pieces of 256 / 512 / 1024 keys 72.7 / 64.8 / 61.1,
+// with the queue asked a piece ahead 512 / 1024 / 2048: 61.2 / 62.2 / 70.7;
+// 128 registers against 80: 60.9 against 62.2.
+constexpr uint32_t SUB_TILE = 512;
+constexpr uint32_t NO_TABLE = 0xFFFFFFFFu;
+
+struct PieceList {  // per warp, in shared memory
+  uint64_t left[64];     // keys without room ...
+  uint32_t left_t[64];   // ... and their tables
+  uint64_t next, hi;     // the current piece's keys that were not looked at
+  uint32_t table, n_left;
+  uint32_t sums_of[4];   // counts of table sums_of[e] (e: its index mod 4)
+  KeySums sums[4];
+};
+
+// Lane 0 of a warp: the counts in place e to their table's counters.
+__device__ __forceinline__ void flush_sums(PieceList& pl, const DevTable* tables, uint32_t e) {
+  if (pl.sums_of[e] == NO_TABLE) return;
+  unsigned long long* ct = tables[pl.sums_of[e]].counters;
+  add_sums(ct, pl.sums[e]);
+  if (pl.sums[e].ok) atomicAdd(ct + C_SIZE, (unsigned long long)pl.sums[e].ok);
+}
+
+// Lane 0 of a warp: the warp's counts of `table`.
+__device__ __forceinline__ KeySums& sums_for(PieceList& pl, const DevTable* tables, uint32_t table) {
+  const uint32_t e = table & 3u;
+  if (pl.sums_of[e] != table) {
+    flush_sums(pl, tables, e);
+    pl.sums_of[e] = table;
+    pl.sums[e] = KeySums{0, 0, 0, 0, 0, 0, 0, 0, 0};
+  }
+  return pl.sums[e];
+}
+
+template <int B, int POL>
+struct TileKeys {
+  DevTable t;  // the lane's table (the fields that differ, over the launch's common ones)
+  const DevTable* tables;
+  const Tile* tiles;
+  uint64_t n_pieces;
+  uint32_t per_tile;  // pieces a tile
+  unsigned long long* ctr;
+  const uint32_t *keys, *vals;
+  uint8_t* status;
+  PieceList& pl;
+  bool more;
+  unsigned long long ahead;  // lane 0: the queue's next piece
+  uint64_t i;
+  uint32_t key, val, tab_of;  // the lane's key, its value and its table's index
+
+  __device__ __forceinline__ const DevTable& table() const { return t; }
+
+  static __device__ __forceinline__ void enter(DevTable& d, const DevTable& s) {
+    d.slots = s.slots;
+    d.meta = s.meta;
+    d.n_bins = s.n_bins;
+    d.bin_mask = s.bin_mask;
+    if (POL == P_RANDOM) d.rng_seed = s.rng_seed;
+  }
+
+  // The warp's next piece; false: the queue is empty.  The queue's answer is
+  // asked for a piece ahead, and the piece's keys and values are brought to
+  // L2 (a line a lane).
+  __device__ __forceinline__ bool next_piece() {
+    for (;;) {
+      const unsigned long long k = __shfl_sync(0xFFFFFFFFu, ahead, 0);
+      if (k >= n_pieces) return false;
+      if (lane_id() == 0) ahead = atomicAdd(ctr, 1ull);
+      const Tile tl = tiles[k / per_tile];
+      const uint64_t lo = tl.lo + (k % per_tile) * SUB_TILE, hi = min(tl.hi, lo + SUB_TILE);
+      if (lo >= hi) continue;
+      for (uint64_t j = lo + 32 * lane_id(); j < hi; j += 32 * 32) {
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(keys + j));
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(vals + j));
+      }
+      if (lane_id() == 0) {
+        pl.table = tl.table;
+        pl.next = lo;
+        pl.hi = hi;
+      }
+      __syncwarp();
+      return true;
+    }
+  }
+
+  __device__ __forceinline__ bool take(unsigned idle) {
+    const uint32_t lane = lane_id(), want = __popc(idle);
+    uint32_t nl = pl.n_left;
+    while (nl < want) {
+      if (pl.next >= pl.hi && !next_piece()) {
+        more = false;
+        break;
+      }
+      const uint64_t j = pl.next + lane;
+      const uint32_t tab = pl.table;
+      const bool on = j < pl.hi;
+      const uint32_t k = on ? __ldcs(keys + j) : RESERVED_KEY, v = on ? __ldcs(vals + j) : 0u;
+      DevTable d = t;
+      enter(d, tables[tab]);
+      uint32_t views = 0;
+      bool lost = false;
+      const bool placed = k != RESERVED_KEY && look_place<B, POL>(d, k, v, views, lost);
+      const bool invalid = on && k == RESERVED_KEY;
+      if ((placed || invalid) && status) status[j] = (uint8_t)(invalid ? ST_INVALID : ST_OK);
+      const unsigned pm = __ballot_sync(0xFFFFFFFFu, placed), lm = __ballot_sync(0xFFFFFFFFu, lost);
+      const uint32_t seen = __reduce_add_sync(0xFFFFFFFFu, placed ? views : 0u);
+      const uint32_t wasted = lm ? __reduce_add_sync(0xFFFFFFFFu, lost ? views : 0u) : 0u;
+      if (lane == 0) {
+        KeySums& s = sums_for(pl, tables, tab);
+        s.ok += __popc(pm);
+        s.viewed += seen;
+        s.viewed_all += seen + wasted;
+        s.aborts += __popc(lm);
+      }
+      const bool rest = on && !placed && !invalid;
+      const unsigned rm = __ballot_sync(0xFFFFFFFFu, rest);
+      if (rest) {
+        const uint32_t at = nl + __popc(rm & ((1u << lane) - 1));
+        pl.left[at] = j;
+        pl.left_t[at] = tab;
+      }
+      nl += __popc(rm);
+      __syncwarp();
+      if (lane == 0) pl.next += 32;
+      __syncwarp();
+    }
+    const uint32_t give = nl < want ? nl : want, r = __popc(idle & ((1u << lane) - 1));
+    const bool got = ((idle >> lane) & 1u) && r < give;
+    if (got) {
+      i = pl.left[nl - give + r];
+      tab_of = pl.left_t[nl - give + r];
+      enter(t, tables[tab_of]);
+      key = __ldcs(keys + i);
+      val = __ldcs(vals + i);
+    }
+    __syncwarp();
+    if (lane == 0) pl.n_left = nl - give;
+    __syncwarp();
+    more = more || nl > give;
+    return got;
+  }
+
+  __device__ __forceinline__ void done(bool over, const Ctx& c, int st, uint32_t aborts) {
+    if (over && status) status[i] = (uint8_t)st;
+    for (unsigned m = __ballot_sync(0xFFFFFFFFu, over); m;) {  // a table at a time
+      const uint32_t tab = __shfl_sync(0xFFFFFFFFu, tab_of, __ffs(m) - 1);
+      const bool in = over && tab_of == tab;
+      const KeySums k = sum_keys(in, c, st, aborts);
+      if (lane_id() == 0) {
+        KeySums& s = sums_for(pl, tables, tab);
+        s.ok += k.ok;
+        s.failed += k.failed;
+        s.aborted += k.aborted;
+        s.kicks += k.kicks;
+        s.chain_max = max(s.chain_max, k.chain_max);
+        s.viewed += k.viewed;
+        s.viewed_all += k.viewed_all;
+        s.aborts += k.aborts;
+        s.reviews += k.reviews;
+      }
+      m &= ~__ballot_sync(0xFFFFFFFFu, in);
+    }
+  }
+};
+
+template <int B, int POL>
+__global__ void __launch_bounds__(256, 2) k_multi_walk(DevTable common, const DevTable* __restrict__ tables,
+                                                       const Tile* __restrict__ tiles, uint64_t n_pieces,
+                                                       uint32_t per_tile, unsigned long long* ctr,
+                                                       const uint32_t* __restrict__ keys,
+                                                       const uint32_t* __restrict__ vals,
+                                                       uint8_t* __restrict__ status) {
+  __shared__ PieceList pl[8];
+  PieceList& mine = pl[threadIdx.x >> 5];
+  if (lane_id() == 0) {
+    mine.next = mine.hi = 0;
+    mine.n_left = 0;
+    for (int e = 0; e < 4; e++) mine.sums_of[e] = NO_TABLE;
+  }
+  __syncwarp();
+  PlanStore<MAX_CHAIN> store;
+  TileKeys<B, POL> src{common, tables, tiles, n_pieces, per_tile, ctr, keys, vals, status, mine, true, 0, 0,
+                       0, 0, 0};
+  if (lane_id() == 0) src.ahead = atomicAdd(ctr, 1ull);
+  walk_keys<B, POL>(src, store.e);
+  if (lane_id() == 0)
+    for (uint32_t e = 0; e < 4; e++) flush_sums(mine, tables, e);
+}
+
 // Lookups across tables: key i belongs to table tab[i].
 __global__ void __launch_bounds__(256) k_multi_lookup(const DevTable* __restrict__ tables,
                                                       const uint32_t* __restrict__ tab,
@@ -242,54 +448,74 @@ __global__ void __launch_bounds__(256) k_multi_lookup(const DevTable* __restrict
   }
 }
 
-using MultiFn = void (*)(const ck_multi*, const uint32_t*, const uint32_t*, uint8_t*, cudaStream_t, unsigned,
-                         unsigned);
-
-template <int POL, bool GHOST>
-void launch_multi(const ck_multi* m, const uint32_t* k, const uint32_t* v, uint8_t* st, cudaStream_t s,
-                  unsigned grid, unsigned block) {
-  k_multi_insert<POL, GHOST><<<grid, block, 0, s>>>(m->d_tables, m->d_tiles, m->n_tiles, m->d_tile_ctr, k, v, st);
-}
-
-MultiFn pick_multi(uint32_t policy) {
-  bool g = (policy & CK_GHOST) != 0;
-  switch (policy & 0xFF) {
-    case CK_RANDOM: return g ? launch_multi<P_RANDOM, true> : launch_multi<P_RANDOM, false>;
-    case CK_QUEUE: return g ? launch_multi<P_QUEUE, true> : launch_multi<P_QUEUE, false>;
-    default: return nullptr;
-  }
-}
-
-int occupancy_blocks(uint32_t policy, uint32_t block) {
+// The launches of one batched insertion, and the blocks of each that fit on
+// an SM.  Ghost policies: one launch of k_multi_insert over all tiles; the
+// others: k_multi_walk over the tiles of the 4-slot tables, then of the
+// 8-slot ones.
+template <class K>
+int blocks_that_fit(K kernel, uint32_t block) {
   int per_sm = 0;
-  cudaError_t e = cudaErrorInvalidValue;
-  bool g = (policy & CK_GHOST) != 0;
-  if ((policy & 0xFF) == CK_QUEUE)
-    e = g ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_multi_insert<P_QUEUE, true>, block, 0)
-          : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_multi_insert<P_QUEUE, false>, block, 0);
-  else
-    e = g ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_multi_insert<P_RANDOM, true>, block, 0)
-          : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_multi_insert<P_RANDOM, false>, block, 0);
-  if (e != cudaSuccess || per_sm < 1) return 1;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, 0) != cudaSuccess || per_sm < 1) return 1;
   return per_sm;
 }
 
-// Build the tile list for the current tile size and upload it.  The tables
-// are taken in groups of about WINDOW_BYTES, in order, and the tiles of a
+unsigned grid_of(const ck_multi* m, int fit, uint64_t most) {
+  int per_sm = fit;
+  if (m->blocks_per_sm && (int)m->blocks_per_sm < per_sm) per_sm = (int)m->blocks_per_sm;
+  const uint64_t g = (uint64_t)per_sm * m->sm_count;
+  return (unsigned)(g < most ? g : most > 0 ? most : 1);
+}
+
+template <int POL>
+void launch_ghost(const ck_multi* m, const uint32_t* k, const uint32_t* v, uint8_t* st, cudaStream_t s) {
+  const unsigned grid = grid_of(m, blocks_that_fit(k_multi_insert<POL, true>, m->block), m->n_tiles);
+  k_multi_insert<POL, true><<<grid, m->block, 0, s>>>(m->d_tables, m->d_tiles, m->n_tiles, m->d_tile_ctr, k, v, st);
+}
+
+template <int B, int POL>
+void launch_walk(const ck_multi* m, const uint32_t* k, const uint32_t* v, uint8_t* st, cudaStream_t s) {
+  const uint32_t first = B == 4 ? 0 : m->n_tiles4, n = B == 4 ? m->n_tiles4 : m->n_tiles - m->n_tiles4;
+  if (!n) return;
+  const uint32_t per_tile = (m->tile + SUB_TILE - 1) / SUB_TILE;
+  const uint64_t pieces = (uint64_t)n * per_tile;
+  const uint32_t warps = m->block / 32;
+  const unsigned grid = grid_of(m, blocks_that_fit(k_multi_walk<B, POL>, m->block), (pieces + warps - 1) / warps);
+  k_multi_walk<B, POL><<<grid, m->block, 0, s>>>(m->host_tables[0], m->d_tables, m->d_tiles + first, pieces, per_tile,
+                                                 m->d_tile_ctr + (B == 4 ? 0 : 1), k, v, st);
+}
+
+bool launch_multi(const ck_multi* m, const uint32_t* k, const uint32_t* v, uint8_t* st, cudaStream_t s) {
+  const bool g = (m->policy & CK_GHOST) != 0;
+  switch (m->policy & 0xFF) {
+    case CK_RANDOM:
+      if (g) return launch_ghost<P_RANDOM>(m, k, v, st, s), true;
+      launch_walk<4, P_RANDOM>(m, k, v, st, s);
+      launch_walk<8, P_RANDOM>(m, k, v, st, s);
+      return true;
+    case CK_QUEUE:
+      if (g) return launch_ghost<P_QUEUE>(m, k, v, st, s), true;
+      launch_walk<4, P_QUEUE>(m, k, v, st, s);
+      launch_walk<8, P_QUEUE>(m, k, v, st, s);
+      return true;
+    default: return false;
+  }
+}
+
+// Build the tile list for the current tile size and upload it: the tiles of
+// the 4-slot tables, then those of the 8-slot ones.  The tables of a kind are
+// taken in groups of about WINDOW_BYTES, in order, and the tiles of a
 // group round-robin over its tables (tile r of each, then tile r + 1): the
 // tables being filled stay in L2 from their first tile to their last, and
 // each keeps only a part of its tiles in flight, so its load grows in order.
-std::vector<Tile> make_tiles(const ck_multi_desc* desc, uint32_t n_tables, uint32_t tile) {
-  std::vector<Tile> tiles;
-  tiles.reserve(count_tiles(desc, n_tables, tile));
-  for (uint32_t first = 0, last; first < n_tables; first = last) {
-    size_t bytes = 0;
-    for (last = first; last < n_tables && (last == first || bytes + table_bytes(desc[last]) <= WINDOW_BYTES); last++)
-      bytes += table_bytes(desc[last]);
+void add_tiles(std::vector<Tile>& tiles, const ck_multi_desc* desc, uint32_t n_tables, uint32_t slots,
+               uint32_t tile) {
+  std::vector<uint32_t> group;
+  size_t bytes = 0;
+  auto flush = [&]() {
     bool any = true;
     for (uint64_t r = 0; any; r++) {
       any = false;
-      for (uint32_t i = first; i < last; i++) {
+      for (const uint32_t i : group) {
         const ck_multi_desc& d = desc[i];
         const uint64_t lo = r * tile;
         if (lo >= d.n_keys) continue;
@@ -297,12 +523,25 @@ std::vector<Tile> make_tiles(const ck_multi_desc* desc, uint32_t n_tables, uint3
         tiles.push_back({i, 0, d.key_offset + lo, d.key_offset + (lo + tile < d.n_keys ? lo + tile : d.n_keys)});
       }
     }
+    group.clear();
+    bytes = 0;
+  };
+  for (uint32_t i = 0; i < n_tables; i++) {
+    if (desc[i].slots_per_bin != slots) continue;
+    const size_t b = table_bytes(desc[i]);
+    if (bytes + b > WINDOW_BYTES) flush();
+    group.push_back(i);
+    bytes += b;
   }
-  return tiles;
+  flush();
 }
 
 int build_tiles(ck_multi* m, cudaStream_t s) {
-  const std::vector<Tile> tiles = make_tiles(m->desc.data(), m->n_tables, m->tile);
+  std::vector<Tile> tiles;
+  tiles.reserve(count_tiles(m->desc.data(), m->n_tables, m->tile));
+  add_tiles(tiles, m->desc.data(), m->n_tables, 4, m->tile);
+  m->n_tiles4 = (uint32_t)tiles.size();
+  add_tiles(tiles, m->desc.data(), m->n_tables, 8, m->tile);
   m->n_tiles = (uint32_t)tiles.size();
   if (cudaMemcpyAsync(m->d_tiles, tiles.data(), tiles.size() * sizeof(Tile), cudaMemcpyHostToDevice, s) !=
       cudaSuccess)
@@ -461,14 +700,8 @@ int ck_multi_set_param(ck_multi* m, int key, int64_t value) {
 int ck_multi_insert(ck_multi* m, const uint32_t* d_keys, const uint32_t* d_vals, uint8_t* d_status, void* stream) {
   if (!m || !d_keys || !d_vals) return CK_EINVAL;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  MultiFn fn = pick_multi(m->policy);
-  if (!fn) return CK_ENOTSUP;
-  int per_sm = occupancy_blocks(m->policy, m->block);
-  if (m->blocks_per_sm && (int)m->blocks_per_sm < per_sm) per_sm = (int)m->blocks_per_sm;
-  unsigned grid = (unsigned)(per_sm * m->sm_count);
-  if (grid > m->n_tiles) grid = m->n_tiles ? m->n_tiles : 1;
-  if (cudaMemsetAsync(m->d_tile_ctr, 0, sizeof(unsigned long long), s) != cudaSuccess) return CK_ECUDA;
-  fn(m, d_keys, d_vals, d_status, s, grid, m->block);
+  if (cudaMemsetAsync(m->d_tile_ctr, 0, 2 * sizeof(unsigned long long), s) != cudaSuccess) return CK_ECUDA;
+  if (!launch_multi(m, d_keys, d_vals, d_status, s)) return CK_ENOTSUP;
   m->last = s;
   return cudaGetLastError() == cudaSuccess ? CK_OK : CK_ECUDA;
 }

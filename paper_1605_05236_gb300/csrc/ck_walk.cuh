@@ -202,6 +202,136 @@ __device__ __forceinline__ void walk_commit(const DevTable& t, Ctx& c) {
 // room for the next launch's (6.43 against 6.46 with every block waiting).
 constexpr int WAITERS = 2;
 
+// Insert the keys of `src`, by a whole warp.  `src` gives each lane its keys
+// and the table they go into, and counts what became of them:
+//   more            keys may be left (the same in all lanes)
+//   take(idle)      the whole warp calls; true in a lane of `idle` that got a
+//                   key (src.key, src.val)
+//   table()         the lane's table
+//   done(over, c, st, aborts)   the whole warp calls: the ends of the keys of
+//                   the lanes with `over`
+template <int B, int POL, class Src>
+__device__ __forceinline__ void walk_keys(Src& src, uint64_t* local_e) {
+  // a lane has no key; has one whose next attempt begins; walks; has an
+  // attempt that ended with st; waits before its next attempt
+  enum Mode { IDLE, READY, WALKING, ENDED, WAITING };
+  int mode = IDLE, st = ST_OK;
+  Ctx c;
+  c.ghosts_made = c.dup_evict = 0;
+  c.kicks = c.viewed = c.viewed0 = c.reviews = 0;
+  Walk<B> w;
+  uint32_t fails = 0, aborts = 0, wake = 0;
+  for (;;) {
+    if (mode == WAITING && (int)((uint32_t)clock() - wake) >= 0) mode = READY;
+    const unsigned walking = __ballot_sync(0xFFFFFFFFu, mode == WALKING);
+    const unsigned waiting = __ballot_sync(0xFFFFFFFFu, mode == WAITING);
+    const unsigned need = __ballot_sync(0xFFFFFFFFu, mode == ENDED || mode == READY || (mode == IDLE && src.more));
+    if (!(walking | waiting | need)) break;
+    if (need && __popc(need) >= WAITERS * __popc(walking)) {
+      bool over = false;
+      if (mode == ENDED) {  // as insert_one ends an attempt
+        if (st == ST_OK) {
+          walk_commit<B>(src.table(), c);
+          over = true;
+        } else {
+          release_all(src.table(), c);
+          const bool ran_out = st == ST_FAILED || c.capped;
+          if (ran_out) {
+            over = ++fails > (st == ST_FAILED ? 6u : 32u);
+            if (over) st = ST_FAILED;
+          } else {
+            aborts++;
+          }
+          if (!over && ++c.attempt >= src.table().max_retries) {
+            st = ST_ABORTED;
+            over = true;
+          }
+          if (!over) {
+            wake = (uint32_t)clock() + 2 * backoff_ns(ran_out ? 6 + 2 * fails : c.attempt, c.key);
+            mode = WAITING;
+          }
+        }
+      }
+      if (over && c.long_id >= 0) release_long(src.table(), c.long_id);
+      if (__any_sync(0xFFFFFFFFu, over)) src.done(over, c, st, aborts);
+      if (over) mode = IDLE;
+      // keys for the idle lanes
+      const unsigned idle = __ballot_sync(0xFFFFFFFFu, mode == IDLE);
+      if (idle && src.more && src.take(idle)) {
+        c.key = src.key;
+        c.krec = ((uint64_t)src.key << 32) | src.val;
+        c.attempt = 0;
+        c.viewed = 0;
+        c.reviews = 0;
+        c.long_id = -1;
+        fails = 0;
+        aborts = 0;
+        mode = READY;
+      }
+      if (mode == READY) {
+        c.kicks = 0;
+        c.draws = 0;
+        c.viewed0 = c.viewed;
+        c.foreign = 0;
+        c.capped = 0;
+        if (c.long_id < 0) {
+          c.pe = local_e;
+          c.pcap = MAX_CHAIN;
+        }
+        c.pn = 0;
+        st = walk_begin<B, POL>(src.table(), c, w);
+        mode = st == WALK ? WALKING : ENDED;
+      }
+    }
+    if (mode == WALKING) {
+      st = walk_step<B, POL>(src.table(), c, w);
+      if (st != WALK) mode = ENDED;
+    } else if (!walking && !need) {
+      __nanosleep(100);
+    }
+    __syncwarp();
+  }
+}
+
+// The keys lo .. hi - 1 of a batch, into one table.
+template <int B, int POL>
+struct BatchKeys {
+  const DevTable& t;
+  const uint32_t *keys, *vals;
+  uint8_t* status;
+  uint32_t* viewed_out;
+  uint64_t hi, load_base;
+  BlockTally& bt;
+  LookState& ls;
+  bool more;
+  uint64_t i;
+  uint32_t key, val;
+
+  __device__ __forceinline__ const DevTable& table() const { return t; }
+  __device__ __forceinline__ bool take(unsigned idle) {
+    uint64_t got = hi;
+    more = ls.template take<B, POL>(t, keys, vals, status, viewed_out, hi, load_base, idle, bt, got);
+    if (got >= hi) return false;
+    i = got;
+    key = __ldcs(keys + i);
+    val = __ldcs(vals + i);
+    return true;
+  }
+  __device__ __forceinline__ void done(bool over, const Ctx& c, int st, uint32_t aborts) {
+    if (over) {
+      const uint32_t v = c.viewed - c.viewed0;
+      if (status) status[i] = (uint8_t)st;
+      if (viewed_out) viewed_out[i] = v;
+      const uint32_t b = load_bucket(load_base + i, t.total_slots);
+      atomicAdd(&bt.views[b], v);
+      atomicAdd(&bt.cnt[b], 1u);
+      if (st == ST_OK) atomicAdd(&bt.chain[chain_bucket(c.kicks)], 1u);
+    }
+    const KeySums s = sum_keys(over, c, st, aborts);
+    if (lane_id() == 0) add_sums(bt.bc, s);
+  }
+};
+
 template <int B, int POL>
 __global__ void __launch_bounds__(256, 3) k_insert_walk(DevTable t, const uint32_t* __restrict__ keys,
                                                         const uint32_t* __restrict__ vals, uint64_t n,
@@ -215,105 +345,9 @@ __global__ void __launch_bounds__(256, 3) k_insert_walk(DevTable t, const uint32
   bt.clear();
   ls.begin(t, lo, load_base);
   __syncthreads();
-
   PlanStore<MAX_CHAIN> store;
-  // a lane has no key; has one whose next attempt begins; walks; has an
-  // attempt that ended with st; waits before its next attempt
-  enum Mode { IDLE, READY, WALKING, ENDED, WAITING };
-  int mode = IDLE, st = ST_OK;
-  Ctx c;
-  c.ghosts_made = c.dup_evict = 0;
-  Walk<B> w;
-  uint64_t i = 0;
-  uint32_t fails = 0, aborts = 0, wake = 0;
-  uint32_t ok = 0, viewed = 0, viewed_all = 0;
-  bool more = true;  // keys are left in the block's range (or in the warp's list)
-  for (;;) {
-    const unsigned walking = __ballot_sync(0xFFFFFFFFu, mode == WALKING);
-    if (mode == WAITING && (int)((uint32_t)clock() - wake) >= 0) mode = READY;
-    const unsigned waiting = __ballot_sync(0xFFFFFFFFu, mode == WAITING);
-    const unsigned need = __ballot_sync(0xFFFFFFFFu, mode == ENDED || mode == READY || (mode == IDLE && more));
-    if (!(walking | waiting | need)) break;
-    if (need && (__popc(need) >= WAITERS * __popc(walking))) {
-      if (mode == ENDED) {  // as insert_one ends an attempt
-        if (st == ST_OK) {
-          walk_commit<B>(t, c);
-        } else {
-          release_all(t, c);
-          const bool ran_out = st == ST_FAILED || c.capped;
-          bool over = false;
-          if (ran_out) {
-            over = ++fails > (st == ST_FAILED ? 6u : 32u);
-            if (over) st = ST_FAILED;
-          } else {
-            aborts++;
-          }
-          if (!over && ++c.attempt >= t.max_retries) {
-            st = ST_ABORTED;
-            over = true;
-          }
-          if (!over) {
-            const uint32_t a = ran_out ? 6 + 2 * fails : c.attempt;
-            const uint32_t ns = 64u << (a < 9 ? a : 9);
-            wake = (uint32_t)clock() + 2 * (ns + (fmix32(c.key ^ a) & (ns - 1)));
-            mode = WAITING;
-          }
-        }
-        if (mode == ENDED) {
-          if (c.long_id >= 0) release_long(t, c.long_id);
-          if (status) status[i] = (uint8_t)st;
-          if (viewed_out) viewed_out[i] = c.viewed - c.viewed0;
-          bt.key_done(c, st, aborts, c.viewed - c.viewed0, load_bucket(load_base + i, t.total_slots));
-          ok += st == ST_OK;
-          viewed += c.viewed - c.viewed0;
-          viewed_all += c.viewed;
-          mode = IDLE;
-        }
-      }
-      // keys for the idle lanes
-      const unsigned idle = __ballot_sync(0xFFFFFFFFu, mode == IDLE);
-      if (idle && more) {
-        uint64_t got = hi;
-        more = ls.template take<B, POL>(t, keys, vals, status, viewed_out, hi, load_base, idle, bt, got);
-        if (got < hi) {
-          i = got;
-          c.key = __ldcs(keys + i);
-          c.krec = ((uint64_t)c.key << 32) | __ldcs(vals + i);
-          c.attempt = 0;
-          c.viewed = 0;
-          c.reviews = 0;
-          c.long_id = -1;
-          fails = 0;
-          aborts = 0;
-          mode = READY;
-        }
-      }
-      if (mode == READY) {
-        c.kicks = 0;
-        c.draws = 0;
-        c.viewed0 = c.viewed;
-        c.foreign = 0;
-        c.capped = 0;
-        if (c.long_id < 0) {
-          c.pe = store.e;
-          c.pcap = MAX_CHAIN;
-        }
-        c.pn = 0;
-        st = walk_begin<B, POL>(t, c, w);
-        mode = st == WALK ? WALKING : ENDED;
-      }
-    }
-    if (mode == WALKING) {
-      st = walk_step<B, POL>(t, c, w);
-      if (st != WALK) mode = ENDED;
-    } else if (!walking && !need) {
-      __nanosleep(100);
-    }
-    __syncwarp();
-  }
-  if (ok) atomicAdd(&bt.bc[C_INS_OK], (unsigned long long)ok);
-  if (viewed) atomicAdd(&bt.bc[C_VIEWED], (unsigned long long)viewed);
-  if (viewed_all) atomicAdd(&bt.bc[C_VIEWED_ALL], (unsigned long long)viewed_all);
+  BatchKeys<B, POL> src{t, keys, vals, status, viewed_out, hi, load_base, bt, ls, true, 0, 0, 0};
+  walk_keys<B, POL>(src, store.e);
   __syncthreads();
   bt.flush(t);
   if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");  // see WAITERS
