@@ -286,6 +286,35 @@ __device__ __forceinline__ uint32_t add_relaxed(uint32_t* p, uint32_t delta) {
   return a.fetch_add(delta, cuda::memory_order_relaxed);
 }
 
+// 64-bit counters of a block in shared memory, added to by 32-bit atomics with
+// a carry: shared memory has no 64-bit atomic add, and the compare-and-swap
+// loop it is built from lets one lane of a warp through at a time.  With
+// those, the end of one 256-thread block that deletes 256 keys (two counts a
+// thread) took most of 27 us.
+__device__ __forceinline__ void count_add(unsigned long long* c, uint32_t x) {
+  uint32_t* w = reinterpret_cast<uint32_t*>(c);
+  const uint32_t old = atomicAdd(w, x);
+  if (old + x < old) atomicAdd(w + 1, 1u);
+}
+// the same for a value of every lane of a warp (all of them call)
+__device__ __forceinline__ void count_add_warp(unsigned long long* c, uint32_t x) {
+  x = __reduce_add_sync(0xFFFFFFFFu, x);
+  if ((threadIdx.x & 31u) == 0 && x) count_add(c, x);
+}
+// The next index from a block's 64-bit counter, for each of the lanes that
+// call together: one add for all of them.
+__device__ __forceinline__ uint64_t take_index(unsigned long long* next) {
+  const unsigned m = __activemask(), lane = threadIdx.x & 31u;
+  const int leader = __ffs(m) - 1;
+  unsigned long long base = 0;
+  if ((int)lane == leader) base = atomicAdd(next, (unsigned long long)__popc(m));
+  return __shfl_sync(m, base, leader) + __popc(m & ((1u << lane) - 1));
+}
+// the maximum of 32-bit values in such a counter
+__device__ __forceinline__ void count_max(unsigned long long* c, uint32_t x) {
+  atomicMax(reinterpret_cast<uint32_t*>(c), x);
+}
+
 // A view of one bin: its metadata word, then its B slots.
 template <int B>
 struct View {

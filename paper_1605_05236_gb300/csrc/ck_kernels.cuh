@@ -6,15 +6,6 @@
 
 namespace ck {
 
-// Block-wide accumulation of per-thread counts, then one global add each.
-struct BlockCounters {
-  unsigned long long v[C_N];
-};
-
-__device__ __forceinline__ void flush_counter(unsigned long long* shared_slot, unsigned long long x) {
-  if (x) atomicAdd(shared_slot, x);
-}
-
 template <int B, int POL, bool GHOST>
 __device__ __forceinline__ int attempt_insert(const DevTable& t, Ctx& c, uint8_t* region) {
   if constexpr (B == 1) {
@@ -386,7 +377,7 @@ __global__ void __launch_bounds__(256, insert_blocks_per_sm<B, POL>()) k_insert(
       DelPlan up;
       int r = update_one<B>(t, key, c.krec, up);
       if (r != 0) {
-        atomicAdd(&bt.bc[r == 1 ? C_UPDATES : C_INS_ABORTED], 1ull);
+        count_add(&bt.bc[r == 1 ? C_UPDATES : C_INS_ABORTED], 1u);
         if (status) status[i] = (uint8_t)(r == 1 ? ST_UPDATED : ST_ABORTED);
         if (viewed_out) viewed_out[i] = 0;
         return;
@@ -421,13 +412,19 @@ __global__ void __launch_bounds__(256, insert_blocks_per_sm<B, POL>()) k_insert(
         continue;
       }
     }
-    i = atomicAdd(&s_next, 1ull);
+    i = take_index(&s_next);
     if (i >= hi) break;
     insert(i);
   }
-  flush_counter(&bt.bc[C_INS_OK], ok);
-  flush_counter(&bt.bc[C_VIEWED], viewed);
-  flush_counter(&bt.bc[C_VIEWED_ALL], viewed_all);
+  if constexpr (SERIAL) {
+    count_add(&bt.bc[C_INS_OK], ok);
+    count_add(&bt.bc[C_VIEWED], viewed);
+    count_add(&bt.bc[C_VIEWED_ALL], viewed_all);
+  } else {
+    count_add_warp(&bt.bc[C_INS_OK], ok);
+    count_add_warp(&bt.bc[C_VIEWED], viewed);
+    count_add_warp(&bt.bc[C_VIEWED_ALL], viewed_all);
+  }
   __syncthreads();
   bt.flush(t);
   if (threadIdx.x == 0) {
@@ -506,8 +503,8 @@ __global__ void __launch_bounds__(256) k_lookup2(DevTable t, const uint32_t* __r
   hits = __reduce_add_sync(0xffffffffu, hits);
   cnt = __reduce_add_sync(0xffffffffu, cnt);
   if ((threadIdx.x & 31) == 0) {
-    if (hits) atomicAdd(&hits_sh, (unsigned long long)hits);
-    if (cnt) atomicAdd(&cnt_sh, (unsigned long long)cnt);
+    if (hits) count_add(&hits_sh, hits);
+    if (cnt) count_add(&cnt_sh, cnt);
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -547,8 +544,8 @@ static __global__ void __launch_bounds__(256) k_lookup_dary(DevTable t, const ui
   hits = __reduce_add_sync(0xffffffffu, hits);
   cnt = __reduce_add_sync(0xffffffffu, cnt);
   if ((threadIdx.x & 31) == 0) {
-    if (hits) atomicAdd(&hits_sh, (unsigned long long)hits);
-    if (cnt) atomicAdd(&cnt_sh, (unsigned long long)cnt);
+    if (hits) count_add(&hits_sh, hits);
+    if (cnt) count_add(&cnt_sh, cnt);
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -618,10 +615,10 @@ __global__ void __launch_bounds__(256) k_delete(DevTable t, const uint32_t* __re
     cnt++;
     if (found_out) found_out[i] = (uint8_t)r;
   }
-  if (hits) atomicAdd(&bc[0], (unsigned long long)hits);
-  if (aborts) atomicAdd(&bc[1], (unsigned long long)aborts);
-  if (ghosts) atomicAdd(&bc[2], (unsigned long long)ghosts);
-  if (cnt) atomicAdd(&bc[3], (unsigned long long)cnt);
+  count_add_warp(&bc[0], hits);
+  count_add_warp(&bc[1], aborts);
+  count_add_warp(&bc[2], ghosts);
+  count_add_warp(&bc[3], cnt);
   __syncthreads();
   if (threadIdx.x == 0) {
     if (bc[0]) {

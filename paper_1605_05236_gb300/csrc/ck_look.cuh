@@ -58,17 +58,27 @@ __device__ __forceinline__ KeySums sum_keys(bool over, const Ctx& c, int st, uin
   s.reviews = __reduce_add_sync(ALL, over ? c.reviews : 0u);
   return s;
 }
-// ... into counters (a block's or a table's), by one lane
+// ... into a block's counters (shared memory) or a table's (global), by one
+// lane
+template <bool SHARED>
 __device__ __forceinline__ void add_sums(unsigned long long* bc, const KeySums& s) {
-  if (s.ok) atomicAdd(bc + C_INS_OK, (unsigned long long)s.ok);
-  if (s.failed) atomicAdd(bc + C_INS_FAILED, (unsigned long long)s.failed);
-  if (s.aborted) atomicAdd(bc + C_INS_ABORTED, (unsigned long long)s.aborted);
-  if (s.kicks) atomicAdd(bc + C_KICKS, (unsigned long long)s.kicks);
-  if (s.chain_max) atomicMax(bc + C_CHAIN_MAX, (unsigned long long)s.chain_max);
-  if (s.viewed) atomicAdd(bc + C_VIEWED, (unsigned long long)s.viewed);
-  if (s.viewed_all) atomicAdd(bc + C_VIEWED_ALL, (unsigned long long)s.viewed_all);
-  if (s.aborts) atomicAdd(bc + C_ABORTS, (unsigned long long)s.aborts);
-  if (s.reviews) atomicAdd(bc + C_REVIEWS, (unsigned long long)s.reviews);
+  auto add = [&](int k, uint32_t x) {
+    if (!x) return;
+    if (SHARED) count_add(bc + k, x);
+    else atomicAdd(bc + k, (unsigned long long)x);
+  };
+  add(C_INS_OK, s.ok);
+  add(C_INS_FAILED, s.failed);
+  add(C_INS_ABORTED, s.aborted);
+  add(C_KICKS, s.kicks);
+  if (s.chain_max) {
+    if (SHARED) count_max(bc + C_CHAIN_MAX, s.chain_max);
+    else atomicMax(bc + C_CHAIN_MAX, (unsigned long long)s.chain_max);
+  }
+  add(C_VIEWED, s.viewed);
+  add(C_VIEWED_ALL, s.viewed_all);
+  add(C_ABORTS, s.aborts);
+  add(C_REVIEWS, s.reviews);
 }
 
 // A block's counts, in shared memory.
@@ -87,17 +97,17 @@ struct BlockTally {
   __device__ __forceinline__ void key_done(const Ctx& c, int st, uint32_t aborts, uint32_t v, uint32_t bucket) {
     if (st == ST_OK) {
       if (c.kicks) {
-        atomicAdd(&bc[C_KICKS], (unsigned long long)c.kicks);
-        atomicMax(&bc[C_CHAIN_MAX], (unsigned long long)c.kicks);
+        count_add(&bc[C_KICKS], c.kicks);
+        count_max(&bc[C_CHAIN_MAX], c.kicks);
       }
       atomicAdd(&chain[chain_bucket(c.kicks)], 1u);
-      if (c.ghosts_made) atomicAdd(&bc[C_GHOSTS_MADE], (unsigned long long)c.ghosts_made);
-      if (c.dup_evict) atomicAdd(&bc[C_DUP_EVICT], (unsigned long long)c.dup_evict);
+      if (c.ghosts_made) count_add(&bc[C_GHOSTS_MADE], c.ghosts_made);
+      if (c.dup_evict) count_add(&bc[C_DUP_EVICT], c.dup_evict);
     } else {
-      atomicAdd(&bc[st == ST_FAILED ? C_INS_FAILED : C_INS_ABORTED], 1ull);
+      count_add(&bc[st == ST_FAILED ? C_INS_FAILED : C_INS_ABORTED], 1u);
     }
-    if (aborts) atomicAdd(&bc[C_ABORTS], (unsigned long long)aborts);
-    if (c.reviews) atomicAdd(&bc[C_REVIEWS], (unsigned long long)c.reviews);
+    if (aborts) count_add(&bc[C_ABORTS], aborts);
+    if (c.reviews) count_add(&bc[C_REVIEWS], c.reviews);
     atomicAdd(&views[bucket], v);
     atomicAdd(&cnt[bucket], 1u);
   }
@@ -208,9 +218,9 @@ struct LookState {
       const uint32_t sum = POL == P_RANDOM ? __reduce_add_sync(0xFFFFFFFFu, placed ? views : 0u) : 2 * n;
       const bool one = base + 32 <= bucket_end;  // the block's first bucket: one add for the warp
       if (lane_id() == 0) {
-        atomicAdd(&bt.bc[C_INS_OK], (unsigned long long)n);
-        atomicAdd(&bt.bc[C_VIEWED], (unsigned long long)sum);
-        atomicAdd(&bt.bc[C_VIEWED_ALL], (unsigned long long)sum);
+        count_add(&bt.bc[C_INS_OK], n);
+        count_add(&bt.bc[C_VIEWED], sum);
+        count_add(&bt.bc[C_VIEWED_ALL], sum);
         atomicAdd(&bt.chain[0], n);
         if (one) {
           atomicAdd(&bt.views[bucket], sum);
@@ -226,8 +236,8 @@ struct LookState {
     if (lm) {
       const uint32_t sum = __reduce_add_sync(0xFFFFFFFFu, lost ? views : 0u);
       if (lane_id() == 0) {
-        atomicAdd(&bt.bc[C_ABORTS], (unsigned long long)__popc(lm));
-        atomicAdd(&bt.bc[C_VIEWED_ALL], (unsigned long long)sum);
+        count_add(&bt.bc[C_ABORTS], __popc(lm));
+        count_add(&bt.bc[C_VIEWED_ALL], sum);
       }
     }
     const bool rest = on && !placed && !invalid;

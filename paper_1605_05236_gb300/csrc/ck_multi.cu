@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(256, 4) k_multi_insert(const DevTable* __restr
     uint32_t ok = 0, failed = 0, aborted = 0, viewed = 0, viewed_all = 0, kicks = 0;  // per tile
     uint32_t aborts = 0, chain_max = 0, ghosts = 0, dupev = 0;
     for (;;) {
-      unsigned long long i = atomicAdd(&s_next, 1ull);
+      const uint64_t i = take_index(&s_next);
       if (i >= hi) break;
       uint32_t key = keys[i];
       if (key == RESERVED_KEY) {
@@ -185,16 +185,16 @@ __global__ void __launch_bounds__(256, 4) k_multi_insert(const DevTable* __restr
       viewed_all += c.viewed;
       if (status) status[i] = (uint8_t)st;
     }
-    if (ok) atomicAdd(&bc[C_INS_OK], ok);
-    if (failed) atomicAdd(&bc[C_INS_FAILED], failed);
-    if (aborted) atomicAdd(&bc[C_INS_ABORTED], aborted);
-    if (viewed) atomicAdd(&bc[C_VIEWED], viewed);
-    if (viewed_all) atomicAdd(&bc[C_VIEWED_ALL], viewed_all);
-    if (kicks) atomicAdd(&bc[C_KICKS], kicks);
-    if (aborts) atomicAdd(&bc[C_ABORTS], (unsigned long long)aborts);
-    if (ghosts) atomicAdd(&bc[C_GHOSTS_MADE], (unsigned long long)ghosts);
-    if (dupev) atomicAdd(&bc[C_DUP_EVICT], (unsigned long long)dupev);
-    if (chain_max) atomicMax(&bc[C_CHAIN_MAX], (unsigned long long)chain_max);
+    if (ok) count_add(&bc[C_INS_OK], ok);
+    if (failed) count_add(&bc[C_INS_FAILED], failed);
+    if (aborted) count_add(&bc[C_INS_ABORTED], aborted);
+    if (viewed) count_add(&bc[C_VIEWED], viewed);
+    if (viewed_all) count_add(&bc[C_VIEWED_ALL], viewed_all);
+    if (kicks) count_add(&bc[C_KICKS], kicks);
+    if (aborts) count_add(&bc[C_ABORTS], aborts);
+    if (ghosts) count_add(&bc[C_GHOSTS_MADE], ghosts);
+    if (dupev) count_add(&bc[C_DUP_EVICT], dupev);
+    if (chain_max) count_max(&bc[C_CHAIN_MAX], chain_max);
     __syncthreads();
     if (threadIdx.x == 0) {
       for (int k = 0; k < C_N; k++) {
@@ -244,7 +244,7 @@ struct PieceList {  // per warp, in shared memory
 __device__ __forceinline__ void flush_sums(PieceList& pl, const DevTable* tables, uint32_t e) {
   if (pl.sums_of[e] == NO_TABLE) return;
   unsigned long long* ct = tables[pl.sums_of[e]].counters;
-  add_sums(ct, pl.sums[e]);
+  add_sums<false>(ct, pl.sums[e]);
   if (pl.sums[e].ok) atomicAdd(ct + C_SIZE, (unsigned long long)pl.sums[e].ok);
 }
 

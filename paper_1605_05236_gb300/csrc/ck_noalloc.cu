@@ -102,16 +102,16 @@ __global__ void __launch_bounds__(128) k_insert_noalloc(DevTable t, uint8_t* scr
     if (status) status[i] = (uint8_t)st;
     if (st != ST_INVALID) {
       const uint32_t v_final = c.viewed - c.viewed0;
-      atomicAdd(&bc[st == ST_OK ? C_INS_OK : st == ST_FAILED ? C_INS_FAILED : C_INS_ABORTED], 1ull);
-      atomicAdd(&bc[C_VIEWED], (unsigned long long)v_final);
-      atomicAdd(&bc[C_VIEWED_ALL], (unsigned long long)c.viewed);
-      if (aborts) atomicAdd(&bc[C_ABORTS], (unsigned long long)aborts);
-      if (c.reviews) atomicAdd(&bc[C_REVIEWS], (unsigned long long)c.reviews);
+      count_add(&bc[st == ST_OK ? C_INS_OK : st == ST_FAILED ? C_INS_FAILED : C_INS_ABORTED], 1u);
+      count_add(&bc[C_VIEWED], v_final);
+      count_add(&bc[C_VIEWED_ALL], c.viewed);
+      if (aborts) count_add(&bc[C_ABORTS], aborts);
+      if (c.reviews) count_add(&bc[C_REVIEWS], c.reviews);
       if (st == ST_OK) {
-        atomicAdd(&bc[C_KICKS], (unsigned long long)c.kicks);
-        atomicMax(&bc[C_CHAIN_MAX], (unsigned long long)c.kicks);
-        if (c.ghosts_made) atomicAdd(&bc[C_GHOSTS_MADE], (unsigned long long)c.ghosts_made);
-        if (c.dup_evict) atomicAdd(&bc[C_DUP_EVICT], (unsigned long long)c.dup_evict);
+        count_add(&bc[C_KICKS], c.kicks);
+        count_max(&bc[C_CHAIN_MAX], c.kicks);
+        if (c.ghosts_made) count_add(&bc[C_GHOSTS_MADE], c.ghosts_made);
+        if (c.dup_evict) count_add(&bc[C_DUP_EVICT], c.dup_evict);
         atomicAdd(t.counters + CHAIN_HIST + chain_bucket(c.kicks), 1ull);
       }
       uint64_t bucket = ((load_base + i) * HIST_BUCKETS) / t.total_slots;

@@ -328,7 +328,7 @@ struct BatchKeys {
       if (st == ST_OK) atomicAdd(&bt.chain[chain_bucket(c.kicks)], 1u);
     }
     const KeySums s = sum_keys(over, c, st, aborts);
-    if (lane_id() == 0) add_sums(bt.bc, s);
+    if (lane_id() == 0) add_sums<true>(bt.bc, s);
   }
 };
 

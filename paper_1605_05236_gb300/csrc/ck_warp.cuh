@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(WARP_BLOCK, 8) k_insert_warp(DevTable t, const
     int st = -1;  // the key's final status once known
     bool need = false;
     if (!have) {
-      i = atomicAdd(&s_next, 1ull);
+      i = take_index(&s_next);
       have = i < hi;
       if (have) {
         const uint32_t key = keys[i];
@@ -392,15 +392,15 @@ __global__ void __launch_bounds__(WARP_BLOCK, 8) k_insert_warp(DevTable t, const
       if (st == ST_OK) {
         ok++;
         if (c.kicks) {
-          atomicAdd(&bc[C_KICKS], (unsigned long long)c.kicks);
-          atomicMax(&bc[C_CHAIN_MAX], (unsigned long long)c.kicks);
+          count_add(&bc[C_KICKS], c.kicks);
+          count_max(&bc[C_CHAIN_MAX], c.kicks);
         }
         atomicAdd(&h_chain[chain_bucket(c.kicks)], 1u);
       } else {
-        atomicAdd(&bc[st == ST_FAILED ? C_INS_FAILED : C_INS_ABORTED], 1ull);
+        count_add(&bc[st == ST_FAILED ? C_INS_FAILED : C_INS_ABORTED], 1u);
       }
-      if (aborts) atomicAdd(&bc[C_ABORTS], (unsigned long long)aborts);
-      if (c.reviews) atomicAdd(&bc[C_REVIEWS], (unsigned long long)c.reviews);
+      if (aborts) count_add(&bc[C_ABORTS], aborts);
+      if (c.reviews) count_add(&bc[C_REVIEWS], c.reviews);
       const uint32_t v_final = c.viewed - c.viewed0;
       viewed += v_final;
       viewed_all += c.viewed;
@@ -413,9 +413,9 @@ __global__ void __launch_bounds__(WARP_BLOCK, 8) k_insert_warp(DevTable t, const
       have = false;
     }
   }
-  flush_counter(&bc[C_INS_OK], ok);
-  flush_counter(&bc[C_VIEWED], viewed);
-  flush_counter(&bc[C_VIEWED_ALL], viewed_all);
+  if (ok) count_add(&bc[C_INS_OK], ok);
+  if (viewed) count_add(&bc[C_VIEWED], viewed);
+  if (viewed_all) count_add(&bc[C_VIEWED_ALL], viewed_all);
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int k = 0; k < C_N; k++) {
