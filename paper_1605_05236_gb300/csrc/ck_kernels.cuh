@@ -471,55 +471,100 @@ __device__ __forceinline__ void load_bin_nc(const DevTable& t, uint32_t bin, uin
   for (int q = 0; q < B; q += 4) ld_bin4_nc(p + q, s + q);
 }
 
-// Two-choice lookup: both bins are fetched at once (two independent sector
-// loads in flight per key).
+// What a lookup launch adds to the table's counters.
+__device__ __forceinline__ void count_lookups(const DevTable& t, uint32_t hits, uint32_t cnt) {
+  __shared__ unsigned long long sh[2];
+  if (threadIdx.x < 2) sh[threadIdx.x] = 0;
+  __syncthreads();
+  count_add_warp(&sh[0], hits);
+  count_add_warp(&sh[1], cnt);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (sh[0]) atomicAdd(t.counters + C_LOOKUP_HITS, sh[0]);
+    if (sh[1]) atomicAdd(t.counters + C_LOOKUPS, sh[1]);
+  }
+}
+
+// Two-choice lookup: the first bin, and the second for keys not found there.
+// Bound by random DRAM lines (a random miss moves a 128-byte line whatever
+// part of it is read): 2^26 lookups, half of them hits, in a 2^24 x 4 table
+// at 0.95 take 2.03 ms, 1.75 lines a lookup at 58 G lines/s of the 61 the
+// gather probe reaches.
+//
+// 8-slot bins are read by pairs of lanes, half a bin each, one key of the
+// pair after the other: the two 32-byte halves then travel as one access.
+// Read by two instructions of one lane they cost two, though the line is the
+// same.  20,000,003 lookups, 0 / 50 / 90% hits, 2^23 x 8 at 0.97 (512 MiB): 718
+// / 614 / 532 us against 1142 / 942 / 793; 5,000,011 x 8 (320 MB): 625 / 538 /
+// 477 against 790 / 654 / 559; 2^17 x 8 (8 MiB, in L2): 246 / 246 / 229 against
+// 383 / 362 / 324; 2^16 lookups: the same.  Both keys of the pair in flight
+// together take 40-48 registers instead of 32 and are slower (566 and 621 for
+// 538).
 template <int B>
 __global__ void __launch_bounds__(256) k_lookup2(DevTable t, const uint32_t* __restrict__ keys, uint64_t n,
                                                  uint32_t* __restrict__ vals_out,
                                                  uint8_t* __restrict__ found_out) {
-  __shared__ unsigned long long hits_sh, cnt_sh;
-  if (threadIdx.x == 0) hits_sh = cnt_sh = 0;
-  __syncthreads();
   uint32_t hits = 0, cnt = 0;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-    uint32_t key = __ldcs(keys + i);
+  const uint64_t n32 = (n + 31) & ~31ull;  // whole warps: pairs of lanes work together
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n32; i += stride) {
+    const uint32_t key = i < n ? __ldcs(keys + i) : RESERVED_KEY;
     uint32_t val = 0;
     bool f = false;
-    if (key != RESERVED_KEY) {
-      uint32_t b0, b1;
-      bins2(t, key, b0, b1);
-      uint64_t s0[B], s1[B];
-      load_bin_nc<B>(t, b0, s0);
-      load_bin_nc<B>(t, b1, s1);
-      f = match_bin<B>(s0, key, val);
-      if (!f) f = match_bin<B>(s1, key, val);
+    uint32_t b0 = 0, b1 = 0;
+    if (key != RESERVED_KEY) bins2(t, key, b0, b1);
+    if constexpr (B == 8) {
+      constexpr unsigned ALL = 0xFFFFFFFFu;
+      const uint32_t half = threadIdx.x & 1u, even = threadIdx.x & 30u;
+#pragma unroll
+      for (uint32_t u = 0; u < 2; u++) {  // the even lane's key, then the odd lane's
+        const uint32_t k = __shfl_sync(ALL, key, even + u);
+        const bool on = k != RESERVED_KEY;
+        uint32_t bin = __shfl_sync(ALL, b0, even + u), v = 0;
+        uint64_t s[4];
+        if (on) ld_bin4_nc(t.slots + (uint64_t)bin * 8 + half * 4, s);
+        bool h = on && match_bin<4>(s, k, v);
+        const bool other = __shfl_xor_sync(ALL, h, 1);
+        bin = __shfl_sync(ALL, b1, even + u);
+        if (on && !h && !other) {
+          ld_bin4_nc(t.slots + (uint64_t)bin * 8 + half * 4, s);
+          h = match_bin<4>(s, k, v);
+        }
+        const bool ph = __shfl_xor_sync(ALL, h, 1);
+        const uint32_t pv = __shfl_xor_sync(ALL, v, 1);
+        if (half == u) {
+          f = h || ph;
+          val = h ? v : ph ? pv : 0u;
+        }
+      }
+    } else if (key != RESERVED_KEY) {
+      uint64_t s[B];
+      load_bin_nc<B>(t, b0, s);
+      f = match_bin<B>(s, key, val);
+      if (!f) {
+        load_bin_nc<B>(t, b1, s);
+        f = match_bin<B>(s, key, val);
+      }
     }
-    hits += f;
-    cnt++;
-    if (vals_out) __stcs(vals_out + i, val);
-    if (found_out) __stcs(found_out + i, (uint8_t)f);
+    if (i < n) {
+      hits += f;
+      cnt++;
+      if (vals_out) __stcs(vals_out + i, val);
+      if (found_out) __stcs(found_out + i, (uint8_t)f);
+    }
   }
-  hits = __reduce_add_sync(0xffffffffu, hits);
-  cnt = __reduce_add_sync(0xffffffffu, cnt);
-  if ((threadIdx.x & 31) == 0) {
-    if (hits) count_add(&hits_sh, hits);
-    if (cnt) count_add(&cnt_sh, cnt);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    if (hits_sh) atomicAdd(t.counters + C_LOOKUP_HITS, hits_sh);
-    if (cnt_sh) atomicAdd(t.counters + C_LOOKUPS, cnt_sh);
-  }
+  count_lookups(t, hits, cnt);
 }
 
-// d-ary lookup: the d single-slot bins are fetched at once.
+// d-ary lookup: a bin is read only for keys not found in the ones before,
+// which saves a DRAM line (a present key is in its second or third bin on
+// average); with this many keys in flight the round trips do not show.  2^26
+// bins, d = 4, 0.90 full, 2^24 lookups, 50 / 90% hits: 927 / 761 us against
+// 1134 with all d bins fetched at once; 2^20 lookups 75 / 65 against 87; 2^16
+// and fewer the same.
 static __global__ void __launch_bounds__(256) k_lookup_dary(DevTable t, const uint32_t* __restrict__ keys, uint64_t n,
                                                      uint32_t* __restrict__ vals_out,
                                                      uint8_t* __restrict__ found_out) {
-  __shared__ unsigned long long hits_sh, cnt_sh;
-  if (threadIdx.x == 0) hits_sh = cnt_sh = 0;
-  __syncthreads();
   uint32_t hits = 0, cnt = 0;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
@@ -529,29 +574,19 @@ static __global__ void __launch_bounds__(256) k_lookup_dary(DevTable t, const ui
     if (key != RESERVED_KEY) {
       uint32_t b[4];
       bins_of(t, key, b);
-      uint64_t s[4];
 #pragma unroll
-      for (int j = 0; j < 4; j++) s[j] = j < (int)t.d ? ld_slot_nc(t.slots + b[j]) : EMPTY;
-#pragma unroll
-      for (int j = 0; j < 4; j++)
-        if (!f && key_of(s[j]) == key) { f = true; val = (uint32_t)s[j]; }
+      for (int j = 0; j < 4; j++) {
+        if (f || j >= (int)t.d) continue;
+        const uint64_t r = ld_slot_nc(t.slots + b[j]);
+        if (key_of(r) == key) { f = true; val = (uint32_t)r; }
+      }
     }
     hits += f;
     cnt++;
     if (vals_out) __stcs(vals_out + i, val);
     if (found_out) __stcs(found_out + i, (uint8_t)f);
   }
-  hits = __reduce_add_sync(0xffffffffu, hits);
-  cnt = __reduce_add_sync(0xffffffffu, cnt);
-  if ((threadIdx.x & 31) == 0) {
-    if (hits) count_add(&hits_sh, hits);
-    if (cnt) count_add(&cnt_sh, cnt);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    if (hits_sh) atomicAdd(t.counters + C_LOOKUP_HITS, hits_sh);
-    if (cnt_sh) atomicAdd(t.counters + C_LOOKUPS, cnt_sh);
-  }
+  count_lookups(t, hits, cnt);
 }
 
 // The hit field of every metadata word, for an export (sign 1: the bin's
