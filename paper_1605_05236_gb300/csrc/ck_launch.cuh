@@ -41,9 +41,9 @@ cudaError_t launch_insert(const InsertLaunch& l, const uint32_t* keys, const uin
     return cudaGetLastError();
   }
   const uint32_t block = l.block;
-  // two-choice walks without ghosts run a step per lane (ck_walk.cuh), except
-  // upserts, which first look for the key under claims
-  constexpr bool WALKS = B > 1 && !GHOST && (POL == P_QUEUE || POL == P_RANDOM);
+  // two-choice walks without ghosts and rattle-kicking run a step per lane
+  // (ck_walk.cuh), except upserts, which first look for the key under claims
+  constexpr bool WALKS = B > 1 ? !GHOST && (POL == P_QUEUE || POL == P_RANDOM) : POL == P_RATTLE;
   const bool walk = WALKS && !upsert;
   // persistent launch: at most the blocks that fit on the GPU at once
   static int cached_block[2] = {0, 0}, cached_per_sm[2] = {0, 0};

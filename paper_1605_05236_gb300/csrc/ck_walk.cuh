@@ -46,14 +46,18 @@ struct Walk {
 template <int B, int POL>
 __device__ __forceinline__ int walk_begin(const DevTable& t, Ctx& c, Walk<B>& w) {
   constexpr uint32_t FULL = (1u << B) - 1;
-  uint32_t b0, b1;
-  bins2(t, c.key, b0, b1);
-  View<B> v0, v1;
-  load_view2_fast<B>(t, b0, b1, v0, v1);
   c.held = c.krec;
   w.pend = nullptr;
   w.tries = 0;
   w.s = -1;
+  if constexpr (POL == P_RATTLE) {
+    w.s = 0;
+    return WALK;
+  }
+  uint32_t b0, b1;
+  bins2(t, c.key, b0, b1);
+  View<B> v0, v1;
+  load_view2_fast<B>(t, b0, b1, v0, v1);
   const uint32_t g0 = empty_mask<B>(v0), g1 = empty_mask<B>(v1);
   c.viewed += (POL == P_RANDOM && g0) ? 1 : 2;
   if (g0 | g1) {
@@ -78,12 +82,63 @@ __device__ __forceinline__ int walk_begin(const DevTable& t, Ctx& c, Walk<B>& w)
   return WALK;
 }
 
+// A step of rattle-kicking (insert_rattle, ck_insert.cuh, which the serial
+// replay runs): one try, the record in hand at its bin h_{r mod d}, where
+// w.s is r and c.draws counts the tries.  The bin's view and the re-read of
+// the slot the kick before claimed go out together.
+__device__ __forceinline__ int rattle_step(const DevTable& t, Ctx& c, Walk<1>& w) {
+  if (c.draws == t.cap) return out_of_cap(c);
+  c.draws++;
+  if (int r = plan_room(t, c)) return r;
+  uint32_t vb[4];
+  bins_of(t, key_of(c.held), vb);
+  const uint32_t j = (uint32_t)w.s % t.d;
+  const uint32_t x = j == 0 ? vb[0] : j == 1 ? vb[1] : j == 2 ? vb[2] : vb[3];
+  const uint32_t rc = w.s < 255 ? w.s + 1 : 255;
+  w.s = (int)rc;
+  const uint64_t chk = w.pend ? ld_slot(w.pend) : c.held;
+  View<1> v;
+  load_view_fast<1>(t, x, v);
+  if (chk != c.held) return ST_CONFLICT;
+  w.pend = nullptr;
+  for (int k = 0;; k++) {
+    if (claimed_mask<1>(v)) {
+      // this chain's own bin: skipped, not viewed; another insertion's:
+      // viewed and ignored (Sec. 8)
+      if (k || !plan_has_bin(c, x)) {
+        if (!k) c.viewed++;
+        c.foreign = 1;
+      }
+      return WALK;
+    }
+    if (!k) c.viewed++;
+    const uint32_t ry = rattle_of(v.m);
+    if (v.s[0] == EMPTY) {
+      if (claim(t, c, x, v.m, 0, K_MOVE, false, c.held, ry, rc)) return ST_OK;
+    } else {
+      if (t.tie_resident ? rc <= ry : rc < ry) return WALK;  // the resident stays
+      if (claim(t, c, x, v.m, 0, K_MOVE, false, c.held, ry, rc)) {
+        c.kicks++;
+        c.held = v.s[0];
+        w.s = (int)ry;
+        w.pend = t.slots + x;
+        return WALK;
+      }
+    }
+    if (k == 3) return ST_CONFLICT;
+    load_view_fast<1>(t, x, v);
+    c.viewed++;
+    c.reviews++;
+  }
+}
+
 // One step at w.x: the free slot that ends the chain (ST_OK, and it is
 // written), or one kick -- the claim of the victim, the view of the bin it
 // moves to and the re-read of the slot the kick before claimed, in one round
 // trip -- or another view of the bin after a lost race (WALK).
 template <int B, int POL>
 __device__ __forceinline__ int walk_step(const DevTable& t, Ctx& c, Walk<B>& w) {
+  if constexpr (POL == P_RATTLE) return rattle_step(t, c, w);
   constexpr uint32_t FULL = (1u << B) - 1;
   const uint64_t chk = w.pend ? ld_slot(w.pend) : c.held;
   const uint32_t fm = empty_mask<B>(w.v);
@@ -161,32 +216,42 @@ __device__ __forceinline__ void load_entries(const Ctx& c, int first, int n, ulo
   }
 }
 
-// The chain's last record is in its free slot: the others' writes, last slot
-// first, then the releases (as commit, ck_insert.cuh).  An entry's content is
-// the record its slot receives.
-template <int B>
-__device__ __forceinline__ void walk_commit(const DevTable& t, Ctx& c) {
+// The writes of a chain, last slot first, then the releases (as commit,
+// ck_insert.cuh).  An entry's content is the record its slot receives.  The
+// last record of a two-choice walk is in its free slot already; rattle-kicking
+// claims that slot, because its counter is in the metadata word, and takes it
+// here (false if it was taken meanwhile, with nothing written).
+template <int B, int POL>
+__device__ __forceinline__ bool walk_commit(const DevTable& t, Ctx& c) {
   const int n = c.pn;
-  if (n == 0) return;
+  if (n == 0) return true;
   ulonglong2 e[4];
   for (int first = (n - 1) & ~3; first >= 0; first -= 4) {
     load_entries(c, first, n, e);
 #pragma unroll
     for (int u = 3; u >= 0; u--) {
       if (first + u >= n || e_sup(e[u].x)) continue;  // a later revisit of the slot writes it
+      if (POL == P_RATTLE && first + u == n - 1) {
+        if (!cas_slot(slot_at<B>(t, e[u].x), EMPTY, e[u].y)) return false;
+        continue;
+      }
       if (t.ordered_writes) fence_release();          // the copy lands before its source is overwritten
       st_slot(slot_at<B>(t, e[u].x), e[u].y);
     }
   }
-  fence_release();
+  // nothing moved when a new key took a free slot: no order to keep
+  if (POL != P_RATTLE || n > 1) fence_release();
   for (int first = 0; first < n; first += 4) {
     load_entries(c, first, n, e);
 #pragma unroll
     for (int u = 0; u < 4; u++) {
       if (first + u >= n) continue;
-      red_relaxed(t.meta + e_bin(e[u].x), VER_ONE - (e_rev(e[u].x) ? 0u : 1u << e_slot(e[u].x)));
+      uint32_t delta = VER_ONE - (e_rev(e[u].x) ? 0u : 1u << e_slot(e[u].x));
+      if (B == 1) delta += (e_new_r(e[u].x) - e_old_r(e[u].x)) << RATTLE_SHIFT;
+      red_relaxed(t.meta + e_bin(e[u].x), delta);
     }
   }
+  return true;
 }
 
 // The lanes whose walk ended, or that wait for a key, are served once they
@@ -230,11 +295,14 @@ __device__ __forceinline__ void walk_keys(Src& src, uint64_t* local_e) {
     if (need && __popc(need) >= WAITERS * __popc(walking)) {
       bool over = false;
       if (mode == ENDED) {  // as insert_one ends an attempt
+        bool undone = false;
         if (st == ST_OK) {
-          walk_commit<B>(src.table(), c);
-          over = true;
-        } else {
-          release_all(src.table(), c);
+          over = walk_commit<B, POL>(src.table(), c);
+          if (!over) st = ST_CONFLICT;
+          undone = !over;
+        }
+        if (!over) {
+          release_all(src.table(), c, undone);
           const bool ran_out = st == ST_FAILED || c.capped;
           if (ran_out) {
             over = ++fails > (st == ST_FAILED ? 6u : 32u);
@@ -310,11 +378,25 @@ struct BatchKeys {
   __device__ __forceinline__ const DevTable& table() const { return t; }
   __device__ __forceinline__ bool take(unsigned idle) {
     uint64_t got = hi;
-    more = ls.template take<B, POL>(t, keys, vals, status, viewed_out, hi, load_base, idle, bt, got);
+    if constexpr (B == 1) {  // straight from the block's range: the walk's first tries are its look
+      const uint32_t lane = lane_id();
+      unsigned long long base = 0;
+      if (lane == 0) base = atomicAdd(&ls.next, (unsigned long long)__popc(idle));
+      base = __shfl_sync(0xFFFFFFFFu, base, 0);
+      more = base + __popc(idle) < hi;
+      if ((idle >> lane) & 1u) got = base + __popc(idle & ((1u << lane) - 1));
+    } else {
+      more = ls.template take<B, POL>(t, keys, vals, status, viewed_out, hi, load_base, idle, bt, got);
+    }
     if (got >= hi) return false;
     i = got;
     key = __ldcs(keys + i);
     val = __ldcs(vals + i);
+    if (B == 1 && key == RESERVED_KEY) {
+      if (status) status[i] = ST_INVALID;
+      if (viewed_out) viewed_out[i] = 0;
+      return false;
+    }
     return true;
   }
   __device__ __forceinline__ void done(bool over, const Ctx& c, int st, uint32_t aborts) {
@@ -333,7 +415,7 @@ struct BatchKeys {
 };
 
 template <int B, int POL>
-__global__ void __launch_bounds__(256, 3) k_insert_walk(DevTable t, const uint32_t* __restrict__ keys,
+__global__ void __launch_bounds__(256, B == 1 ? 4 : 3) k_insert_walk(DevTable t, const uint32_t* __restrict__ keys,
                                                         const uint32_t* __restrict__ vals, uint64_t n,
                                                         uint8_t* __restrict__ status,
                                                         uint32_t* __restrict__ viewed_out, uint64_t load_base) {
