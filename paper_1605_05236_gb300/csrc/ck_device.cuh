@@ -101,6 +101,7 @@ struct DevTable {
   uint64_t total_slots;
   uint64_t rng_seed;
   uint32_t bin_mask;             // n_bins - 1 when n_bins is a power of two, else 0
+  uint64_t bin_inv;              // floor((2^64 - 1) / n_bins) + 1 (reduce_bin)
   uint32_t B, d, policy, ghost;
   uint32_t cap, max_retries;
   uint32_t ordered_writes, tie_resident;
@@ -139,9 +140,22 @@ __device__ __forceinline__ uint64_t draw(const DevTable& t, uint32_t key, uint32
   return splitmix64_at(t.rng_seed ^ (uint64_t)key ^ ((uint64_t)i << 32) ^ ((uint64_t)attempt << 48));
 }
 
-__device__ __forceinline__ uint32_t reduce_bin(const DevTable& t, uint32_t h) {
-  return t.bin_mask ? (h & t.bin_mask) : (uint32_t)((uint64_t)h % t.n_bins);
+// A draw below n (1 .. 16), r mod n; n is mostly 4 or 8.
+__device__ __forceinline__ uint32_t below(uint64_t r, uint32_t n) {
+  return (n & (n - 1)) == 0 ? (uint32_t)r & (n - 1) : (uint32_t)(r % n);
 }
+
+// h mod n_bins.  Without a power of two: the fraction h / n_bins in 64 bits
+// (a multiplication by bin_inv), times n_bins (Lemire, Kaser, Kurz, "Faster
+// remainder by direct computation", 2019; exact for 32-bit h and n_bins).
+// Walks hash the record they displace before they can look at its other bin,
+// so a division stood in the chain of every step.
+__device__ __forceinline__ uint32_t reduce_bin(const DevTable& t, uint32_t h) {
+  return t.bin_mask ? (h & t.bin_mask) : (uint32_t)__umul64hi(t.bin_inv * h, t.n_bins);
+}
+
+// The inverse for n bins (2 <= n < 2^32).
+inline uint64_t inverse_of(uint64_t n_bins) { return ~0ull / n_bins + 1; }
 
 __device__ __forceinline__ uint32_t next_bin(const DevTable& t, uint32_t b) {
   return (uint64_t)(b + 1) == t.n_bins ? 0u : b + 1;

@@ -510,7 +510,7 @@ __device__ int insert_random2(const DevTable& t, Ctx& c) {
   uint32_t e1 = FULL & ~claimed_mask<B>(v1) & ~(v1.m >> DUP_SHIFT);
   uint32_t n0 = __popc(e0), ne = n0 + __popc(e1);
   if (ne == 0) return ST_CONFLICT;
-  uint32_t idx = (uint32_t)(draw(t, c.key, c.draws++, c.attempt) % ne);
+  uint32_t idx = below(draw(t, c.key, c.draws++, c.attempt), ne);
   uint32_t x;
   int s;
   View<B> vx;
@@ -562,7 +562,7 @@ __device__ int insert_random2(const DevTable& t, Ctx& c) {
     if (!e) return claims_all_ours<B>(c, x, claimed) ? ST_FAILED : ST_CONFLICT;
     if (int r0 = plan_room(t, c)) return r0;
     uint64_t r = draw(t, c.key, c.draws++, c.attempt);
-    s = nth_bit(e, (uint32_t)(r % __popc(e)));
+    s = nth_bit(e, below(r, __popc(e)));
   }
 }
 
@@ -749,7 +749,7 @@ __device__ inline int insert_random_dary(const DevTable& t, Ctx& c) {
       continue;
     }
     if (nc == 0) return dead_end(c);
-    uint32_t k = (uint32_t)(draw(t, c.key, c.draws++, c.attempt) % nc);
+    uint32_t k = below(draw(t, c.key, c.draws++, c.attempt), nc);
     uint32_t x = cb[k];
     View<1> vx = cv[k];
     if (!counted) c.viewed++;

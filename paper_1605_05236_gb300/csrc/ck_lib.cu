@@ -136,6 +136,7 @@ int init_table(ck_table* t, void* buf, size_t bytes, bool owns, uint64_t bins, u
   dt.total_slots = bins * B;
   dt.rng_seed = seed;
   dt.bin_mask = (bins & (bins - 1)) == 0 ? (uint32_t)(bins - 1) : 0u;
+  dt.bin_inv = inverse_of(bins);
   dt.B = B;
   dt.d = d;
   dt.policy = policy & 0xFF;

@@ -282,6 +282,7 @@ struct TileKeys {
     d.meta = s.meta;
     d.n_bins = s.n_bins;
     d.bin_mask = s.bin_mask;
+    d.bin_inv = s.bin_inv;
     if (POL == P_RANDOM) d.rng_seed = s.rng_seed;
   }
 
@@ -637,6 +638,7 @@ int ck_multi_create_on(ck_multi** out, void* dev_buf, size_t bytes, const ck_mul
     t.total_slots = d.bins * d.slots_per_bin;
     t.rng_seed = seed + i;
     t.bin_mask = (d.bins & (d.bins - 1)) == 0 ? (uint32_t)(d.bins - 1) : 0u;
+    t.bin_inv = inverse_of(d.bins);
     t.B = d.slots_per_bin;
     t.d = 2;
     t.policy = pol;

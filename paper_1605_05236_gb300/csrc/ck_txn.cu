@@ -1125,6 +1125,7 @@ int ck_txn_create(ck_txn_table** out, uint64_t bins, uint32_t slots_per_bin, uin
   t.h.n_bins = bins;
   t.h.total_slots = bins * slots_per_bin;
   t.h.bin_mask = (bins & (bins - 1)) == 0 ? (uint32_t)(bins - 1) : 0u;
+  t.h.bin_inv = inverse_of(bins);
   t.h.d = 2;
   t.h.B = slots_per_bin;
   t.h.hash_family = 0;

@@ -71,7 +71,7 @@ __device__ __forceinline__ int walk_begin(const DevTable& t, Ctx& c, Walk<B>& w)
     const uint32_t e0 = FULL & ~claimed_mask<B>(v0), e1 = FULL & ~claimed_mask<B>(v1);
     const uint32_t n0 = __popc(e0), ne = n0 + __popc(e1);
     if (ne == 0) return ST_CONFLICT;
-    const uint32_t idx = (uint32_t)(draw(t, c.key, c.draws++, c.attempt) % ne);
+    const uint32_t idx = below(draw(t, c.key, c.draws++, c.attempt), ne);
     first = idx < n0;
     w.s = first ? nth_bit(e0, idx) : nth_bit(e1, idx - n0);
   }
@@ -169,7 +169,7 @@ __device__ __forceinline__ int walk_step(const DevTable& t, Ctx& c, Walk<B>& w) 
       if (s < 0) {  // uniform over the slots no chain holds
         const uint32_t e = FULL & ~claimed;
         if (!e) return claims_all_ours<B>(c, w.x, claimed) ? (int)ST_FAILED : (int)ST_CONFLICT;
-        s = nth_bit(e, (uint32_t)(draw(t, c.key, c.draws++, c.attempt) % __popc(e)));
+        s = nth_bit(e, below(draw(t, c.key, c.draws++, c.attempt), __popc(e)));
         w.s = s;
       } else if ((claimed >> s) & 1u) {  // taken while the claim was tried
         return ST_CONFLICT;
