@@ -261,11 +261,15 @@ __device__ __forceinline__ bool unchanged_since(const uint32_t* meta, const uint
   return ok;
 }
 
-__device__ __forceinline__ bool cas_acquire(uint32_t* p, uint32_t expected, uint32_t desired) {
+__device__ __forceinline__ uint32_t cas_acquire_old(uint32_t* p, uint32_t expected, uint32_t desired) {
   uint32_t old;
   asm volatile("atom.acquire.gpu.global.cas.b32 %0, [%1], %2, %3;"
                : "=r"(old) : "l"(p), "r"(expected), "r"(desired) : "memory");
-  return old == expected;
+  return old;
+}
+
+__device__ __forceinline__ bool cas_acquire(uint32_t* p, uint32_t expected, uint32_t desired) {
+  return cas_acquire_old(p, expected, desired) == expected;
 }
 
 __device__ __forceinline__ uint32_t add_release(uint32_t* p, uint32_t delta) {

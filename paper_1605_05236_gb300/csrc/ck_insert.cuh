@@ -468,11 +468,27 @@ __device__ __forceinline__ int take_victim(const DevTable& t, Ctx& c, uint32_t b
   }
 }
 
+// A kick-out walk between two kicks.  Walks and searches are written as a
+// first step and the steps that follow, each ending in a status or in KICKING
+// (more to do), so that the concurrent kernels can have every lane of a warp
+// at a step of its own (ck_walk.cuh).
+constexpr int KICKING = -1;
+
+template <int B>
+struct Kicks {
+  uint32_t x;            // the bin
+  int s;                 // random kicking: the slot to kick
+  View<B> v;             // x as viewed
+  const uint64_t* pend;  // the slot claimed by the last kick, not read again yet (reread), or null
+  uint64_t pend_v;       // the record it must hold
+};
+
 // ------------------------------------------------------------------
 // random kicking, two bins of B slots (Sec. 1; ghosts Sec. 4)
 // ------------------------------------------------------------------
+// The first step: placed (a status), or KICKING with the first victim drawn.
 template <int B, bool GHOST>
-__device__ int insert_random2(const DevTable& t, Ctx& c) {
+__device__ __forceinline__ int random_first(const DevTable& t, Ctx& c, Kicks<B>& k) {
   constexpr uint32_t FULL = (1u << B) - 1;
   uint32_t b0, b1;
   bins2(t, c.key, b0, b1);
@@ -511,59 +527,68 @@ __device__ int insert_random2(const DevTable& t, Ctx& c) {
   uint32_t n0 = __popc(e0), ne = n0 + __popc(e1);
   if (ne == 0) return ST_CONFLICT;
   uint32_t idx = below(draw(t, c.key, c.draws++, c.attempt), ne);
-  uint32_t x;
-  int s;
-  View<B> vx;
-  if (idx < n0) { x = b0; vx = v0; s = nth_bit(e0, idx); }
-  else { x = b1; vx = v1; s = nth_bit(e1, idx - n0); }
-  // One kick a round trip: the victim's claim goes out together with the
-  // view of the bin it moves to (metadata word and slots, unordered) and the
-  // re-read of the slot the previous kick claimed (reread; that claim has
-  // completed), which is compared once the claim is back.
-  const uint64_t* pend = nullptr;
-  uint64_t pend_v = 0;
-  for (;;) {
-    if (c.kicks == t.cap) return ST_FAILED;
-    uint64_t victim = slot_of<B>(vx, s);
-    uint32_t xn = other_bin2(t, victim, x);
-    const uint64_t chk = pend ? ld_slot(pend) : 0;
-    View<B> vn;
+  if (idx < n0) { k.x = b0; k.v = v0; k.s = nth_bit(e0, idx); }
+  else { k.x = b1; k.v = v1; k.s = nth_bit(e1, idx - n0); }
+  k.pend = nullptr;
+  return KICKING;
+}
+
+// One kick a round trip: the victim's claim goes out together with the
+// view of the bin it moves to (metadata word and slots, unordered) and the
+// re-read of the slot the previous kick claimed (reread; that claim has
+// completed), which is compared once the claim is back.
+template <int B, bool GHOST>
+__device__ __forceinline__ int random_kick(const DevTable& t, Ctx& c, Kicks<B>& k) {
+  constexpr uint32_t FULL = (1u << B) - 1;
+  if (c.kicks == t.cap) return ST_FAILED;
+  uint64_t victim = slot_of<B>(k.v, k.s);
+  uint32_t xn = other_bin2(t, victim, k.x);
+  const uint64_t chk = k.pend ? ld_slot(k.pend) : 0;
+  View<B> vn;
+  load_view_fast<B>(t, xn, vn);
+  int st = take_victim<B>(t, c, k.x, k.v, k.s, false);
+  if (st != ST_OK) return st;
+  if (k.pend && chk != k.pend_v) return ST_CONFLICT;
+  if (slot_of<B>(k.v, k.s) != victim) {  // x was viewed again: another record is moving
+    victim = slot_of<B>(k.v, k.s);
+    xn = other_bin2(t, victim, k.x);
     load_view_fast<B>(t, xn, vn);
-    int st = take_victim<B>(t, c, x, vx, s, false);
-    if (st != ST_OK) return st;
-    if (pend && chk != pend_v) return ST_CONFLICT;
-    if (slot_of<B>(vx, s) != victim) {  // x was viewed again: another record is moving
-      victim = slot_of<B>(vx, s);
-      xn = other_bin2(t, victim, x);
-      load_view_fast<B>(t, xn, vn);
-    }
-    c.kicks++;
-    pend = t.slots + (uint64_t)x * B + s;
-    pend_v = victim;
-    x = xn;
-    vx = vn;
-    c.viewed++;
-    uint32_t fm = free_mask<B>(vx);
-    if (fm) {
-      const uint64_t chk_last = ld_slot(pend);
-      const int r = take_free<B>(t, c, x, vx, lowest(fm), false);
-      return (r == ST_OK && chk_last != pend_v) ? (int)ST_CONFLICT : r;
-    }
-    if (GHOST) {
-      uint32_t dm = dup_mask<B>(vx);
-      if (dm) {
-        const uint64_t chk_last = ld_slot(pend);
-        const int r = take_dup<B>(t, c, x, vx, lowest(dm), false);
-        return (r == ST_OK && chk_last != pend_v) ? (int)ST_CONFLICT : r;
-      }
-    }
-    uint32_t claimed = claimed_mask<B>(vx);
-    uint32_t e = FULL & ~claimed & ~(vx.m >> DUP_SHIFT);
-    if (!e) return claims_all_ours<B>(c, x, claimed) ? ST_FAILED : ST_CONFLICT;
-    if (int r0 = plan_room(t, c)) return r0;
-    uint64_t r = draw(t, c.key, c.draws++, c.attempt);
-    s = nth_bit(e, below(r, __popc(e)));
   }
+  c.kicks++;
+  k.pend = t.slots + (uint64_t)k.x * B + k.s;
+  k.pend_v = victim;
+  k.x = xn;
+  k.v = vn;
+  c.viewed++;
+  uint32_t fm = free_mask<B>(k.v);
+  if (fm) {
+    const uint64_t chk_last = ld_slot(k.pend);
+    const int r = take_free<B>(t, c, k.x, k.v, lowest(fm), false);
+    return (r == ST_OK && chk_last != k.pend_v) ? (int)ST_CONFLICT : r;
+  }
+  if (GHOST) {
+    uint32_t dm = dup_mask<B>(k.v);
+    if (dm) {
+      const uint64_t chk_last = ld_slot(k.pend);
+      const int r = take_dup<B>(t, c, k.x, k.v, lowest(dm), false);
+      return (r == ST_OK && chk_last != k.pend_v) ? (int)ST_CONFLICT : r;
+    }
+  }
+  uint32_t claimed = claimed_mask<B>(k.v);
+  uint32_t e = FULL & ~claimed & ~(k.v.m >> DUP_SHIFT);
+  if (!e) return claims_all_ours<B>(c, k.x, claimed) ? ST_FAILED : ST_CONFLICT;
+  if (int r0 = plan_room(t, c)) return r0;
+  uint64_t r = draw(t, c.key, c.draws++, c.attempt);
+  k.s = nth_bit(e, below(r, __popc(e)));
+  return KICKING;
+}
+
+template <int B, bool GHOST>
+__device__ int insert_random2(const DevTable& t, Ctx& c) {
+  Kicks<B> k;
+  int r = random_first<B, GHOST>(t, c, k);
+  while (r == KICKING) r = random_kick<B, GHOST>(t, c, k);
+  return r;
 }
 
 // ------------------------------------------------------------------
@@ -577,9 +602,9 @@ __device__ int insert_random2(const DevTable& t, Ctx& c) {
 // this is slot h mod B); a full bin gives up the record at h mod B, the one
 // that has been there longest -- also when this chain placed it there on an
 // earlier visit -- skipping only slots another insertion holds.
+// The first step: placed (a status), or KICKING at the bin chosen.
 template <int B, bool GHOST>
-__device__ int insert_queue(const DevTable& t, Ctx& c) {
-  constexpr uint32_t FULL = (1u << B) - 1;
+__device__ __forceinline__ int queue_first(const DevTable& t, Ctx& c, Kicks<B>& k) {
   uint32_t b0, b1;
   bins2(t, c.key, b0, b1);
   View<B> v0, v1;
@@ -615,79 +640,89 @@ __device__ int insert_queue(const DevTable& t, Ctx& c) {
     c.ghosts_made++;
     return ST_OK;
   }
-  uint32_t x;
-  View<B> vx;
+  k.pend = nullptr;
   if (f0 > 0 || f1 > 0) {
     bool first = f0 >= f1;
-    x = first ? b0 : b1;
-    vx = first ? v0 : v1;
+    k.x = first ? b0 : b1;
+    k.v = first ? v0 : v1;
   } else if (GHOST && (dup_mask<B>(v0) || dup_mask<B>(v1))) {
     bool first = dup_mask<B>(v0) != 0;
-    x = first ? b0 : b1;
-    vx = first ? v0 : v1;
+    k.x = first ? b0 : b1;
+    k.v = first ? v0 : v1;
   } else {
     bool first = hit_of_full<B>(v0.m) <= hit_of_full<B>(v1.m);
-    x = first ? b0 : b1;
-    vx = first ? v0 : v1;
+    k.x = first ? b0 : b1;
+    k.v = first ? v0 : v1;
   }
-  // One kick a round trip: the claim goes out together with the view of
-  // the next bin (metadata word and slots, unordered) and the re-read of the
-  // slot the previous kick claimed (reread; that claim has completed),
-  // compared once the claim is back.
-  const uint64_t* pend = nullptr;
-  uint64_t pend_v = 0;
-  for (;;) {
-    int tries = 0;
-    for (;;) {  // one step at bin x: free slot, duplicate, or victim from hit mod B
-      uint32_t h = hit_of_full<B>(vx.m) % B;  // used when no slot is free
-      uint32_t fm = free_mask<B>(vx);
-      const uint64_t chk = pend ? ld_slot(pend) : 0;
-      if (fm) {
-        if (claim(t, c, x, vx.m, lowest(fm), K_MOVE, false, EMPTY))
-          return (pend && chk != pend_v) ? (int)ST_CONFLICT : (int)ST_OK;
-      } else if (GHOST && dup_mask<B>(vx)) {
-        const int r = take_dup<B>(t, c, x, vx, first_from<B>(dup_mask<B>(vx), h), true);
-        return (r == ST_OK && pend && chk != pend_v) ? (int)ST_CONFLICT : r;
-      } else {
-        // the victim: the record at slot h mod B, skipping slots another
-        // insertion holds; a slot this chain already wrote is taken again
-        // (the walk came back to the bin; its queue has moved on), with the
-        // record the chain put there
-        uint32_t claimed = claimed_mask<B>(vx);
-        uint32_t own = claimed ? own_slots(c, x) : 0u;
-        uint32_t foreign = claimed & ~own;
-        uint32_t um = FULL & ~foreign & ~((vx.m >> DUP_SHIFT) & ~own);
-        // a detour around another insertion's claim: reaching the cap after
-        // one is not the serial algorithm's failure
-        if (foreign) c.foreign = 1;
-        int s = first_from<B>(um, h);
-        if (s < 0) return dead_end(c);
-        if (c.kicks == t.cap) return out_of_cap(c);
-        if (int r0 = plan_room(t, c)) return r0;
-        const bool rev = (own >> s) & 1u;
-        const int jprev = rev ? last_entry_for(c, x, (uint32_t)s) : -1;
-        const uint64_t victim = rev ? placed_by(c, jprev) : slot_of<B>(vx, s);
-        const uint32_t xn = other_bin2(t, victim, x);
-        View<B> vn;
-        load_view_fast<B>(t, xn, vn);
-        if (rev ? claim_again(t, c, x, vx.m, s, jprev, victim) : claim(t, c, x, vx.m, s, K_MOVE, true, victim)) {
-          if (pend && chk != pend_v) return ST_CONFLICT;
-          c.kicks++;
-          // a slot the chain holds already carries the plan's record: no re-read
-          pend = rev ? nullptr : t.slots + (uint64_t)x * B + s;
-          pend_v = victim;
-          x = xn;
-          vx = vn;
-          break;
-        }
+  return KICKING;
+}
+
+// One kick a round trip: the claim goes out together with the view of the
+// next bin (metadata word and slots, unordered) and the re-read of the slot
+// the previous kick claimed (reread; that claim has completed), compared
+// once the claim is back.
+template <int B, bool GHOST>
+__device__ __forceinline__ int queue_kick(const DevTable& t, Ctx& c, Kicks<B>& k) {
+  constexpr uint32_t FULL = (1u << B) - 1;
+  int tries = 0;
+  for (;;) {  // one step at bin k.x: free slot, duplicate, or victim from hit mod B
+    uint32_t h = hit_of_full<B>(k.v.m) % B;  // used when no slot is free
+    uint32_t fm = free_mask<B>(k.v);
+    const uint64_t chk = k.pend ? ld_slot(k.pend) : 0;
+    if (fm) {
+      if (claim(t, c, k.x, k.v.m, lowest(fm), K_MOVE, false, EMPTY))
+        return (k.pend && chk != k.pend_v) ? (int)ST_CONFLICT : (int)ST_OK;
+    } else if (GHOST && dup_mask<B>(k.v)) {
+      const int r = take_dup<B>(t, c, k.x, k.v, first_from<B>(dup_mask<B>(k.v), h), true);
+      return (r == ST_OK && k.pend && chk != k.pend_v) ? (int)ST_CONFLICT : r;
+    } else {
+      // the victim: the record at slot h mod B, skipping slots another
+      // insertion holds; a slot this chain already wrote is taken again
+      // (the walk came back to the bin; its queue has moved on), with the
+      // record the chain put there
+      uint32_t claimed = claimed_mask<B>(k.v);
+      uint32_t own = claimed ? own_slots(c, k.x) : 0u;
+      uint32_t foreign = claimed & ~own;
+      uint32_t um = FULL & ~foreign & ~((k.v.m >> DUP_SHIFT) & ~own);
+      // a detour around another insertion's claim: reaching the cap after
+      // one is not the serial algorithm's failure
+      if (foreign) c.foreign = 1;
+      int s = first_from<B>(um, h);
+      if (s < 0) return dead_end(c);
+      if (c.kicks == t.cap) return out_of_cap(c);
+      if (int r0 = plan_room(t, c)) return r0;
+      const bool rev = (own >> s) & 1u;
+      const int jprev = rev ? last_entry_for(c, k.x, (uint32_t)s) : -1;
+      const uint64_t victim = rev ? placed_by(c, jprev) : slot_of<B>(k.v, s);
+      const uint32_t xn = other_bin2(t, victim, k.x);
+      View<B> vn;
+      load_view_fast<B>(t, xn, vn);
+      if (rev ? claim_again(t, c, k.x, k.v.m, s, jprev, victim) : claim(t, c, k.x, k.v.m, s, K_MOVE, true, victim)) {
+        if (k.pend && chk != k.pend_v) return ST_CONFLICT;
+        c.kicks++;
+        // a slot the chain holds already carries the plan's record: no re-read
+        k.pend = rev ? nullptr : t.slots + (uint64_t)k.x * B + s;
+        k.pend_v = victim;
+        k.x = xn;
+        k.v = vn;
+        break;
       }
-      if (++tries == 4) return ST_CONFLICT;
-      load_view_fast<B>(t, x, vx);
-      c.viewed++;
-      c.reviews++;
     }
+    if (++tries == 4) return ST_CONFLICT;
+    load_view_fast<B>(t, k.x, k.v);
     c.viewed++;
+    c.reviews++;
   }
+  c.viewed++;
+  return KICKING;
+}
+
+template <int B, bool GHOST>
+__device__ int insert_queue(const DevTable& t, Ctx& c) {
+  Kicks<B> k;
+  int r = queue_first<B, GHOST>(t, c, k);
+  while (r == KICKING) r = queue_kick<B, GHOST>(t, c, k);
+  return r;
 }
 
 // ------------------------------------------------------------------
@@ -697,7 +732,18 @@ __device__ int insert_queue(const DevTable& t, Ctx& c) {
 // Random kicking: view h_0.. in order until an empty bin; when all d are
 // full displace the occupant of a uniformly drawn h_j, which moves to a
 // uniformly drawn bin of its own that the chain has not written, and so on.
-__device__ inline int insert_random_dary(const DevTable& t, Ctx& c) {
+// A d-ary random walk between two kicks: the candidates for the next one.
+struct DaryKicks {
+  uint32_t cb[4], nc;    // bins of the record in hand whose claim flag is clear ...
+  View<1> cv[4];         // ... and their views
+  bool counted;          // the candidates were counted as viewed
+  uint32_t holder;       // the bin whose record is in hand (the last one claimed)
+  const uint64_t* pend;  // the slot claimed by the last kick, not read again yet (reread), or null
+  uint64_t pend_v;       // the record it must hold
+  uint32_t waits;
+};
+
+__device__ __forceinline__ int random_dary_first(const DevTable& t, Ctx& c, DaryKicks& k) {
   uint32_t b[4];
   bins_of(t, c.key, b);
   View<1> v[4];
@@ -715,87 +761,96 @@ __device__ inline int insert_random_dary(const DevTable& t, Ctx& c) {
   // candidates' slots are fetched together; only the drawn one counts as
   // viewed.  A candidate another insertion took meanwhile is dropped and the
   // draw repeated.
-  uint32_t cb[4], nc = 0;
-  View<1> cv[4];
+  k.nc = 0;
   for (uint32_t i = 0; i < t.d; i++) {
-    if (!claimed_mask<1>(v[i])) { cb[nc] = b[i]; cv[nc] = v[i]; nc++; }
+    if (!claimed_mask<1>(v[i])) { k.cb[k.nc] = b[i]; k.cv[k.nc] = v[i]; k.nc++; }
     else c.foreign = 1;  // no claim of ours exists before the first kick
   }
-  bool counted = true;  // the first candidates were counted above
-  uint32_t holder = NO_BIN;  // the bin whose record is in hand (the last one claimed)
-  // One kick a round trip: the displaced record's other bins are viewed
-  // together with its claim, and the slot the previous kick claimed is read
-  // again (reread) in the same round trip.
-  const uint64_t* pend = nullptr;
-  uint64_t pend_v = 0;
+  k.counted = true;  // the first candidates were counted above
+  k.holder = NO_BIN;
+  k.pend = nullptr;
+  k.waits = 0;
+  return KICKING;
+}
+
+// One kick a round trip: the displaced record's other bins are viewed
+// together with its claim, and the slot the previous kick claimed is read
+// again (reread) in the same round trip.
+__device__ __forceinline__ int random_dary_kick(const DevTable& t, Ctx& c, DaryKicks& k) {
   uint32_t vb[4];
   View<1> w[4];
-  for (uint32_t waits = 0;;) {
-    if (nc == 0 && c.foreign && holder != NO_BIN && waits < 8) {
-      // every candidate is held by other insertions, which release their
-      // claims within microseconds: view the candidates again rather than
-      // abandon the whole walk (a bounded wait, so no deadlock)
-      __nanosleep(256u << waits);
-      waits++;
-      bins_of(t, key_of(c.held), vb);
+  if (k.nc == 0 && c.foreign && k.holder != NO_BIN && k.waits < 8) {
+    // every candidate is held by other insertions, which release their
+    // claims within microseconds: view the candidates again rather than
+    // abandon the whole walk (a bounded wait, so no deadlock)
+    __nanosleep(256u << k.waits);
+    k.waits++;
+    bins_of(t, key_of(c.held), vb);
 #pragma unroll
-      for (int i = 0; i < 4; i++)
-        if (i < (int)t.d && vb[i] != holder) load_view_fast<1>(t, vb[i], w[i]);
-      for (uint32_t i = 0; i < t.d; i++) {
-        if (vb[i] == holder) continue;
-        if (!claimed_mask<1>(w[i])) { cb[nc] = vb[i]; cv[nc] = w[i]; nc++; }
-      }
-      c.reviews += nc;
-      continue;
-    }
-    if (nc == 0) return dead_end(c);
-    uint32_t k = below(draw(t, c.key, c.draws++, c.attempt), nc);
-    uint32_t x = cb[k];
-    View<1> vx = cv[k];
-    if (!counted) c.viewed++;
-    bool kicked = false, lost = false;
-    for (int tries = 0; tries < 4 && !kicked && !lost; tries++) {
-      if (tries) {  // lost a race for x: view it again
-        load_view_fast<1>(t, x, vx);
-        c.viewed++;
-        c.reviews++;
-      }
-      if (claimed_mask<1>(vx)) { lost = true; break; }
-      const uint64_t chk = pend ? ld_slot(pend) : 0;
-      if (vx.s[0] == EMPTY) {
-        if (claim(t, c, x, vx.m, 0, K_MOVE, false, EMPTY))
-          return (pend && chk != pend_v) ? (int)ST_CONFLICT : (int)ST_OK;
-        continue;
-      }
-      if (c.kicks == t.cap) return ST_FAILED;
-      if (int r = plan_room(t, c)) return r;
-      bins_of(t, key_of(vx.s[0]), vb);
-#pragma unroll
-      for (int i = 0; i < 4; i++)
-        if (i < (int)t.d && vb[i] != x) load_view_fast<1>(t, vb[i], w[i]);
-      kicked = claim(t, c, x, vx.m, 0, K_MOVE, false, vx.s[0]);
-      if (kicked && pend && chk != pend_v) return ST_CONFLICT;
-    }
-    if (!kicked) {
-      c.foreign = 1;
-      cb[k] = cb[nc - 1];
-      cv[k] = cv[nc - 1];
-      nc--;
-      continue;
-    }
-    c.kicks++;
-    holder = x;
-    c.held = vx.s[0];
-    pend = t.slots + x;
-    pend_v = c.held;
-    nc = 0;
+    for (int i = 0; i < 4; i++)
+      if (i < (int)t.d && vb[i] != k.holder) load_view_fast<1>(t, vb[i], w[i]);
     for (uint32_t i = 0; i < t.d; i++) {
-      if (vb[i] == x) continue;  // just claimed by this chain
-      if (!claimed_mask<1>(w[i])) { cb[nc] = vb[i]; cv[nc] = w[i]; nc++; }
-      else if (!plan_has_bin(c, vb[i])) c.foreign = 1;
+      if (vb[i] == k.holder) continue;
+      if (!claimed_mask<1>(w[i])) { k.cb[k.nc] = vb[i]; k.cv[k.nc] = w[i]; k.nc++; }
     }
-    counted = false;
+    c.reviews += k.nc;
+    return KICKING;
   }
+  if (k.nc == 0) return dead_end(c);
+  uint32_t at = below(draw(t, c.key, c.draws++, c.attempt), k.nc);
+  uint32_t x = k.cb[at];
+  View<1> vx = k.cv[at];
+  if (!k.counted) c.viewed++;
+  bool kicked = false, lost = false;
+  for (int tries = 0; tries < 4 && !kicked && !lost; tries++) {
+    if (tries) {  // lost a race for x: view it again
+      load_view_fast<1>(t, x, vx);
+      c.viewed++;
+      c.reviews++;
+    }
+    if (claimed_mask<1>(vx)) { lost = true; break; }
+    const uint64_t chk = k.pend ? ld_slot(k.pend) : 0;
+    if (vx.s[0] == EMPTY) {
+      if (claim(t, c, x, vx.m, 0, K_MOVE, false, EMPTY))
+        return (k.pend && chk != k.pend_v) ? (int)ST_CONFLICT : (int)ST_OK;
+      continue;
+    }
+    if (c.kicks == t.cap) return ST_FAILED;
+    if (int r = plan_room(t, c)) return r;
+    bins_of(t, key_of(vx.s[0]), vb);
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+      if (i < (int)t.d && vb[i] != x) load_view_fast<1>(t, vb[i], w[i]);
+    kicked = claim(t, c, x, vx.m, 0, K_MOVE, false, vx.s[0]);
+    if (kicked && k.pend && chk != k.pend_v) return ST_CONFLICT;
+  }
+  if (!kicked) {
+    c.foreign = 1;
+    k.cb[at] = k.cb[k.nc - 1];
+    k.cv[at] = k.cv[k.nc - 1];
+    k.nc--;
+    return KICKING;
+  }
+  c.kicks++;
+  k.holder = x;
+  c.held = vx.s[0];
+  k.pend = t.slots + x;
+  k.pend_v = c.held;
+  k.nc = 0;
+  for (uint32_t i = 0; i < t.d; i++) {
+    if (vb[i] == x) continue;  // just claimed by this chain
+    if (!claimed_mask<1>(w[i])) { k.cb[k.nc] = vb[i]; k.cv[k.nc] = w[i]; k.nc++; }
+    else if (!plan_has_bin(c, vb[i])) c.foreign = 1;
+  }
+  k.counted = false;
+  return KICKING;
+}
+
+__device__ inline int insert_random_dary(const DevTable& t, Ctx& c) {
+  DaryKicks k;
+  int r = random_dary_first(t, c, k);
+  while (r == KICKING) r = random_dary_kick(t, c, k);
+  return r;
 }
 
 // Rattle-kicking with rattle balancing (Sec. 7).  r counts the bins a key

@@ -21,30 +21,6 @@ __device__ __forceinline__ int attempt_insert(const DevTable& t, Ctx& c, uint8_t
   }
 }
 
-// A block's search scratch: ceil(blockDim / SLAB) slabs of SLAB consecutive
-// per-thread regions, taken together at block start (all or none: a block
-// never waits while holding a slab, so blocks of overlapping launches cannot
-// hold each other up) and returned at block end.  A block of the next launch
-// may wait for slabs while the previous launch drains; the wait is bounded
-// (about 10 ms), after which the block reports its keys as aborted.
-__device__ __forceinline__ bool acquire_slabs(const DevTable& t, int* out, int need) {
-  const uint32_t n_slabs = t.n_searchers / SLAB;
-  if (n_slabs < (uint32_t)need) return false;
-  for (uint32_t round = 0; round < 4096; round++) {
-    int got = 0;
-    uint32_t start = (blockIdx.x * (uint32_t)need + round * 7919u) % n_slabs;
-    for (uint32_t k = 0; k < n_slabs && got < need; k++) {
-      uint32_t r = start + k;
-      if (r >= n_slabs) r -= n_slabs;
-      if (*(volatile uint32_t*)(t.slab_busy + r) == 0 && atomicCAS(t.slab_busy + r, 0u, 1u) == 0u) out[got++] = (int)r;
-    }
-    if (got == need) return true;
-    for (int j = 0; j < got; j++) atomicExch(t.slab_busy + out[j], 0u);
-    __nanosleep(2000);
-  }
-  return false;
-}
-
 // One insertion with bounded retries after claim conflicts.  A chain that
 // outgrows the local plan continues in a scratch plan.  retry_failed: a
 // random walk that failed in concurrent mode is tried again with new draws
@@ -92,14 +68,8 @@ __device__ __forceinline__ int insert_one(const DevTable& t, Ctx& c, uint8_t* re
         break;
       }
       // a search out of budget tries again in a larger space (search_space)
-      if (region && c.big_id < 0 && (POL == P_BFS || POL == P_SORTED || POL == P_HYBRID)) {
-        c.big_id = acquire_long(t, c.key ^ 0x5bd1e995u);
-        if (c.big_id >= 0) {
-          uint64_t* vis = reinterpret_cast<uint64_t*>(t.long_scratch + (uint64_t)c.big_id * LONG_REGION + SEARCH_HDR +
-                                                      BIG_GROUPS * sizeof(Group));
-          for (int i = 0; i < BIG_VISITED; i++) vis[i] = 0;  // the region held a plan: no stale tags
-        }
-      }
+      if (region && c.big_id < 0 && (POL == P_BFS || POL == P_SORTED || POL == P_HYBRID))
+        c.big_id = take_big_space(t, c.key);
     } else {
       aborts++;
     }
@@ -313,19 +283,12 @@ __global__ void __launch_bounds__(256, insert_blocks_per_sm<B, POL>()) k_insert(
   __shared__ BlockTally bt;
   __shared__ unsigned long long s_next;  // next key of this block's range
   __shared__ int s_slab[SLABS_PER_BLOCK], s_long;
-  // searches on two-choice tables take their keys through a first look
-  // (ck_look.cuh); the other kernels built from this template are for ghosts,
-  // upserts and single-slot bins, whose keys need claims from the start
-  constexpr bool LOOK = B > 1 && !GHOST && !SERIAL && (POL == P_BFS || POL == P_SORTED || POL == P_HYBRID);
-  __shared__ LookMaybe<LOOK> ls;
-  const bool look = LOOK && !upsert;
   bt.clear();
   // each block owns a contiguous range of the batch; its threads pull keys
   // from it one at a time, so a thread held up by a long chain does not
   // hold up the others
   const uint64_t per = (n + gridDim.x - 1) / gridDim.x;
   const uint64_t lo = min(n, (uint64_t)blockIdx.x * per), hi = min(n, lo + per);
-  if constexpr (LOOK) ls.begin(t, lo, load_base);
   if (threadIdx.x == 0) {
     s_next = lo;
     const int need = (int)((blockDim.x + SLAB - 1) / SLAB);
@@ -346,9 +309,7 @@ __global__ void __launch_bounds__(256, insert_blocks_per_sm<B, POL>()) k_insert(
       usable = false;
     }
   }
-  uint8_t* region = s_slab[0] >= 0 ? t.scratch + ((uint64_t)s_slab[threadIdx.x / SLAB] * SLAB + threadIdx.x % SLAB) *
-                                                   SEARCH_REGION
-                                   : nullptr;
+  uint8_t* region = slab_region(t, s_slab);
   if (t.scratch && !region) usable = false;
 
   // per-thread tallies of the counts every key adds to (32-bit: a thread
@@ -395,17 +356,7 @@ __global__ void __launch_bounds__(256, insert_blocks_per_sm<B, POL>()) k_insert(
     bt.key_done(c, st, aborts, v_final, load_bucket(load_base + i, t.total_slots));
   };
   for (;;) {
-    uint64_t i = hi;
-    if constexpr (LOOK) {
-      if (look) {
-        const bool more = ls.template take<B, POL>(t, keys, vals, status, viewed_out, hi, load_base, 0xFFFFFFFFu, bt, i);
-        if (i < hi) insert(i);
-        __syncwarp();
-        if (!more) break;
-        continue;
-      }
-    }
-    i = take_index(&s_next);
+    const uint64_t i = take_index(&s_next);
     if (i >= hi) break;
     insert(i);
   }
@@ -421,10 +372,7 @@ __global__ void __launch_bounds__(256, insert_blocks_per_sm<B, POL>()) k_insert(
   __syncthreads();
   bt.flush(t);
   if (threadIdx.x == 0) {
-    if (s_slab[0] >= 0) {
-      __threadfence();
-      for (int j = 0; j < (int)((blockDim.x + SLAB - 1) / SLAB); j++) atomicExch(t.slab_busy + s_slab[j], 0u);
-    }
+    release_slabs(t, s_slab);
     if (s_long >= 0) release_long(t, s_long);
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");

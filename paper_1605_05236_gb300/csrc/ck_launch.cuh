@@ -41,20 +41,22 @@ cudaError_t launch_insert(const InsertLaunch& l, const uint32_t* keys, const uin
     return cudaGetLastError();
   }
   const uint32_t block = l.block;
-  // two-choice walks without ghosts and rattle-kicking run a step per lane
-  // (ck_walk.cuh), except upserts, which first look for the key under claims
-  constexpr bool WALKS = B > 1 ? !GHOST && (POL == P_QUEUE || POL == P_RANDOM) : POL == P_RATTLE;
-  const bool walk = WALKS && !upsert;
+  // a step per lane (ck_walk.cuh), except upserts, which first look for the
+  // key under claims
+  const bool walk = !upsert;
+  const size_t shared = walk ? walk_shared<B, POL, GHOST>(block) : 0;
+  if (shared) {  // on every launch: the attribute is the current device's
+    const cudaError_t e = cudaFuncSetAttribute(k_insert_walk<B, POL, GHOST>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shared);
+    if (e != cudaSuccess) return e;
+  }
   // persistent launch: at most the blocks that fit on the GPU at once
   static int cached_block[2] = {0, 0}, cached_per_sm[2] = {0, 0};
   if (cached_block[walk] != (int)block) {
     int per_sm = 0;
-    cudaError_t e;
-    if constexpr (WALKS)
-      e = walk ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_insert_walk<B, POL>, block, 0)
-               : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_insert<B, POL, GHOST, false>, block, 0);
-    else
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_insert<B, POL, GHOST, false>, block, 0);
+    const cudaError_t e =
+        walk ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_insert_walk<B, POL, GHOST>, block, shared)
+             : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_insert<B, POL, GHOST, false>, block, 0);
     if (e != cudaSuccess || per_sm < 1) per_sm = 1;
     cached_per_sm[walk] = per_sm;
     cached_block[walk] = (int)block;
@@ -87,15 +89,14 @@ cudaError_t launch_insert(const InsertLaunch& l, const uint32_t* keys, const uin
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = shared;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = l.overlap ? 1 : 0;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if constexpr (WALKS)
-    if (walk) return cudaLaunchKernelEx(&cfg, k_insert_walk<B, POL>, dt, keys, vals, n, st, viewed, load_base);
+  if (walk) return cudaLaunchKernelEx(&cfg, k_insert_walk<B, POL, GHOST>, dt, keys, vals, n, st, viewed, load_base);
   return cudaLaunchKernelEx(&cfg, k_insert<B, POL, GHOST, false>, dt, keys, vals, n, st, viewed, load_base, upsert);
 }
 

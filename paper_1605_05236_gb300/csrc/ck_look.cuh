@@ -277,13 +277,4 @@ struct LookState {
   }
 };
 
-// LookState, or nothing for kernels that take no look.
-struct NoLook {};
-template <bool LOOK>
-struct LookMaybeT { using type = LookState; };
-template <>
-struct LookMaybeT<false> { using type = NoLook; };
-template <bool LOOK>
-using LookMaybe = typename LookMaybeT<LOOK>::type;
-
 }  // namespace ck

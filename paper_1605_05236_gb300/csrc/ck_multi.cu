@@ -410,7 +410,7 @@ __global__ void __launch_bounds__(256, 2) k_multi_walk(DevTable common, const De
   TileKeys<B, POL> src{common, tables, tiles, n_pieces, per_tile, ctr, keys, vals, status, mine, true, 0, 0,
                        0, 0, 0};
   if (lane_id() == 0) src.ahead = atomicAdd(ctr, 1ull);
-  walk_keys<B, POL>(src, store.e);
+  walk_keys<B, POL, false>(src, store.e);
   if (lane_id() == 0)
     for (uint32_t e = 0; e < 4; e++) flush_sums(mine, tables, e);
 }

@@ -255,9 +255,284 @@ __device__ __forceinline__ void bucket_pop(Buckets& bq, const Group* G, uint32_t
   else bq.q[b] = G[g].link;
 }
 
-// ORDER: P_BFS, P_SORTED or P_HYBRID
-template <int B, int ORDER, bool GHOST>
-__device__ int insert_search(const DevTable& t, Ctx& c, uint8_t* region) {
+// ------------------------------------------------------------------
+// two-choice searches
+// ------------------------------------------------------------------
+
+// Groups a search tests bins against one by one before it turns to the hash
+// set, and how many of them the concurrent kernels keep in shared memory.
+constexpr uint32_t LIST_GROUPS = 64;
+constexpr uint32_t NEAR_GROUPS = 12;
+// A thread's share of shared memory: those groups and the bucket queues (an
+// odd number of 16-byte units, so that the threads of a warp meet different
+// banks).
+constexpr uint32_t NEAR_BYTES = NEAR_GROUPS * 16 + 64 * 2 + 16;
+static_assert(NEAR_BYTES / 16 % 2 == 1 && NEAR_BYTES % 16 == 0, "bank-conflict-free stride");
+
+// A search under way.  Most searches view a few tens of bins, and what they
+// touch of their region decides their speed: with every resident thread
+// searching, the lines of the regions in use displace the table's from L2 (a
+// third fewer threads were faster).  So the first groups and the bucket
+// queues are in shared memory (NEAR; the serial replay, upserts and the
+// insertion without allocation keep all of it in the region), and the bins
+// viewed are the groups' own, behind a 128-bit filter in registers that
+// answers most tests; past LIST_GROUPS groups the hash set takes over (also
+// with spawn_k > 1, where bins are viewed that are no group yet).
+template <int B, bool NEAR>
+struct Search {
+  uint8_t* base;           // the region (or big region): header, groups, visited set
+  uint32_t ng;             // groups
+  uint32_t gen;            // the hash set's generation, 0: not in use
+  uint64_t filter[2];      // one bit a marked bin
+  uint32_t mask, depth;    // bucket queues (Buckets)
+  uint32_t cur, bucket;    // the group popped from (~0u: none yet), its bucket
+  uint32_t bin, meta, next;
+
+  static __device__ __forceinline__ uint8_t* near_base() {
+    extern __shared__ uint4 near_mem[];
+    return reinterpret_cast<uint8_t*>(near_mem) + threadIdx.x * NEAR_BYTES;
+  }
+  __device__ __forceinline__ uint32_t* hdr() const { return reinterpret_cast<uint32_t*>(base); }
+  __device__ __forceinline__ Group* groups() const { return reinterpret_cast<Group*>(base + SEARCH_HDR); }
+  __device__ __forceinline__ Group& at(uint32_t g) const {
+    if (NEAR && g < NEAR_GROUPS) return reinterpret_cast<Group*>(near_base())[g];
+    return groups()[g];
+  }
+  // q[b]: head of bucket b, q[32 + b]: its tail
+  __device__ __forceinline__ uint16_t* queues() const {
+    return reinterpret_cast<uint16_t*>(NEAR ? near_base() + NEAR_GROUPS * 16 : reinterpret_cast<uint8_t*>(hdr() + 4));
+  }
+  static __device__ __forceinline__ uint32_t max_groups(const Ctx& c) { return c.big_id >= 0 ? BIG_GROUPS : MAX_GROUPS; }
+  static __device__ __forceinline__ uint32_t vis_bits(const Ctx& c) { return c.big_id >= 0 ? 12 : 10; }
+  static __device__ __forceinline__ uint32_t budget(const DevTable& t, const Ctx& c) {
+    return c.big_id >= 0 ? min(4u * t.cap, (uint32_t)BIG_GROUPS - 8u) : t.cap;
+  }
+  __device__ __forceinline__ uint64_t* vis(const Ctx& c) const {
+    return reinterpret_cast<uint64_t*>(groups() + max_groups(c));
+  }
+
+  static __device__ __forceinline__ uint32_t filter_bit(uint32_t y) { return (y * 0x9E3779B1u) >> 25; }
+  // Was y viewed already?
+  __device__ __forceinline__ bool marked(const Ctx& c, uint32_t y) const {
+    const uint32_t h = filter_bit(y);
+    if (!(((h & 64u ? filter[1] : filter[0]) >> (h & 63u)) & 1u)) return false;
+    if (gen) return vis_has(vis(c), vis_bits(c), gen, y);
+    bool hit = false;
+    for (uint32_t i = 0; i < ng; i++) hit |= at(i).bin == y;
+    return hit;
+  }
+  __device__ __forceinline__ void use_set(const Ctx& c) {
+    gen = next_generation(hdr(), vis(c), vis_bits(c));
+    for (uint32_t i = 0; i < ng; i++) vis_insert(vis(c), vis_bits(c), gen, at(i).bin);
+  }
+  // y is viewed now (it becomes a group unless it ends the search)
+  __device__ __forceinline__ void mark(const Ctx& c, uint32_t y) {
+    const uint32_t h = filter_bit(y);
+    if (h & 64u) filter[1] |= 1ull << (h & 63u);
+    else filter[0] |= 1ull << h;
+    if (!gen && ng >= LIST_GROUPS) use_set(c);
+    if (gen) vis_insert(vis(c), vis_bits(c), gen, y);
+  }
+  template <int ORDER>
+  __device__ __forceinline__ void push(uint32_t bin_, uint32_t m, uint32_t parent) {
+    Group g;
+    g.bin = bin_;
+    g.meta = m;
+    g.parent = (uint16_t)parent;
+    g.link = 0;
+    g.next = 0;
+    const uint32_t d = (ORDER == P_HYBRID && parent != NO_PARENT) ? (at(parent >> 3).key >> 4) + 1u : 0u;
+    g.key = (uint16_t)(d * 16 + spawn_of(m));
+    g.stale = 0;
+    at(ng) = g;
+    if (ORDER != P_BFS) {
+      const uint32_t b = bucket_of(ORDER, g.key);
+      uint16_t* q = queues();
+      if ((mask >> b) & 1u) at(q[32 + b]).link = (uint16_t)ng;
+      else q[b] = (uint16_t)ng;
+      q[32 + b] = (uint16_t)ng;
+      mask |= 1u << b;
+    }
+    ng++;
+  }
+  // Group g becomes the one popped from.
+  __device__ __forceinline__ void take(uint32_t g) {
+    const Group gr = at(g);
+    cur = g;
+    bin = gr.bin;
+    meta = gr.meta;
+    next = gr.next;
+  }
+  // The next candidate, slot s of group `cur`; false: none is left.
+  template <int ORDER>
+  __device__ __forceinline__ bool pop(uint32_t& s) {
+    if (ORDER == P_BFS) {  // the oldest group with a record left
+      if (cur == ~0u || next >= B) {
+        if (cur + 1 == ng) return false;
+        take(cur + 1);
+      }
+      s = next++;
+      return true;
+    }
+    // the smallest key, oldest first among equals
+    Buckets bq;
+    bq.mask = mask;
+    bq.depth = depth;
+    const int bk = bucket_min(ORDER, bq);
+    depth = bq.depth;
+    if (bk < 0) return false;
+    uint16_t* q = queues();
+    if (cur == ~0u || next >= B || bucket != (uint32_t)bk) {
+      if (cur != ~0u && next < B) at(cur).next = (uint8_t)next;
+      bucket = (uint32_t)bk;
+      take(q[bk]);
+    }
+    s = next++;
+    if (next >= B) {  // no record left to spawn
+      if (q[32 + bucket] == (uint16_t)cur) mask &= ~(1u << bucket);
+      else q[bucket] = at(cur).link;
+    }
+    return true;
+  }
+};
+
+// The search for a key whose bins b0, b1 (metadata words m0, m1 as viewed)
+// are full.
+template <int B, int ORDER, bool NEAR>
+__device__ __forceinline__ void search_begin(const DevTable& t, Ctx& c, Search<B, NEAR>& S, uint8_t* region,
+                                             uint32_t b0, uint32_t m0, uint32_t b1, uint32_t m1) {
+  S.base = c.big_id >= 0 ? t.long_scratch + (uint64_t)c.big_id * LONG_REGION : region;
+  S.ng = S.gen = S.mask = S.depth = 0;
+  S.filter[0] = S.filter[1] = 0;
+  S.cur = ~0u;
+  S.next = 0;
+  S.bucket = 0;
+  if (t.spawn_k > 1) S.use_set(c);
+  S.mark(c, b0);
+  S.template push<ORDER>(b0, m0, NO_PARENT);
+  S.mark(c, b1);
+  S.template push<ORDER>(b1, m1, NO_PARENT);
+}
+
+constexpr int SEARCHING = -1;
+
+// One round: up to spawn_k spawns in candidate order, their bins fetched
+// together (Sec. 5: spawning the k best records at a time lets the fetches
+// overlap); the first of them with room ends the search, the others join as
+// groups.  spawn_k = 1 is the plain search: one spawn, whose count goes up
+// while its bin is viewed.  SEARCHING: another round follows.
+template <int B, int ORDER, bool GHOST, bool NEAR>
+__device__ __forceinline__ int search_round(const DevTable& t, Ctx& c, Search<B, NEAR>& S) {
+  uint32_t rg[8], ry[8];
+  uint8_t rs[8];
+  uint32_t nr = 0, g0 = 0, s0 = 0, y0 = 0;
+  View<B> vy;
+  bool out = false;  // budget spent during the round
+  while (nr < t.spawn_k) {
+    uint32_t s;
+    if (!S.template pop<ORDER>(s)) break;
+    if ((S.meta >> s) & 1u) {  // claimed by another insertion: ignore it (Sec. 8)
+      c.foreign = 1;
+      continue;
+    }
+    const uint64_t rec = ld_slot(t.slots + (uint64_t)S.bin * B + s);
+    if (rec == EMPTY) continue;
+    const uint32_t y = other_bin2(t, rec, S.bin), g = S.cur;
+    if (S.marked(c, y)) continue;
+    const bool spent = c.viewed - c.viewed0 >= S.budget(t, c) || S.ng + nr >= S.max_groups(c);
+    // the spawn counts even where the budget ends the search
+    const bool count = ORDER != P_BFS && spawn_of(S.meta) < 15;
+    const uint32_t nm = S.meta + (1u << SPAWN_SHIFT);
+    uint32_t old = S.meta;
+    if (count) old = cas_acquire_old(t.meta + S.bin, S.meta, nm);
+    if (!spent && t.spawn_k == 1) load_view_fast<B>(t, y, vy);
+    if (count) {
+      if (old == S.meta) {
+        S.meta = nm;
+        S.at(g).meta = nm;
+      } else {
+        S.at(g).stale = 1;
+        uint32_t m = ld_acquire(t.meta + S.bin);
+        for (int k = 0; k < 64 && spawn_of(m) < 15; k++) {  // bounded: a lost count is harmless
+          if (cas_acquire(t.meta + S.bin, m, m + (1u << SPAWN_SHIFT))) break;
+          m = ld_acquire(t.meta + S.bin);
+        }
+      }
+    }
+    if (spent) {
+      out = true;
+      break;
+    }
+    S.mark(c, y);
+    c.viewed++;
+    if (nr == 0) {
+      g0 = g;
+      s0 = s;
+      y0 = y;
+    } else {
+      rg[nr] = g;
+      rs[nr] = (uint8_t)s;
+      ry[nr] = y;
+    }
+    if (t.spawn_k > 1) prefetch_bin<B>(t, y);
+    nr++;
+  }
+  if (nr == 0) return dead_end(c);
+  for (uint32_t i = 0; i < nr; i++) {
+    const uint32_t g = i ? rg[i] : g0, s = i ? rs[i] : s0, y = i ? ry[i] : y0;
+    if (t.spawn_k > 1) load_view_fast<B>(t, y, vy);
+    if (claimed_mask<B>(vy)) c.foreign = 1;
+    int term = lowest(free_mask<B>(vy));
+    bool isdup = false;
+    if (term < 0 && GHOST) {
+      term = lowest(dup_mask<B>(vy));
+      isdup = term >= 0;
+    }
+    if (term < 0) {
+      S.template push<ORDER>(y, vy.m, (g << 3) | s);
+      continue;
+    }
+    // path root -> ... -> (g, s): depth entries in chain order
+    uint32_t depth = 1;
+    for (uint32_t q = g; S.at(q).parent != NO_PARENT; q = S.at(q).parent >> 3) depth++;
+    if ((int)depth + 4 > c.pcap) return ST_LONG;
+    {
+      // entries in chain order; the group index rides in the content word
+      // until the slot is claimed
+      uint32_t q = g, qs = s;
+      for (int e = (int)depth - 1; e >= 0; e--) {
+        set_entry(c, e, pack_entry(S.at(q).bin, (int)qs, K_MOVE, false, 0, 0), q);
+        uint32_t par = S.at(q).parent;
+        if (par != NO_PARENT) { qs = par & 7u; q = par >> 3; }
+      }
+    }
+    // claim the path in chain order; each CAS checks its bin is as viewed,
+    // so the record read after the claim is the one the search saw
+    c.pn = 0;
+    for (uint32_t e = 0; e < depth; e++) {
+      Group gq = S.at((uint32_t)content_at(c, (int)e));
+      uint32_t sl = e_slot(desc_at(c, (int)e));
+      if (gq.stale) return ST_CONFLICT;
+      if (!cas_acquire(t.meta + gq.bin, gq.meta, gq.meta + (1u << sl))) return ST_CONFLICT;
+      c.pn = (int)e + 1;
+      // the record must move into the next bin of the path: it is the one
+      // the search saw unless the bin's word came back to its viewed value
+      const uint64_t r = reread<B>(t, gq.bin, sl);
+      const uint32_t to = e + 1 < depth ? S.at((uint32_t)content_at(c, (int)e + 1)).bin : y;
+      set_content(c, (int)e, r);
+      if (!belongs<B>(t, r, to)) return ST_CONFLICT;
+    }
+    c.kicks = depth;
+    if (isdup) return take_dup<B>(t, c, y, vy, term, false);
+    return take_free<B>(t, c, y, vy, term, false);
+  }
+  return out ? out_of_cap(c) : SEARCHING;
+}
+
+// The first step of a search policy's insertion: room in one of the key's
+// bins (or, with ghosts, a duplicate), or SEARCHING with the search begun.
+template <int B, int ORDER, bool GHOST, bool NEAR>
+__device__ __forceinline__ int search_first(const DevTable& t, Ctx& c, Search<B, NEAR>& S, uint8_t* region) {
   uint32_t b0, b1;
   bins2(t, c.key, b0, b1);
   View<B> v0, v1;
@@ -293,144 +568,17 @@ __device__ int insert_search(const DevTable& t, Ctx& c, uint8_t* region) {
     if (f0) return take_free<B>(t, c, b0, v0, lowest(f0), false);
     if (f1) return take_free<B>(t, c, b1, v1, lowest(f1), false);
   }
+  search_begin<B, ORDER, NEAR>(t, c, S, region, b0, v0.m, b1, v1.m);
+  return SEARCHING;
+}
 
-  const SearchSpace sp = search_space(t, c, region);
-  Group* G = sp.G;
-  uint64_t* vis = sp.vis;
-  const uint32_t vb = sp.vis_bits;
-  const uint32_t gen = next_generation(sp.hdr, vis, vb);
-
-  uint32_t ng = 0, head = 0;
-  Buckets bq;
-  bq.q = reinterpret_cast<uint16_t*>(sp.hdr + 4);
-  bq.mask = 0;
-  bq.depth = 0;
-  auto push = [&](uint32_t bin, uint32_t m, uint32_t parent) {
-    Group g;
-    g.bin = bin;
-    g.meta = m;
-    g.parent = (uint16_t)parent;
-    g.link = 0;
-    g.next = 0;
-    uint32_t depth = (ORDER == P_HYBRID && parent != NO_PARENT) ? (G[parent >> 3].key >> 4) + 1u : 0u;
-    g.key = (uint16_t)(depth * 16 + spawn_of(m));
-    g.stale = 0;
-    G[ng] = g;
-    if (ORDER != P_BFS) bucket_push(bq, G, bucket_of(ORDER, g.key), ng);
-    ng++;
-    vis_insert(vis, vb, gen, bin);
-  };
-  push(b0, v0.m, NO_PARENT);
-  push(b1, v1.m, NO_PARENT);
-
-  for (;;) {
-    // one round: up to spawn_k spawns in candidate order, their bins
-    // prefetched together (Sec. 5: spawning the k best records at a time
-    // lets the fetches overlap); the first of them with room ends the
-    // search, the others join as groups.  spawn_k = 1: the plain search.
-    uint32_t rg[8], ry[8];
-    uint8_t rs[8];
-    uint32_t nr = 0;
-    bool out = false;  // budget spent during the round
-    while (nr < t.spawn_k) {
-      uint32_t g;
-      int bk = 0;
-      if (ORDER == P_BFS) {  // the oldest group with a record left
-        while (head < ng && G[head].next >= B) head++;
-        if (head == ng) break;  // nothing left to spawn
-        g = head;
-      } else {  // the smallest key, oldest first among equals
-        bk = bucket_min(ORDER, bq);
-        if (bk < 0) break;
-        g = bq.q[bk];
-      }
-      Group gr = G[g];
-      uint32_t s = gr.next;
-      G[g].next = (uint8_t)(s + 1);
-      if (ORDER != P_BFS && s + 1 >= B) bucket_pop(bq, G, (uint32_t)bk, g);
-      if ((gr.meta >> s) & 1u) {  // claimed by another insertion: ignore it (Sec. 8)
-        c.foreign = 1;
-        continue;
-      }
-      uint64_t rec = ld_slot(t.slots + (uint64_t)gr.bin * B + s);
-      if (rec == EMPTY) continue;
-      uint32_t y = other_bin2(t, rec, gr.bin);
-      if (vis_has(vis, vb, gen, y)) continue;
-      if (ORDER != P_BFS && spawn_of(gr.meta) < 15) {
-        uint32_t nm = gr.meta + (1u << SPAWN_SHIFT);
-        if (cas_acquire(t.meta + gr.bin, gr.meta, nm)) {
-          G[g].meta = nm;
-        } else {
-          G[g].stale = 1;
-          uint32_t m = ld_acquire(t.meta + gr.bin);
-          for (int k = 0; k < 64 && spawn_of(m) < 15; k++) {  // bounded: a lost count is harmless
-            if (cas_acquire(t.meta + gr.bin, m, m + (1u << SPAWN_SHIFT))) break;
-            m = ld_acquire(t.meta + gr.bin);
-          }
-        }
-      }
-      if (c.viewed - c.viewed0 >= sp.budget || ng + nr >= sp.max_groups) { out = true; break; }  // budget spent
-      vis_insert(vis, vb, gen, y);
-      c.viewed++;
-      prefetch_bin<B>(t, y);
-      rg[nr] = g;
-      rs[nr] = (uint8_t)s;
-      ry[nr] = y;
-      nr++;
-    }
-    if (nr == 0) return dead_end(c);
-    for (uint32_t i = 0; i < nr; i++) {
-      const uint32_t g = rg[i], s = rs[i], y = ry[i];
-      View<B> vy;
-      load_view_fast<B>(t, y, vy);
-      if (claimed_mask<B>(vy)) c.foreign = 1;
-      uint32_t fm = free_mask<B>(vy);
-      int term = lowest(fm);
-      bool isdup = false;
-      if (term < 0 && GHOST) {
-        term = lowest(dup_mask<B>(vy));
-        isdup = term >= 0;
-      }
-      if (term < 0) {
-        push(y, vy.m, (g << 3) | s);
-        continue;
-      }
-      // path root -> ... -> (g, s): depth entries in chain order
-      uint32_t depth = 1;
-      for (uint32_t q = g; G[q].parent != NO_PARENT; q = G[q].parent >> 3) depth++;
-      if ((int)depth + 4 > c.pcap) return ST_LONG;
-      {
-        // entries in chain order; the group index rides in the content word
-        // until the slot is claimed
-        uint32_t q = g, qs = s;
-        for (int e = (int)depth - 1; e >= 0; e--) {
-          set_entry(c, e, pack_entry(G[q].bin, (int)qs, K_MOVE, false, 0, 0), q);
-          uint32_t par = G[q].parent;
-          if (par != NO_PARENT) { qs = par & 7u; q = par >> 3; }
-        }
-      }
-      // claim the path in chain order; each CAS checks its bin is as viewed,
-      // so the record read after the claim is the one the search saw
-      c.pn = 0;
-      for (uint32_t e = 0; e < depth; e++) {
-        Group gq = G[(uint32_t)content_at(c, (int)e)];
-        uint32_t sl = e_slot(desc_at(c, (int)e));
-        if (gq.stale) return ST_CONFLICT;
-        if (!cas_acquire(t.meta + gq.bin, gq.meta, gq.meta + (1u << sl))) return ST_CONFLICT;
-        c.pn = (int)e + 1;
-        // the record must move into the next bin of the path: it is the one
-        // the search saw unless the bin's word came back to its viewed value
-        const uint64_t r = reread<B>(t, gq.bin, sl);
-        const uint32_t to = e + 1 < depth ? G[(uint32_t)content_at(c, (int)e + 1)].bin : y;
-        set_content(c, (int)e, r);
-        if (!belongs<B>(t, r, to)) return ST_CONFLICT;
-      }
-      c.kicks = depth;
-      if (isdup) return take_dup<B>(t, c, y, vy, term, false);
-      return take_free<B>(t, c, y, vy, term, false);
-    }
-    if (out) return out_of_cap(c);
-  }
+// ORDER: P_BFS, P_SORTED or P_HYBRID
+template <int B, int ORDER, bool GHOST>
+__device__ int insert_search(const DevTable& t, Ctx& c, uint8_t* region) {
+  Search<B, false> S;
+  int r = search_first<B, ORDER, GHOST, false>(t, c, S, region);
+  while (r == SEARCHING) r = search_round<B, ORDER, GHOST, false>(t, c, S);
+  return r;
 }
 
 // ------------------------------------------------------------------
@@ -444,8 +592,35 @@ __device__ int insert_search(const DevTable& t, Ctx& c, uint8_t* region) {
 // search, full makes it a group.  Same group order, budget and claiming of
 // the path as the two-choice searches above.
 // ------------------------------------------------------------------
+struct DarySearch {
+  SearchSpace sp;
+  uint32_t gen, ng, head;
+  Buckets bq;
+  GroupCache<4> k;  // BFS: the head group's record, its bins and which of them may be tried
+};
+
+// A full bin joins the candidates.
 template <int ORDER>
-__device__ int insert_search_dary(const DevTable& t, Ctx& c, uint8_t* region) {
+__device__ __forceinline__ void push_dary(DarySearch& S, uint32_t bin, uint32_t m, uint32_t parent) {
+  Group* G = S.sp.G;
+  Group g;
+  g.bin = bin;
+  g.meta = m;
+  g.parent = (uint16_t)parent;
+  g.link = 0;
+  g.next = 0;
+  uint32_t depth = (ORDER == P_HYBRID && parent != NO_PARENT) ? (G[parent >> 3].key >> 4) + 1u : 0u;
+  g.key = (uint16_t)(depth * 16 + spawn_of(m));
+  g.stale = 0;
+  G[S.ng] = g;
+  if (ORDER != P_BFS) bucket_push(S.bq, G, bucket_of(ORDER, g.key), S.ng);
+  S.ng++;
+  vis_insert(S.sp.vis, S.sp.vis_bits, S.gen, bin);
+}
+
+// The first step: placed (a status), or SEARCHING with the search begun.
+template <int ORDER>
+__device__ __forceinline__ int search_first_dary(const DevTable& t, Ctx& c, DarySearch& S, uint8_t* region) {
   const uint32_t d = t.d;
   uint32_t b[4];
   bins_of(t, c.key, b);
@@ -458,137 +633,184 @@ __device__ int insert_search_dary(const DevTable& t, Ctx& c, uint8_t* region) {
     if (free_mask<1>(v[i])) return take_free<1>(t, c, b[i], v[i], 0, false);
   }
 
-  const SearchSpace sp = search_space(t, c, region);
-  Group* G = sp.G;
-  uint64_t* vis = sp.vis;
-  const uint32_t vb = sp.vis_bits;
-  const uint32_t gen = next_generation(sp.hdr, vis, vb);
+  S.sp = search_space(t, c, region);
+  S.gen = next_generation(S.sp.hdr, S.sp.vis, S.sp.vis_bits);
+  S.ng = S.head = 0;
+  S.bq.q = reinterpret_cast<uint16_t*>(S.sp.hdr + 4);
+  S.bq.mask = 0;
+  S.bq.depth = 0;
+  for (uint32_t i = 0; i < d; i++) push_dary<ORDER>(S, b[i], v[i].m, NO_PARENT);
+  S.k.g = ~0u;
+  return SEARCHING;
+}
 
-  uint32_t ng = 0, head = 0;
-  Buckets bq;
-  bq.q = reinterpret_cast<uint16_t*>(sp.hdr + 4);
-  bq.mask = 0;
-  bq.depth = 0;
-  auto push = [&](uint32_t bin, uint32_t m, uint32_t parent) {
-    Group g;
-    g.bin = bin;
-    g.meta = m;
-    g.parent = (uint16_t)parent;
-    g.link = 0;
-    g.next = 0;
-    uint32_t depth = (ORDER == P_HYBRID && parent != NO_PARENT) ? (G[parent >> 3].key >> 4) + 1u : 0u;
-    g.key = (uint16_t)(depth * 16 + spawn_of(m));
-    g.stale = 0;
-    G[ng] = g;
-    if (ORDER != P_BFS) bucket_push(bq, G, bucket_of(ORDER, g.key), ng);
-    ng++;
-    vis_insert(vis, vb, gen, bin);
-  };
-  for (uint32_t i = 0; i < d; i++) push(b[i], v[i].m, NO_PARENT);
-
-  GroupCache<4> k;  // BFS: the head group's record, its bins and which of them may be tried
-  k.g = ~0u;
-  for (;;) {
-    // rounds of spawn_k tries, as in the two-choice searches
-    uint32_t rg[8], ry[8];
-    uint32_t nr = 0;
-    bool out = false;
-    while (nr < t.spawn_k) {
-      uint32_t g, j, y;
-      if (ORDER == P_BFS) {  // the oldest group, until its hash functions run out
-        if (k.g == head && k.next >= d) head++;
-        if (head == ng) break;  // nothing left to try
-        if (k.g != head) take_group_dary(t, G, head, vis, vb, gen, k);
-        g = head;
-        j = k.next++;
-        if (k.meta & 1u) {  // claimed by another insertion: ignore it (Sec. 8)
-          c.foreign = 1;
-          continue;
-        }
-        // empty, the record's own bin, or a bin already viewed
-        if (!((k.ok >> j) & 1u)) continue;
-        y = pick<4>(k.y, j);
-        if (spawned_to<4>(k, y)) continue;
-      } else {  // the smallest key, oldest first among equals
-        const int bk = bucket_min(ORDER, bq);
-        if (bk < 0) break;
-        g = bq.q[bk];
-        Group gr = G[g];
-        j = gr.next;
-        G[g].next = (uint8_t)(j + 1);
-        if (j + 1 >= d) bucket_pop(bq, G, (uint32_t)bk, g);
-        if (gr.meta & 1u) {
-          c.foreign = 1;
-          continue;
-        }
-        uint64_t rec = ld_slot(t.slots + gr.bin);
-        if (rec == EMPTY) continue;
-        uint32_t rb[4];
-        bins_of(t, key_of(rec), rb);
-        y = rb[j];
-        if (y == gr.bin || vis_has(vis, vb, gen, y)) continue;
-        if (spawn_of(gr.meta) < 15) {
-          uint32_t nm = gr.meta + (1u << SPAWN_SHIFT);
-          if (cas_acquire(t.meta + gr.bin, gr.meta, nm)) {
-            G[g].meta = nm;
-          } else {
-            G[g].stale = 1;
-            uint32_t m = ld_acquire(t.meta + gr.bin);
-            for (int q = 0; q < 64 && spawn_of(m) < 15; q++) {  // bounded: a lost count is harmless
-              if (cas_acquire(t.meta + gr.bin, m, m + (1u << SPAWN_SHIFT))) break;
-              m = ld_acquire(t.meta + gr.bin);
-            }
+// A round of spawn_k tries, as in the two-choice searches.
+template <int ORDER>
+__device__ __forceinline__ int search_round_dary(const DevTable& t, Ctx& c, DarySearch& S) {
+  const uint32_t d = t.d;
+  Group* G = S.sp.G;
+  uint64_t* vis = S.sp.vis;
+  const uint32_t vb = S.sp.vis_bits, gen = S.gen;
+  uint32_t &ng = S.ng, &head = S.head;
+  Buckets& bq = S.bq;
+  GroupCache<4>& k = S.k;
+  const SearchSpace& sp = S.sp;
+  uint32_t rg[8], ry[8];
+  uint32_t nr = 0;
+  bool out = false;
+  while (nr < t.spawn_k) {
+    uint32_t g, j, y;
+    if (ORDER == P_BFS) {  // the oldest group, until its hash functions run out
+      if (k.g == head && k.next >= d) head++;
+      if (head == ng) break;  // nothing left to try
+      if (k.g != head) take_group_dary(t, G, head, vis, vb, gen, k);
+      g = head;
+      j = k.next++;
+      if (k.meta & 1u) {  // claimed by another insertion: ignore it (Sec. 8)
+        c.foreign = 1;
+        continue;
+      }
+      // empty, the record's own bin, or a bin already viewed
+      if (!((k.ok >> j) & 1u)) continue;
+      y = pick<4>(k.y, j);
+      if (spawned_to<4>(k, y)) continue;
+    } else {  // the smallest key, oldest first among equals
+      const int bk = bucket_min(ORDER, bq);
+      if (bk < 0) break;
+      g = bq.q[bk];
+      Group gr = G[g];
+      j = gr.next;
+      G[g].next = (uint8_t)(j + 1);
+      if (j + 1 >= d) bucket_pop(bq, G, (uint32_t)bk, g);
+      if (gr.meta & 1u) {
+        c.foreign = 1;
+        continue;
+      }
+      uint64_t rec = ld_slot(t.slots + gr.bin);
+      if (rec == EMPTY) continue;
+      uint32_t rb[4];
+      bins_of(t, key_of(rec), rb);
+      y = rb[j];
+      if (y == gr.bin || vis_has(vis, vb, gen, y)) continue;
+      if (spawn_of(gr.meta) < 15) {
+        uint32_t nm = gr.meta + (1u << SPAWN_SHIFT);
+        if (cas_acquire(t.meta + gr.bin, gr.meta, nm)) {
+          G[g].meta = nm;
+        } else {
+          G[g].stale = 1;
+          uint32_t m = ld_acquire(t.meta + gr.bin);
+          for (int q = 0; q < 64 && spawn_of(m) < 15; q++) {  // bounded: a lost count is harmless
+            if (cas_acquire(t.meta + gr.bin, m, m + (1u << SPAWN_SHIFT))) break;
+            m = ld_acquire(t.meta + gr.bin);
           }
         }
       }
-      if (c.viewed - c.viewed0 >= sp.budget || ng + nr >= sp.max_groups) { out = true; break; }  // budget spent
-      vis_insert(vis, vb, gen, y);
-      if (ORDER == P_BFS) k.spawned |= 1u << j;
-      c.viewed++;
-      prefetch_bin<1>(t, y);
-      rg[nr] = g;
-      ry[nr] = y;
-      nr++;
     }
-    if (nr == 0) return dead_end(c);
-    for (uint32_t i = 0; i < nr; i++) {
-      const uint32_t g = rg[i], y = ry[i];
-      View<1> vy;
-      load_view_fast<1>(t, y, vy);
-      if (claimed_mask<1>(vy)) c.foreign = 1;
-      if (!free_mask<1>(vy)) {
-        push(y, vy.m, g << 3);
-        continue;
-      }
-      // path: root group -> ... -> group g, one record each, in chain order
-      uint32_t depth = 1;
-      for (uint32_t q = g; G[q].parent != NO_PARENT; q = G[q].parent >> 3) depth++;
-      if ((int)depth + 4 > c.pcap) return ST_LONG;
-      {
-        uint32_t q = g;
-        for (int e = (int)depth - 1; e >= 0; e--) {
-          set_entry(c, e, pack_entry(G[q].bin, 0, K_MOVE, false, 0, 0), q);
-          if (G[q].parent != NO_PARENT) q = G[q].parent >> 3;
-        }
-      }
-      // claim the path in chain order from the metadata words as viewed; the
-      // record read after a claim is the one the search saw
-      c.pn = 0;
-      for (uint32_t e = 0; e < depth; e++) {
-        Group gq = G[(uint32_t)content_at(c, (int)e)];
-        if (gq.stale) return ST_CONFLICT;
-        if (!cas_acquire(t.meta + gq.bin, gq.meta, gq.meta + 1u)) return ST_CONFLICT;
-        c.pn = (int)e + 1;
-        const uint64_t r = reread<1>(t, gq.bin, 0);
-        const uint32_t to = e + 1 < depth ? G[(uint32_t)content_at(c, (int)e + 1)].bin : y;
-        set_content(c, (int)e, r);
-        if (!belongs<1>(t, r, to)) return ST_CONFLICT;
-      }
-      c.kicks = depth;
-      return take_free<1>(t, c, y, vy, 0, false);
-    }
-    if (out) return out_of_cap(c);
+    if (c.viewed - c.viewed0 >= sp.budget || ng + nr >= sp.max_groups) { out = true; break; }  // budget spent
+    vis_insert(vis, vb, gen, y);
+    if (ORDER == P_BFS) k.spawned |= 1u << j;
+    c.viewed++;
+    prefetch_bin<1>(t, y);
+    rg[nr] = g;
+    ry[nr] = y;
+    nr++;
   }
+  if (nr == 0) return dead_end(c);
+  for (uint32_t i = 0; i < nr; i++) {
+    const uint32_t g = rg[i], y = ry[i];
+    View<1> vy;
+    load_view_fast<1>(t, y, vy);
+    if (claimed_mask<1>(vy)) c.foreign = 1;
+    if (!free_mask<1>(vy)) {
+      push_dary<ORDER>(S, y, vy.m, g << 3);
+      continue;
+    }
+    // path: root group -> ... -> group g, one record each, in chain order
+    uint32_t depth = 1;
+    for (uint32_t q = g; G[q].parent != NO_PARENT; q = G[q].parent >> 3) depth++;
+    if ((int)depth + 4 > c.pcap) return ST_LONG;
+    {
+      uint32_t q = g;
+      for (int e = (int)depth - 1; e >= 0; e--) {
+        set_entry(c, e, pack_entry(G[q].bin, 0, K_MOVE, false, 0, 0), q);
+        if (G[q].parent != NO_PARENT) q = G[q].parent >> 3;
+      }
+    }
+    // claim the path in chain order from the metadata words as viewed; the
+    // record read after a claim is the one the search saw
+    c.pn = 0;
+    for (uint32_t e = 0; e < depth; e++) {
+      Group gq = G[(uint32_t)content_at(c, (int)e)];
+      if (gq.stale) return ST_CONFLICT;
+      if (!cas_acquire(t.meta + gq.bin, gq.meta, gq.meta + 1u)) return ST_CONFLICT;
+      c.pn = (int)e + 1;
+      const uint64_t r = reread<1>(t, gq.bin, 0);
+      const uint32_t to = e + 1 < depth ? G[(uint32_t)content_at(c, (int)e + 1)].bin : y;
+      set_content(c, (int)e, r);
+      if (!belongs<1>(t, r, to)) return ST_CONFLICT;
+    }
+    c.kicks = depth;
+    return take_free<1>(t, c, y, vy, 0, false);
+  }
+  if (out) return out_of_cap(c);
+  return SEARCHING;
+}
+
+template <int ORDER>
+__device__ int insert_search_dary(const DevTable& t, Ctx& c, uint8_t* region) {
+  DarySearch S;
+  int r = search_first_dary<ORDER>(t, c, S, region);
+  while (r == SEARCHING) r = search_round_dary<ORDER>(t, c, S);
+  return r;
+}
+
+
+// A block's search scratch: ceil(blockDim / SLAB) slabs of SLAB consecutive
+// per-thread regions, taken together at block start (all or none: a block
+// never waits while holding a slab, so blocks of overlapping launches cannot
+// hold each other up) and returned at block end.  A block of the next launch
+// may wait for slabs while the previous launch drains; the wait is bounded
+// (about 10 ms), after which the block reports its keys as aborted.
+__device__ __forceinline__ bool acquire_slabs(const DevTable& t, int* out, int need) {
+  const uint32_t n_slabs = t.n_searchers / SLAB;
+  if (n_slabs < (uint32_t)need) return false;
+  for (uint32_t round = 0; round < 4096; round++) {
+    int got = 0;
+    uint32_t start = (blockIdx.x * (uint32_t)need + round * 7919u) % n_slabs;
+    for (uint32_t k = 0; k < n_slabs && got < need; k++) {
+      uint32_t r = start + k;
+      if (r >= n_slabs) r -= n_slabs;
+      if (*(volatile uint32_t*)(t.slab_busy + r) == 0 && atomicCAS(t.slab_busy + r, 0u, 1u) == 0u) out[got++] = (int)r;
+    }
+    if (got == need) return true;
+    for (int j = 0; j < got; j++) atomicExch(t.slab_busy + out[j], 0u);
+    __nanosleep(2000);
+  }
+  return false;
+}
+
+// The calling thread's region in a block's slabs (null if it got none).
+__device__ __forceinline__ uint8_t* slab_region(const DevTable& t, const int* slabs) {
+  if (slabs[0] < 0) return nullptr;
+  return t.scratch + ((uint64_t)slabs[threadIdx.x / SLAB] * SLAB + threadIdx.x % SLAB) * SEARCH_REGION;
+}
+
+// By one thread, after a barrier.
+__device__ __forceinline__ void release_slabs(const DevTable& t, const int* slabs) {
+  if (slabs[0] < 0) return;
+  __threadfence();
+  for (int j = 0; j < (int)((blockDim.x + SLAB - 1) / SLAB); j++) atomicExch(t.slab_busy + slabs[j], 0u);
+}
+
+// A larger search space (search_space) for the retries of a key, or -1.
+__device__ __forceinline__ int take_big_space(const DevTable& t, uint32_t key) {
+  const int id = acquire_long(t, key ^ 0x5bd1e995u);
+  if (id >= 0) {
+    uint64_t* vis = reinterpret_cast<uint64_t*>(t.long_scratch + (uint64_t)id * LONG_REGION + SEARCH_HDR +
+                                                BIG_GROUPS * sizeof(Group));
+    for (int i = 0; i < BIG_VISITED; i++) vis[i] = 0;  // the region held a plan: no stale tags
+  }
+  return id;
 }
 
 }  // namespace ck

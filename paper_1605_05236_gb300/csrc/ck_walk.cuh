@@ -30,6 +30,15 @@
 namespace ck {
 
 constexpr int WALK = -1;  // the walk goes on
+static_assert(WALK == SEARCHING && WALK == KICKING, "every unfinished insertion says so alike");
+
+template <bool C, class X, class Y>
+struct Choose { using type = X; };
+template <class X, class Y>
+struct Choose<false, X, Y> { using type = Y; };
+
+template <int POL>
+constexpr bool is_search_policy = POL == P_BFS || POL == P_SORTED || POL == P_HYBRID;
 
 // A walk at a bin it has viewed, with the record c.held in hand.
 template <int B>
@@ -267,7 +276,64 @@ __device__ __forceinline__ bool walk_commit(const DevTable& t, Ctx& c) {
 // room for the next launch's (6.43 against 6.46 with every block waiting).
 constexpr int WAITERS = 2;
 
-// Insert the keys of `src`, by a whole warp.  `src` gives each lane its keys
+// Searches that keep their first groups in shared memory (Search).  Measured,
+// 4,194,304 x 4 to 0.95 / 1,500,007 x 8 to 0.97, against all of it in the
+// region: sorted search 5.14 / 3.24 ms against 5.46 / 3.44, the hybrid 6.38 /
+// 3.19 against 6.71 / 3.42; but BFS 6.24 / 3.15 against 6.02 / 3.16, and with
+// ghosts sorted search 6.43 against 5.98 (4 slots), BFS 4.86 against 4.70 (8
+// slots).  8 or 20 groups instead of 12 are slower.
+template <int B, int POL, bool GHOST>
+constexpr bool search_near = B > 1 && !GHOST && (POL == P_SORTED || POL == P_HYBRID);
+
+// What a lane keeps of its insertion between two steps, and the steps: the
+// walks above for two-choice tables without ghosts and for rattle-kicking,
+// else the steps that the serial replay runs (ck_insert.cuh, ck_search.cuh).
+template <int B, int POL, bool GHOST>
+struct Lane {
+  static constexpr bool SEARCH = is_search_policy<POL>;
+  static constexpr bool NEAR = search_near<B, POL, GHOST>;
+  static constexpr bool OWN = POL == P_RATTLE || (B > 1 && !GHOST && !SEARCH);
+  using Dary = typename Choose<SEARCH, DarySearch, DaryKicks>::type;
+  using Two = typename Choose<SEARCH, Search<B, NEAR>, Kicks<B>>::type;
+  using Rest = typename Choose<B == 1, Dary, Two>::type;
+  using State = typename Choose<OWN, Walk<B>, Rest>::type;
+
+  static __device__ __forceinline__ int begin(const DevTable& t, Ctx& c, State& w, uint8_t* region) {
+    if constexpr (SEARCH) {
+      if (!region) return ST_ABORTED;
+      if constexpr (B == 1) return search_first_dary<POL>(t, c, w, region);
+      else return search_first<B, POL, GHOST, NEAR>(t, c, w, region);
+    } else if constexpr (OWN) {
+      return walk_begin<B, POL>(t, c, w);
+    } else if constexpr (B == 1) {
+      return random_dary_first(t, c, w);
+    } else if constexpr (POL == P_QUEUE) {
+      return queue_first<B, GHOST>(t, c, w);
+    } else {
+      return random_first<B, GHOST>(t, c, w);
+    }
+  }
+  static __device__ __forceinline__ int step(const DevTable& t, Ctx& c, State& w) {
+    if constexpr (SEARCH) {
+      if constexpr (B == 1) return search_round_dary<POL>(t, c, w);
+      else return search_round<B, POL, GHOST, NEAR>(t, c, w);
+    } else if constexpr (OWN) {
+      return walk_step<B, POL>(t, c, w);
+    } else if constexpr (B == 1) {
+      return random_dary_kick(t, c, w);
+    } else if constexpr (POL == P_QUEUE) {
+      return queue_kick<B, GHOST>(t, c, w);
+    } else {
+      return random_kick<B, GHOST>(t, c, w);
+    }
+  }
+  static __device__ __forceinline__ bool finish(const DevTable& t, Ctx& c) {
+    if constexpr (OWN) return walk_commit<B, POL>(t, c);
+    else return commit<B>(t, c);
+  }
+};
+
+// Insert the keys of `src`, by a whole warp; region: the lane's search region.  `src` gives each lane its keys
 // and the table they go into, and counts what became of them:
 //   more            keys may be left (the same in all lanes)
 //   take(idle)      the whole warp calls; true in a lane of `idle` that got a
@@ -275,8 +341,10 @@ constexpr int WAITERS = 2;
 //   table()         the lane's table
 //   done(over, c, st, aborts)   the whole warp calls: the ends of the keys of
 //                   the lanes with `over`
-template <int B, int POL, class Src>
-__device__ __forceinline__ void walk_keys(Src& src, uint64_t* local_e) {
+template <int B, int POL, bool GHOST, class Src>
+__device__ __forceinline__ void walk_keys(Src& src, uint64_t* local_e, uint8_t* region = nullptr) {
+  using L = Lane<B, POL, GHOST>;
+  constexpr bool SEARCH = L::SEARCH;
   // a lane has no key; has one whose next attempt begins; walks; has an
   // attempt that ended with st; waits before its next attempt
   enum Mode { IDLE, READY, WALKING, ENDED, WAITING };
@@ -284,7 +352,7 @@ __device__ __forceinline__ void walk_keys(Src& src, uint64_t* local_e) {
   Ctx c;
   c.ghosts_made = c.dup_evict = 0;
   c.kicks = c.viewed = c.viewed0 = c.reviews = 0;
-  Walk<B> w;
+  typename L::State w;
   uint32_t fails = 0, aborts = 0, wake = 0;
   for (;;) {
     if (mode == WAITING && (int)((uint32_t)clock() - wake) >= 0) mode = READY;
@@ -297,30 +365,40 @@ __device__ __forceinline__ void walk_keys(Src& src, uint64_t* local_e) {
       if (mode == ENDED) {  // as insert_one ends an attempt
         bool undone = false;
         if (st == ST_OK) {
-          over = walk_commit<B, POL>(src.table(), c);
+          over = L::finish(src.table(), c);
           if (!over) st = ST_CONFLICT;
           undone = !over;
         }
         if (!over) {
           release_all(src.table(), c, undone);
           const bool ran_out = st == ST_FAILED || c.capped;
-          if (ran_out) {
+          const bool longer = SEARCH && st == ST_LONG;  // the path goes on in a scratch plan
+          if (longer) {
+            over = c.long_id >= 0 || !grow_plan(src.table(), c);
+            if (over) st = c.long_id >= 0 ? ST_FAILED : ST_ABORTED;
+            else mode = READY;
+          } else if (SEARCH && st == ST_ABORTED) {  // no search region
+            over = true;
+          } else if (ran_out) {
             over = ++fails > (st == ST_FAILED ? 6u : 32u);
             if (over) st = ST_FAILED;
+            // a search out of budget tries again in a larger space
+            if (SEARCH && !over && c.big_id < 0) c.big_id = take_big_space(src.table(), c.key);
           } else {
             aborts++;
           }
-          if (!over && ++c.attempt >= src.table().max_retries) {
+          if (!over && !longer && ++c.attempt >= src.table().max_retries) {
             st = ST_ABORTED;
             over = true;
           }
-          if (!over) {
+          if (!over && !longer) {
             wake = (uint32_t)clock() + 2 * backoff_ns(ran_out ? 6 + 2 * fails : c.attempt, c.key);
             mode = WAITING;
           }
         }
       }
       if (over && c.long_id >= 0) release_long(src.table(), c.long_id);
+      if (SEARCH && over && c.big_id >= 0) release_long(src.table(), c.big_id);
       if (__any_sync(0xFFFFFFFFu, over)) src.done(over, c, st, aborts);
       if (over) mode = IDLE;
       // keys for the idle lanes
@@ -332,6 +410,7 @@ __device__ __forceinline__ void walk_keys(Src& src, uint64_t* local_e) {
         c.viewed = 0;
         c.reviews = 0;
         c.long_id = -1;
+        c.big_id = -1;
         fails = 0;
         aborts = 0;
         mode = READY;
@@ -342,17 +421,19 @@ __device__ __forceinline__ void walk_keys(Src& src, uint64_t* local_e) {
         c.viewed0 = c.viewed;
         c.foreign = 0;
         c.capped = 0;
+        c.ghosts_made = 0;
+        c.dup_evict = 0;
         if (c.long_id < 0) {
           c.pe = local_e;
           c.pcap = MAX_CHAIN;
         }
         c.pn = 0;
-        st = walk_begin<B, POL>(src.table(), c, w);
+        st = L::begin(src.table(), c, w, region);
         mode = st == WALK ? WALKING : ENDED;
       }
     }
     if (mode == WALKING) {
-      st = walk_step<B, POL>(src.table(), c, w);
+      st = L::step(src.table(), c, w);
       if (st != WALK) mode = ENDED;
     } else if (!walking && !need) {
       __nanosleep(100);
@@ -362,7 +443,7 @@ __device__ __forceinline__ void walk_keys(Src& src, uint64_t* local_e) {
 }
 
 // The keys lo .. hi - 1 of a batch, into one table.
-template <int B, int POL>
+template <int B, int POL, bool LOOK>
 struct BatchKeys {
   const DevTable& t;
   const uint32_t *keys, *vals;
@@ -378,7 +459,7 @@ struct BatchKeys {
   __device__ __forceinline__ const DevTable& table() const { return t; }
   __device__ __forceinline__ bool take(unsigned idle) {
     uint64_t got = hi;
-    if constexpr (B == 1) {  // straight from the block's range: the walk's first tries are its look
+    if constexpr (!LOOK) {  // straight from the block's range
       const uint32_t lane = lane_id();
       unsigned long long base = 0;
       if (lane == 0) base = atomicAdd(&ls.next, (unsigned long long)__popc(idle));
@@ -392,7 +473,7 @@ struct BatchKeys {
     i = got;
     key = __ldcs(keys + i);
     val = __ldcs(vals + i);
-    if (B == 1 && key == RESERVED_KEY) {
+    if (!LOOK && key == RESERVED_KEY) {
       if (status) status[i] = ST_INVALID;
       if (viewed_out) viewed_out[i] = 0;
       return false;
@@ -411,11 +492,25 @@ struct BatchKeys {
     }
     const KeySums s = sum_keys(over, c, st, aborts);
     if (lane_id() == 0) add_sums<true>(bt.bc, s);
+    if (over && st == ST_OK) {
+      if (c.ghosts_made) count_add(&bt.bc[C_GHOSTS_MADE], c.ghosts_made);
+      if (c.dup_evict) count_add(&bt.bc[C_DUP_EVICT], c.dup_evict);
+    }
   }
 };
 
-template <int B, int POL>
-__global__ void __launch_bounds__(256, B == 1 ? 4 : 3) k_insert_walk(DevTable t, const uint32_t* __restrict__ keys,
+// Blocks of 256 threads on an SM.  Fewer searches at a time leave more of L2
+// to the table: 8-slot sorted search 3.44 ms with 2 blocks, 3.54 with 3.
+template <int B, int POL, bool GHOST>
+constexpr int walk_blocks_per_sm =
+    B == 1 ? 4 : is_search_policy<POL> && (B == 8 || search_near<B, POL, GHOST>) ? 2 : 3;
+
+// dynamic shared memory of a block
+template <int B, int POL, bool GHOST>
+constexpr size_t walk_shared(uint32_t block) { return search_near<B, POL, GHOST> ? (size_t)block * NEAR_BYTES : 0; }
+
+template <int B, int POL, bool GHOST>
+__global__ void __launch_bounds__(256, walk_blocks_per_sm<B, POL, GHOST>) k_insert_walk(DevTable t, const uint32_t* __restrict__ keys,
                                                         const uint32_t* __restrict__ vals, uint64_t n,
                                                         uint8_t* __restrict__ status,
                                                         uint32_t* __restrict__ viewed_out, uint64_t load_base) {
@@ -424,14 +519,18 @@ __global__ void __launch_bounds__(256, B == 1 ? 4 : 3) k_insert_walk(DevTable t,
   __shared__ LookState ls;
   const uint64_t per = (n + gridDim.x - 1) / gridDim.x;
   const uint64_t lo = min(n, (uint64_t)blockIdx.x * per), hi = min(n, lo + per);
+  constexpr bool SEARCH = is_search_policy<POL>;
+  __shared__ int s_slab[SEARCH ? SLABS_PER_BLOCK : 1];
   bt.clear();
   ls.begin(t, lo, load_base);
+  if (SEARCH && threadIdx.x == 0 && !acquire_slabs(t, s_slab, (int)((blockDim.x + SLAB - 1) / SLAB))) s_slab[0] = -1;
   __syncthreads();
   PlanStore<MAX_CHAIN> store;
-  BatchKeys<B, POL> src{t, keys, vals, status, viewed_out, hi, load_base, bt, ls, true, 0, 0, 0};
-  walk_keys<B, POL>(src, store.e);
+  BatchKeys<B, POL, (B > 1 && !GHOST)> src{t, keys, vals, status, viewed_out, hi, load_base, bt, ls, true, 0, 0, 0};
+  walk_keys<B, POL, GHOST>(src, store.e, SEARCH ? slab_region(t, s_slab) : nullptr);
   __syncthreads();
   bt.flush(t);
+  if (SEARCH && threadIdx.x == 0) release_slabs(t, s_slab);
   if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");  // see WAITERS
 }
 
