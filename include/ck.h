@@ -87,7 +87,8 @@ extern "C" {
 #define CK_PARAM_MAX_INFLIGHT 35 /* insertions one insert launch keeps in flight at most
                                     (0, the default: as many threads as fit on the GPU --
                                     nine tenths of that for random kicking and queue-kicking,
-                                    eight tenths for rattle-kicking, when launches overlap,
+                                    eight tenths for rattle-kicking, seven tenths for the
+                                    searches, when launches overlap,
                                     so that the next launch starts beside this one's longest
                                     walks; else
                                     whole blocks, one at least).  Claim conflicts grow with the

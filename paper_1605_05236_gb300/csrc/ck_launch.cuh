@@ -63,18 +63,19 @@ cudaError_t launch_insert(const InsertLaunch& l, const uint32_t* keys, const uin
   }
   uint64_t grid = (n + block - 1) / block;
   uint64_t resident = (uint64_t)cached_per_sm[walk] * l.sm_count;
-  // Walks whose launches overlap leave part of the GPU to the next launch:
-  // its blocks start while this launch's longest walks finish.  Measured
-  // (whole fills, one GB300): two-choice queue-kicking 10.18 ms against
-  // 10.45-10.50 with every block resident (2^24 x 4 to 0.95) and 12.4
-  // against 14.1-14.3 (2^23 x 8 to 0.99), random kicking 22.8 against 24.5
-  // and 34.4 against 38.3; 3-ary random kicking 204.5 against 207.9 (2^26
-  // bins to 0.90); rattle-kicking keeps 0.8 of the blocks, 51.6 against
-  // 58.4 (4-ary to 0.96).  Searches, which need every thread they can get,
-  // are slower that way (BFS 22.5 against 20.8) and keep the full grid.  A
-  // limit the caller sets (CK_PARAM_MAX_INFLIGHT) replaces this one.
-  constexpr uint64_t tenths = (POL == P_QUEUE || POL == P_RANDOM) ? 9 : POL == P_RATTLE ? 8 : 10;
-  if (tenths < 10 && l.overlap && l.max_threads == ~0ull) {
+  // A launch that may overlap the next leaves part of the GPU to it: its
+  // blocks start while this launch's longest walks finish.  Walks keep 0.9 of
+  // the resident blocks, rattle-kicking 0.8, measured when a warp still waited
+  // for its longest walk (queue-kicking 10.18 ms against 10.45-10.50 with
+  // every block, rattle-kicking 51.6 against 58.4); now the share hardly
+  // shows (4- and 8-slot queue-kicking 6.41 / 0.84 ms against 6.39 / 0.87,
+  // rattle-kicking 6.80 against 6.76).  Searches keep 0.7, which leaves L2 to
+  // the table too: 2^22 x 4 to 0.95, sorted search 4.60 ms against 4.81 with
+  // every block and 4.75 with 0.9, BFS 5.42 against 5.74 and 5.48, d = 4 sorted
+  // search 6.32 against 6.56 and 6.47.  A limit the caller sets
+  // (CK_PARAM_MAX_INFLIGHT) replaces this one.
+  constexpr uint64_t tenths = (POL == P_QUEUE || POL == P_RANDOM) ? 9 : POL == P_RATTLE ? 8 : 7;
+  if (l.overlap && l.max_threads == ~0ull) {
     const uint64_t most = resident * tenths / 10;
     resident = most > 0 ? most : 1;
   }

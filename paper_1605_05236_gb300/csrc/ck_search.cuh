@@ -789,6 +789,38 @@ __device__ __forceinline__ bool acquire_slabs(const DevTable& t, int* out, int n
   return false;
 }
 
+// The same by a whole warp, 32 flags at a time from a place of the block's
+// own: the slabs of the launch before are still taken when a launch starts
+// beside it, and one thread looking at them one by one took a round trip for
+// each.  2^22 x 4 to 0.95: sorted search 4.84 ms against 5.15, BFS 5.59 against
+// 6.07; d = 4 sorted search, 2^23 bins to 0.9: 6.61 against 7.59.
+__device__ __forceinline__ bool acquire_slabs_warp(const DevTable& t, int* out, int need) {
+  const uint32_t n = t.n_searchers / SLAB, lane = threadIdx.x & 31u;
+  if (n < (uint32_t)need) return false;
+  const uint32_t start = __shfl_sync(0xFFFFFFFFu, fmix32(blockIdx.x ^ fmix32((uint32_t)clock())), 0) % n;
+  for (uint32_t round = 0; round < 4096; round++) {
+    int got = 0;
+    for (uint32_t k = 0; k < n && got < need; k += 32) {
+      uint32_t r = start + k + lane;
+      if (r >= n) r -= n;
+      const bool free = k + lane < n && *(volatile uint32_t*)(t.slab_busy + r) == 0;
+      const unsigned m = __ballot_sync(0xFFFFFFFFu, free);
+      const bool mine = free && (int)__popc(m & ((1u << lane) - 1)) < need - got &&
+                        atomicCAS(t.slab_busy + r, 0u, 1u) == 0u;
+      const unsigned g = __ballot_sync(0xFFFFFFFFu, mine);
+      if (mine) out[got + __popc(g & ((1u << lane) - 1))] = (int)r;
+      got += __popc(g);
+    }
+    __syncwarp();
+    if (got == need) return true;
+    if (lane == 0)
+      for (int j = 0; j < got; j++) atomicExch(t.slab_busy + out[j], 0u);
+    __syncwarp();
+    __nanosleep(2000);
+  }
+  return false;
+}
+
 // The calling thread's region in a block's slabs (null if it got none).
 __device__ __forceinline__ uint8_t* slab_region(const DevTable& t, const int* slabs) {
   if (slabs[0] < 0) return nullptr;

@@ -523,7 +523,10 @@ __global__ void __launch_bounds__(256, walk_blocks_per_sm<B, POL, GHOST>) k_inse
   __shared__ int s_slab[SEARCH ? SLABS_PER_BLOCK : 1];
   bt.clear();
   ls.begin(t, lo, load_base);
-  if (SEARCH && threadIdx.x == 0 && !acquire_slabs(t, s_slab, (int)((blockDim.x + SLAB - 1) / SLAB))) s_slab[0] = -1;
+  if (SEARCH && threadIdx.x < 32) {
+    const bool got = acquire_slabs_warp(t, s_slab, (int)((blockDim.x + SLAB - 1) / SLAB));
+    if (!got && threadIdx.x == 0) s_slab[0] = -1;
+  }
   __syncthreads();
   PlanStore<MAX_CHAIN> store;
   BatchKeys<B, POL, (B > 1 && !GHOST)> src{t, keys, vals, status, viewed_out, hi, load_base, bt, ls, true, 0, 0, 0};
