@@ -564,7 +564,7 @@ def multi_form(torch, ck, stream):
 # its 61 launches) from an ncu capture of the current kernel build: a
 # half-size fill (2^23 x 4, the same 61-launch load trajectory, half the keys
 # per launch), scaled by 2; None until captured for this build
-INSERT_TRAFFIC_PER_LAUNCH = 382_100_000
+INSERT_TRAFFIC_PER_LAUNCH = 328_800_000
 
 SERVE_BINS = 1 << 26
 SERVE_PREFILL = 255013683  # floor(0.95 * 2^28)
@@ -948,7 +948,7 @@ def run_gpu(args, rank, world, local):
     # random 32-B reads over a buffer the size of the slots, best launch shape
     g32, g32_shape, g32_sweep = gather_roofline(torch, ck, BINS * B * 8, 32, 1 << 26, stream)
     profile = batch_profile(torch, ck, table, kt, vt, st, stream)
-    roofline = {"kernel": "k_insert<4,QUEUE> (one launch per 2^20-key batch)", "bound": "hbm",
+    roofline = {"kernel": "k_insert_walk<4,QUEUE> (one launch per 2^20-key batch)", "bound": "hbm",
                 "achieved": round(achieved, 1), "peak": hbm, "unit": "GB/s",
                 "frac": round(achieved / hbm, 4), "peak_kind": peak_kind + " (MEASURED_PEAKS.json hbm_gbs)",
                 "traffic": INSERT_TRAFFIC_PER_LAUNCH,
@@ -958,18 +958,18 @@ def run_gpu(args, rank, world, local):
     gather_section = {"buffer": "512 MiB (the slot array's size)", "width_bytes": 32, "reads": 1 << 26,
                       "best_gbs": round(g32, 1), "best_shape": g32_shape, "sweep": g32_sweep}
     # the random-operation model of a low-load launch: a key reads its two
-    # bins' 32-B slot sectors, writes one slot by a 64-bit compare-and-swap
-    # and updates its bin's metadata word by a 32-bit add, each class at its
-    # measured rate over an array of the table's size
+    # bins' 32-B slot sectors and writes one slot by a 64-bit compare-and-swap,
+    # each class at its measured rate over an array of the table's size (the
+    # rate of adds to the metadata words is measured for reference: kicks add)
     red = atomic_rate(torch, ck, BINS * 4, 0, 1 << 26, stream)   # metadata words
     cas = atomic_rate(torch, ck, BINS * B * 8, 2, 1 << 26, stream)  # slots
-    model_ms = BATCH * (2 * 32 / (g32 * 1e9) + 1 / (cas * 1e9) + 1 / (red * 1e9)) * 1e3
+    model_ms = BATCH * (2 * 32 / (g32 * 1e9) + 1 / (cas * 1e9)) * 1e3
     first_ms = profile["launch_ms_at_load"]["0.000"]
     roofline["random_ops_model"] = {
         "gather32_g_per_s": round(g32 / 32, 2), "cas64_g_per_s": round(cas, 2), "red32_g_per_s": round(red, 2),
         "first_launch_ms": first_ms, "model_ms": round(model_ms, 4), "frac": round(model_ms / first_ms, 4),
         "note": "first 2^20-key launch (load 0 to 0.016, serialised) against 2 random 32-B reads + 1 random "
-                "64-bit CAS + 1 random 32-bit add per key at the probes' measured rates"}
+                "64-bit CAS per key at the probes' measured rates"}
     # against the random-gather roofline only the gathered bytes count: two
     # random 32-B sectors per lookup (the key in and the result out stream)
     look_random_gbs = N_LOOKUP * 2 * 32 / (look_ms / K * 1e-3) / 1e9
