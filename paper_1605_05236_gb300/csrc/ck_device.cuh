@@ -268,6 +268,14 @@ __device__ __forceinline__ uint32_t cas_acquire_old(uint32_t* p, uint32_t expect
   return old;
 }
 
+// relaxed: for a claim after which nothing is read (a free slot's)
+__device__ __forceinline__ uint32_t cas_relaxed_old(uint32_t* p, uint32_t expected, uint32_t desired) {
+  uint32_t old;
+  asm volatile("atom.relaxed.gpu.global.cas.b32 %0, [%1], %2, %3;"
+               : "=r"(old) : "l"(p), "r"(expected), "r"(desired) : "memory");
+  return old;
+}
+
 __device__ __forceinline__ bool cas_acquire(uint32_t* p, uint32_t expected, uint32_t desired) {
   return cas_acquire_old(p, expected, desired) == expected;
 }

@@ -310,15 +310,14 @@ __device__ __forceinline__ bool commit(const DevTable& t, Ctx& c) {
     }
     if (t.ordered_writes && i > 0) fence_release();  // the copy lands before its source is overwritten
   }
-  // ghost pairs (Sec. 4): the new record into both free slots
-  for (int i = n_chain; i < c.pn; i++) {
-    const uint64_t e = desc_at(c, i);
-    if (e_kind(e) != K_GHOST) continue;
-    if (!cas_slot(slot_at<B>(t, e), EMPTY, c.krec)) {
-      for (int j = n_chain; j < i; j++) {
-        const uint64_t f = desc_at(c, j);
-        if (e_kind(f) == K_GHOST) st_slot(slot_at<B>(t, f), EMPTY);
-      }
+  // a ghost pair (Sec. 4), a plan of its own: the new record into both free
+  // slots, in one round trip
+  if (c.pn == 2 && e_kind(desc_at(c, 0)) == K_GHOST) {
+    uint64_t *p0 = slot_at<B>(t, desc_at(c, 0)), *p1 = slot_at<B>(t, desc_at(c, 1));
+    const uint64_t o0 = cas_slot_old(p0, EMPTY, c.krec), o1 = cas_slot_old(p1, EMPTY, c.krec);
+    if (o0 != EMPTY || o1 != EMPTY) {
+      if (o0 == EMPTY) st_slot(p0, EMPTY);
+      if (o1 == EMPTY) st_slot(p1, EMPTY);
       fence_release();
       return false;
     }
@@ -361,12 +360,21 @@ __device__ __forceinline__ int dead_end(Ctx& c) {
   return ST_FAILED;
 }
 
-// Claim both free slots of a ghost pair (Sec. 4), the lower bin first: two
-// insertions whose keys hash to the same two bins in opposite order would
-// otherwise each claim its first bin, fail on the other's, release, and
-// meet again on every retry.
+// Claim both free slots of a ghost pair (Sec. 4).  The first attempt claims
+// them together, in one round trip.  After a conflict the lower bin goes
+// first: two insertions whose keys hash to the same two bins in opposite
+// order would otherwise each claim one bin, fail on the other's, release, and
+// meet again on every retry.  Nothing is read under these claims before the
+// slots are written by compare-and-swaps from empty.
 __device__ __forceinline__ bool claim_ghost_pair(const DevTable& t, Ctx& c, uint32_t b0, uint32_t m0, int s0,
                                                  uint32_t b1, uint32_t m1, int s1) {
+  if (c.attempt == 0) {
+    const uint32_t o0 = cas_relaxed_old(t.meta + b0, m0, m0 + (1u << s0));
+    const uint32_t o1 = cas_relaxed_old(t.meta + b1, m1, m1 + (1u << s1));
+    if (o0 == m0) put_entry(c, pack_entry(b0, s0, K_GHOST, false, 0, 0), EMPTY);
+    if (o1 == m1) put_entry(c, pack_entry(b1, s1, K_GHOST, false, 0, 0), EMPTY);
+    return o0 == m0 && o1 == m1;
+  }
   if (b1 < b0) {
     if (!claim(t, c, b1, m1, s1, K_GHOST, false, EMPTY)) return false;
     return claim(t, c, b0, m0, s0, K_GHOST, false, EMPTY);

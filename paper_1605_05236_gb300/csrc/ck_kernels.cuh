@@ -251,11 +251,12 @@ __device__ __forceinline__ int update_one(const DevTable& t, uint32_t key, uint6
   return 2;
 }
 
-// Insert kernel.  Concurrent mode: each block takes a contiguous range of
-// the batch and its threads pull keys from it, one insertion per thread at
-// a time, plans in local memory.  Serial mode (SERIAL, one
-// thread): keys in batch order, one insertion in flight, a scratch-backed
-// plan; this replays the paper's serial algorithms exactly.
+// Insert kernel, one insertion a thread from view to commit.  Serial mode
+// (SERIAL, one thread): keys in batch order, one insertion in flight, a
+// scratch-backed plan; this replays the paper's serial algorithms exactly.
+// Concurrent mode runs upserts (the other concurrent insertions go a step per
+// lane, ck_walk.cuh): each block takes a contiguous range of the batch and its
+// threads pull keys from it, plans in local memory.
 //
 // Consecutive insert launches may overlap (programmatic dependent launch):
 // each block lets the next launch start at once, and each thread waits for
