@@ -30,8 +30,7 @@
 // the word came back to the value seen (the 4-bit version wraps after 16
 // releases).  The writes themselves are therefore 64-bit compare-and-swaps
 // from the records the plan saw, undone if one fails, which closes that
-// gap.  The metadata word is read with acquire semantics before the slots,
-// so the slots seen are at least as new as that word.
+// gap.
 #pragma once
 #include <cstdint>
 #include <cuda/atomic>
@@ -280,12 +279,6 @@ __device__ __forceinline__ bool cas_acquire(uint32_t* p, uint32_t expected, uint
   return cas_acquire_old(p, expected, desired) == expected;
 }
 
-__device__ __forceinline__ uint32_t add_release(uint32_t* p, uint32_t delta) {
-  cuda::atomic_ref<uint32_t, cuda::thread_scope_device> a(*p);
-  return a.fetch_add(delta, cuda::memory_order_release);
-}
-
-// Fire-and-forget atomic add (no value returned).
 // 64-bit compare-and-swap of one slot (relaxed): the unclaimed placement
 // of a new key into a free slot, and a chain's write of its terminal free
 // slot, both of which must not overwrite a key another thread placed there.
@@ -305,11 +298,6 @@ __device__ __forceinline__ bool cas_slot(uint64_t* p, uint64_t expected, uint64_
 
 __device__ __forceinline__ void red_relaxed(uint32_t* p, uint32_t delta) {
   asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" :: "l"(p), "r"(delta) : "memory");
-}
-
-__device__ __forceinline__ uint32_t add_relaxed(uint32_t* p, uint32_t delta) {
-  cuda::atomic_ref<uint32_t, cuda::thread_scope_device> a(*p);
-  return a.fetch_add(delta, cuda::memory_order_relaxed);
 }
 
 // 64-bit counters of a block in shared memory, added to by 32-bit atomics with
@@ -349,18 +337,6 @@ struct View {
 };
 
 template <int B>
-__device__ __forceinline__ void load_view(const DevTable& t, uint32_t bin, View<B>& v) {
-  v.m = ld_acquire(t.meta + bin);
-  const uint64_t* p = t.slots + (uint64_t)bin * B;
-  if constexpr (B == 1) {
-    v.s[0] = ld_slot(p);
-  } else {
-#pragma unroll
-    for (int q = 0; q < B; q += 4) ld_bin4(p + q, v.s + q);
-  }
-}
-
-template <int B>
 __device__ __forceinline__ void load_slots(const DevTable& t, uint32_t bin, View<B>& v) {
   const uint64_t* p = t.slots + (uint64_t)bin * B;
   if constexpr (B == 1) {
@@ -376,7 +352,7 @@ __device__ __forceinline__ void load_slots(const DevTable& t, uint32_t bin, View
 // written by a compare-and-swap from empty, and every record they move is
 // read again after its claim (reread) -- so a view whose slots are older or
 // newer than its word costs a retry, never a wrong move.  Deletes, which
-// prove misses from their views, use load_view.
+// prove misses, read the words of all the key's bins first (read_words).
 template <int B>
 __device__ __forceinline__ void load_view_fast(const DevTable& t, uint32_t bin, View<B>& v) {
   v.m = ld_relaxed(t.meta + bin);
