@@ -78,7 +78,9 @@ extern "C" {
                                            either validates against claims (server lookups,
                                            deletes) or does not overlap writers (bulk lookups) */
 #define CK_PARAM_OVERLAP 32     /* 1 (default): an insert launch may start while the previous
-                                   one on the stream finishes its longest chains */
+                                   one on the stream finishes its longest chains.  Calls with
+                                   CK_INS_UPSERT or CK_INS_SERIAL overlap neither what is
+                                   before them on the stream nor what follows */
 #define CK_PARAM_SPAWN_K 34     /* searches (BFS, sorted, hybrid): spawns per round, 1..8
                                    (default 1).  Sec. 5: spawning the k best candidates at a
                                    time lets their bins be fetched together; every bin of a

@@ -258,12 +258,12 @@ __device__ __forceinline__ int update_one(const DevTable& t, uint32_t key, uint6
 // lane, ck_walk.cuh): each block takes a contiguous range of the batch and its
 // threads pull keys from it, plans in local memory.
 //
-// Consecutive insert launches may overlap (programmatic dependent launch):
-// each block lets the next launch start at once, and each thread waits for
-// the previous launch to finish before it exits, so a launch completes only
-// after its predecessor.  Insertions of distinct absent keys commute under
-// the claim protocol, so the overlap changes no result.  `load_base` is the
-// number of keys the table held before this batch (for the histogram).
+// Neither mode overlaps the launches around it (those of k_insert_walk do): an
+// upsert must find the keys of the calls before it, what follows must find
+// the upsert's, and a serial replay has one insertion in flight.  So there is
+// no launch_dependents here, and the launch waits for its predecessor.
+// `load_base` is the number of keys the table held before this batch (for the
+// histogram).
 // Registers: at most 64 (4 blocks of 256 or 8 of 128 threads per SM) for
 // most policies, 80 for 4-slot queue-kicking (3 blocks of 256).  Measured on
 // one GB300, fill of 2^24 x 4 to 0.95: queue-kicking 10.36-10.52 ms at 80
@@ -280,7 +280,6 @@ __global__ void __launch_bounds__(256, insert_blocks_per_sm<B, POL>()) k_insert(
                                                 uint8_t* __restrict__ status,
                                                 uint32_t* __restrict__ viewed_out, uint64_t load_base,
                                                 uint32_t upsert) {
-  asm volatile("griddepcontrol.launch_dependents;");
   __shared__ BlockTally bt;
   __shared__ unsigned long long s_next;  // next key of this block's range
   __shared__ int s_slab[SLABS_PER_BLOCK], s_long;
@@ -376,7 +375,6 @@ __global__ void __launch_bounds__(256, insert_blocks_per_sm<B, POL>()) k_insert(
     release_slabs(t, s_slab);
     if (s_long >= 0) release_long(t, s_long);
   }
-  asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // ------------------------------------------------------------------

@@ -16,7 +16,7 @@ struct InsertLaunch {
   const DevTable* dt;
   uint32_t block;
   int sm_count;
-  bool overlap;          // the launch may start while its predecessor finishes
+  bool overlap;          // the launch may start while its predecessor finishes (not upserts)
   uint64_t load_base;    // keys already in the table (the bins-viewed histogram's load)
   uint64_t max_threads;  // insertions in flight at most
 };
@@ -44,6 +44,10 @@ cudaError_t launch_insert(const InsertLaunch& l, const uint32_t* keys, const uin
   // a step per lane (ck_walk.cuh), except upserts, which first look for the
   // key under claims
   const bool walk = !upsert;
+  // An upsert's answer depends on the calls before it and the calls after it
+  // on its own writes, so it starts when its predecessor is complete (and
+  // k_insert lets nothing start beside it).
+  const bool overlap = l.overlap && walk;
   const size_t shared = walk ? walk_shared<B, POL, GHOST>(block) : 0;
   if (shared) {  // on every launch: the attribute is the current device's
     const cudaError_t e = cudaFuncSetAttribute(k_insert_walk<B, POL, GHOST>,
@@ -75,7 +79,7 @@ cudaError_t launch_insert(const InsertLaunch& l, const uint32_t* keys, const uin
   // search 6.32 against 6.56 and 6.47.  A limit the caller sets
   // (CK_PARAM_MAX_INFLIGHT) replaces this one.
   constexpr uint64_t tenths = (POL == P_QUEUE || POL == P_RANDOM) ? 9 : POL == P_RATTLE ? 8 : 7;
-  if (l.overlap && l.max_threads == ~0ull) {
+  if (overlap && l.max_threads == ~0ull) {
     const uint64_t most = resident * tenths / 10;
     resident = most > 0 ? most : 1;
   }
@@ -94,7 +98,7 @@ cudaError_t launch_insert(const InsertLaunch& l, const uint32_t* keys, const uin
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = l.overlap ? 1 : 0;
+  attr[0].val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   if (walk) return cudaLaunchKernelEx(&cfg, k_insert_walk<B, POL, GHOST>, dt, keys, vals, n, st, viewed, load_base);

@@ -509,6 +509,11 @@ constexpr int walk_blocks_per_sm =
 template <int B, int POL, bool GHOST>
 constexpr size_t walk_shared(uint32_t block) { return search_near<B, POL, GHOST> ? (size_t)block * NEAR_BYTES : 0; }
 
+// Consecutive launches may overlap (programmatic dependent launch): each block
+// lets the next launch start at once, and block 0 ends after the launch
+// before (see WAITERS), so a launch completes only after its predecessor.
+// Insertions of distinct absent keys commute under the claim protocol, so the
+// overlap changes no result.
 template <int B, int POL, bool GHOST>
 __global__ void __launch_bounds__(256, walk_blocks_per_sm<B, POL, GHOST>) k_insert_walk(DevTable t, const uint32_t* __restrict__ keys,
                                                         const uint32_t* __restrict__ vals, uint64_t n,
