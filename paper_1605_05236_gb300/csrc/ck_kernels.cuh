@@ -472,9 +472,9 @@ __global__ void __launch_bounds__(256) k_lookup2(DevTable t, const uint32_t* __r
         }
         const bool ph = __shfl_xor_sync(ALL, h, 1);
         const uint32_t pv = __shfl_xor_sync(ALL, v, 1);
-        if (half == u) {
+        if (half == u) {  // stored twice: the lower half's copy, for either lane
           f = h || ph;
-          val = h ? v : ph ? pv : 0u;
+          val = h && (half == 0 || !ph) ? v : ph ? pv : 0u;
         }
       }
     } else if (key != RESERVED_KEY) {
