@@ -175,6 +175,13 @@ __device__ __forceinline__ uint64_t next_draw(Txn& x) {
   return splitmix64_at(x.rng);
 }
 
+// A random wait of less than 128 ns << k (at most 0.52 ms), different for
+// every worker and attempt; it draws nothing from the worker's sequence.
+__device__ void random_wait(const Txn& x, uint32_t k) {
+  const uint64_t r = splitmix64_at(x.rng ^ ((uint64_t)x.epoch << 40) ^ k);
+  __nanosleep((uint32_t)r & ((128u << (k < 12 ? k : 12)) - 1));
+}
+
 // ---- the attempt's hash set of slots and bins in its read/write sets ----
 
 static_assert(HS == 1 << 11, "hs_home takes 11 bits");
@@ -785,11 +792,16 @@ __device__ bool lock_ws(const TxDev& t, Txn& x) {
 // holds with the write set locked.  Only a bin that is locked by another
 // transaction, or changing, makes the transaction release its locks, wait
 // for the check, and lock again (the paper's local retry; waiting while
-// holding locks could deadlock).
+// holding locks could deadlock).  Two workers that each read a bin the other
+// writes set each other off: both wait for the other to unlock and then lock
+// again together, and with write sets of nearly one size they would stay in
+// step for every pass of every attempt.  A random wait before locking again,
+// up to about the time a pass takes once a few were in vain, separates them.
 __device__ bool stage2(const TxDev& t, Txn& x) {
   const bool local = t.flags & CK_TXF_LOCAL_RETRY;
   sort_lock_order(x);
   int passes = 0;
+  uint32_t relocks = 0;
   while (passes < STAGE2_PASSES) {
     if (!lock_ws(t, x)) return false;
     bool relock = false;
@@ -861,6 +873,7 @@ __device__ bool stage2(const TxDev& t, Txn& x) {
       e.ver = w & ~3ull;
       atomicAdd(t.stats + TXS_LOCAL_RETRIES, 1ull);
     }
+    random_wait(x, 3 + ++relocks);
   }
   x.cause = TXS_ABORT_RS;
   return false;
@@ -1035,7 +1048,7 @@ __global__ void __launch_bounds__(32 * WORKERS_PER_BLOCK) k_txn_run(
         // eligible slot on every attempt: give those up
         if (x.cause == TXS_ABORT_OVERFLOW && ++overflows == OVERFLOWS_MAX) rc = 2;
         else if (x.cause == TXS_ABORT_CHAIN && ++chain_aborts == CHAIN_ABORTS_MAX) rc = 2;
-        else if (a > 16) __nanosleep(64u << (a < 24 ? a - 16 : 8));
+        else if (a > 16) random_wait(x, a - 16);  // attempts that keep meeting each other drift apart
       }
     }
     atomicAdd(t.stats + TXS_ATTEMPTS, (unsigned long long)a);
