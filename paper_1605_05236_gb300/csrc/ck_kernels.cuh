@@ -261,7 +261,8 @@ __device__ __forceinline__ int update_one(const DevTable& t, uint32_t key, uint6
 // Neither mode overlaps the launches around it (those of k_insert_walk do): an
 // upsert must find the keys of the calls before it, what follows must find
 // the upsert's, and a serial replay has one insertion in flight.  So there is
-// no launch_dependents here, and the launch waits for its predecessor.
+// no launch_dependents here, and the first thing done is the wait for the
+// launch before.
 // `load_base` is the number of keys the table held before this batch (for the
 // histogram).
 // Registers: at most 64 (4 blocks of 256 or 8 of 128 threads per SM) for
@@ -280,6 +281,7 @@ __global__ void __launch_bounds__(256, insert_blocks_per_sm<B, POL>()) k_insert(
                                                 uint8_t* __restrict__ status,
                                                 uint32_t* __restrict__ viewed_out, uint64_t load_base,
                                                 uint32_t upsert) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   __shared__ BlockTally bt;
   __shared__ unsigned long long s_next;  // next key of this block's range
   __shared__ int s_slab[SLABS_PER_BLOCK], s_long;
