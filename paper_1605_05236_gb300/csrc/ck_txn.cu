@@ -680,8 +680,8 @@ __device__ int plan_insert(const TxDev& t, Txn& x, uint64_t rec, uint32_t b0, ui
       if (!mini_move(t, path[q - 1], pword[q - 1], path[q], pword[q], pbin[q], pold[q - 1])) {
         moved_all = false;
         atomicAdd(t.stats + TXS_MINI_ABORTS, 1ull);
-        if (claim)
-          for (int r = 0; r < q; r++) unclaim(t, path[r]);
+        if (claim)  // path[q] too: the move would have ended its claim
+          for (int r = 0; r <= q; r++) unclaim(t, path[r]);
         break;
       }
       atomicAdd(t.stats + TXS_MINI_TXNS, 1ull);
