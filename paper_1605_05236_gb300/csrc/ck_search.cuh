@@ -767,10 +767,9 @@ __device__ int insert_search_dary(const DevTable& t, Ctx& c, uint8_t* region) {
 
 // A block's search scratch: ceil(blockDim / SLAB) slabs of SLAB consecutive
 // per-thread regions, taken together at block start (all or none: a block
-// never waits while holding a slab, so blocks of overlapping launches cannot
-// hold each other up) and returned at block end.  A block of the next launch
-// may wait for slabs while the previous launch drains; the wait is bounded
-// (about 10 ms), after which the block reports its keys as aborted.
+// never waits while holding a slab) and returned at block end.  A launch has
+// at most as many blocks as there are slabs for.  This form is for launches
+// that overlap no other (k_insert): false if the pool is too small.
 __device__ __forceinline__ bool acquire_slabs(const DevTable& t, int* out, int need) {
   const uint32_t n_slabs = t.n_searchers / SLAB;
   if (n_slabs < (uint32_t)need) return false;
@@ -819,6 +818,18 @@ __device__ __forceinline__ bool acquire_slabs_warp(const DevTable& t, int* out, 
     __nanosleep(2000);
   }
   return false;
+}
+
+// The slabs of a block whose launch may have started beside the one before, by
+// a whole warp.  That launch can hold them for as long as its slowest keys
+// search (longer than any fixed number of looks, about 10 ms of them here), so
+// then its end is waited for: after it only this launch's blocks hold slabs,
+// because the launch after this one starts once every block of this one has
+// its own (the callers' launch_dependents comes after this).
+__device__ __forceinline__ bool take_slabs(const DevTable& t, int* out, int need) {
+  if (acquire_slabs_warp(t, out, need)) return true;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  return acquire_slabs_warp(t, out, need);
 }
 
 // The calling thread's region in a block's slabs (null if it got none).

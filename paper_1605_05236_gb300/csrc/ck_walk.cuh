@@ -510,8 +510,8 @@ template <int B, int POL, bool GHOST>
 constexpr size_t walk_shared(uint32_t block) { return search_near<B, POL, GHOST> ? (size_t)block * NEAR_BYTES : 0; }
 
 // Consecutive launches may overlap (programmatic dependent launch): each block
-// lets the next launch start at once, and block 0 ends after the launch
-// before (see WAITERS), so a launch completes only after its predecessor.
+// lets the next launch start at once (a search once it has its slabs), and
+// block 0 ends after the launch before (see WAITERS), so a launch completes only after its predecessor.
 // Insertions of distinct absent keys commute under the claim protocol, so the
 // overlap changes no result.
 template <int B, int POL, bool GHOST>
@@ -519,20 +519,21 @@ __global__ void __launch_bounds__(256, walk_blocks_per_sm<B, POL, GHOST>) k_inse
                                                         const uint32_t* __restrict__ vals, uint64_t n,
                                                         uint8_t* __restrict__ status,
                                                         uint32_t* __restrict__ viewed_out, uint64_t load_base) {
-  asm volatile("griddepcontrol.launch_dependents;");
+  constexpr bool SEARCH = is_search_policy<POL>;
+  if (!SEARCH) asm volatile("griddepcontrol.launch_dependents;");
   __shared__ BlockTally bt;
   __shared__ LookState ls;
   const uint64_t per = (n + gridDim.x - 1) / gridDim.x;
   const uint64_t lo = min(n, (uint64_t)blockIdx.x * per), hi = min(n, lo + per);
-  constexpr bool SEARCH = is_search_policy<POL>;
   __shared__ int s_slab[SEARCH ? SLABS_PER_BLOCK : 1];
   bt.clear();
   ls.begin(t, lo, load_base);
   if (SEARCH && threadIdx.x < 32) {
-    const bool got = acquire_slabs_warp(t, s_slab, (int)((blockDim.x + SLAB - 1) / SLAB));
+    const bool got = take_slabs(t, s_slab, (int)((blockDim.x + SLAB - 1) / SLAB));
     if (!got && threadIdx.x == 0) s_slab[0] = -1;
   }
   __syncthreads();
+  if (SEARCH) asm volatile("griddepcontrol.launch_dependents;");  // see take_slabs
   PlanStore<MAX_CHAIN> store;
   BatchKeys<B, POL, (B > 1 && !GHOST)> src{t, keys, vals, status, viewed_out, hi, load_base, bt, ls, true, 0, 0, 0};
   walk_keys<B, POL, GHOST>(src, store.e, SEARCH ? slab_region(t, s_slab) : nullptr);

@@ -232,7 +232,6 @@ __global__ void __launch_bounds__(WARP_BLOCK, 8) k_insert_warp(DevTable t, const
                                                                const uint32_t* __restrict__ vals, uint64_t n,
                                                                uint8_t* __restrict__ status,
                                                                uint32_t* __restrict__ viewed_out, uint64_t load_base) {
-  asm volatile("griddepcontrol.launch_dependents;");
   __shared__ WarpGroups<B> ws[WARP_BLOCK / 32];
   __shared__ unsigned int h_views[HIST_BUCKETS];
   __shared__ unsigned int h_cnt[HIST_BUCKETS];
@@ -245,12 +244,13 @@ __global__ void __launch_bounds__(WARP_BLOCK, 8) k_insert_warp(DevTable t, const
   for (int i = threadIdx.x; i < C_N; i += blockDim.x) bc[i] = 0;
   const uint64_t per = (n + gridDim.x - 1) / gridDim.x;
   const uint64_t lo = min(n, (uint64_t)blockIdx.x * per), hi = min(n, lo + per);
-  if (threadIdx.x == 0) {
-    s_next = lo;
-    const int need = (int)((blockDim.x + SLAB - 1) / SLAB);
-    if (!t.scratch || !acquire_slabs(t, s_slab, need)) s_slab[0] = -1;
+  if (threadIdx.x == 0) s_next = lo;
+  if (threadIdx.x < 32) {
+    const bool got = t.scratch && take_slabs(t, s_slab, (int)((blockDim.x + SLAB - 1) / SLAB));
+    if (!got && threadIdx.x == 0) s_slab[0] = -1;
   }
   __syncthreads();
+  asm volatile("griddepcontrol.launch_dependents;");  // see take_slabs
   WarpGroups<B>& W = ws[threadIdx.x / 32];
   const uint32_t lane = threadIdx.x & 31u;
   PlanStore<MAX_CHAIN> store;
