@@ -531,48 +531,56 @@ static __global__ void __launch_bounds__(256) k_lookup_dary(DevTable t, const ui
   count_lookups(t, hits, cnt);
 }
 
-// The hit field of every metadata word, for an export (sign 1: the bin's
+// The hit field of n bins' metadata words, for an export (sign 1: the bin's
 // occupied slots added, which makes it queue-kicking's hit counter) and back
-// (sign -1).  B is 4 or 8.
-static __global__ void __launch_bounds__(256) k_convert_hits(const uint64_t* slots, uint32_t* meta, uint64_t n_bins,
-                                                             uint32_t B, int sign) {
+// (sign -1).  B is 4 or 8; in and out may be the same words.
+static __global__ void __launch_bounds__(256) k_convert_hits(const uint64_t* slots, const uint32_t* in, uint32_t* out,
+                                                             uint64_t n, uint32_t B, int sign) {
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; b < n_bins; b += stride) {
+  for (uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; b < n; b += stride) {
     uint32_t occupied = 0;
     for (uint32_t s = 0; s < B; s++) occupied += slots[b * B + s] != EMPTY;
-    const uint32_t m = meta[b];
+    const uint32_t m = in[b];
     const uint32_t h = ((m >> HIT_SHIFT) + (uint32_t)sign * occupied) & 255u;
-    meta[b] = (m & ~(255u << HIT_SHIFT)) | (h << HIT_SHIFT);
+    out[b] = (m & ~(255u << HIT_SHIFT)) | (h << HIT_SHIFT);
   }
 }
 
+inline cudaError_t convert_hits(const DevTable& t, uint64_t first, uint64_t n, uint32_t* out, int sign) {
+  const unsigned grid = (unsigned)(n < 256 * 4096 ? (n + 255) / 256 : 4096);
+  k_convert_hits<<<grid, 256>>>(t.slots + first * t.B, t.meta + first, out, n, t.B, sign);
+  return cudaGetLastError();
+}
+
 // Metadata words to host memory in the exported form (hit counters of
-// queue-kicking tables), the device's words as they were afterwards.  On the
-// legacy default stream, with no other work on the table.
+// queue-kicking tables), converted a part at a time in a buffer of its own:
+// an export reads the table and writes nothing of it, so exports may run
+// beside each other and beside lookups.  On the legacy default stream.
 inline cudaError_t copy_meta_out(const DevTable& t, uint32_t* h_meta) {
-  const bool convert = t.policy == P_QUEUE && t.B > 1;
-  const unsigned grid = (unsigned)(t.n_bins < 256 * 4096 ? (t.n_bins + 255) / 256 : 4096);
-  if (convert) {
-    k_convert_hits<<<grid, 256>>>(t.slots, t.meta, t.n_bins, t.B, 1);
-    const cudaError_t e1 = cudaGetLastError();
-    if (e1 != cudaSuccess) return e1;
+  if (t.policy != P_QUEUE || t.B == 1)
+    return cudaMemcpy(h_meta, t.meta, t.n_bins * sizeof(uint32_t), cudaMemcpyDeviceToHost);
+  uint64_t part = t.n_bins < (1u << 22) ? t.n_bins : 1u << 22;  // 16 MiB at most, less where memory is short
+  uint32_t* buf = nullptr;
+  cudaError_t e;
+  while ((e = cudaMalloc(&buf, part * sizeof(uint32_t))) == cudaErrorMemoryAllocation && part > 4096) {
+    cudaGetLastError();
+    part /= 2;
   }
-  cudaError_t e = cudaMemcpy(h_meta, t.meta, t.n_bins * sizeof(uint32_t), cudaMemcpyDeviceToHost);
-  if (convert) {
-    k_convert_hits<<<grid, 256>>>(t.slots, t.meta, t.n_bins, t.B, -1);
-    const cudaError_t e2 = cudaStreamSynchronize(nullptr);  // callers may go on on another stream
-    if (e == cudaSuccess) e = e2;
+  if (e != cudaSuccess) return e;
+  for (uint64_t b = 0; b < t.n_bins && e == cudaSuccess; b += part) {
+    const uint64_t n = t.n_bins - b < part ? t.n_bins - b : part;
+    e = convert_hits(t, b, n, buf, 1);
+    if (e == cudaSuccess) e = cudaMemcpy(h_meta + b, buf, n * sizeof(uint32_t), cudaMemcpyDeviceToHost);
   }
+  cudaFree(buf);
   return e;
 }
 
 // Words as exported, back into the device's form (the slots are in place).
 inline cudaError_t convert_meta_in(const DevTable& t) {
   if (t.policy != P_QUEUE || t.B == 1) return cudaSuccess;
-  const unsigned grid = (unsigned)(t.n_bins < 256 * 4096 ? (t.n_bins + 255) / 256 : 4096);
-  k_convert_hits<<<grid, 256>>>(t.slots, t.meta, t.n_bins, t.B, -1);
-  const cudaError_t e = cudaGetLastError();
-  return e == cudaSuccess ? cudaStreamSynchronize(nullptr) : e;
+  const cudaError_t e = convert_hits(t, 0, t.n_bins, t.meta, -1);
+  return e == cudaSuccess ? cudaStreamSynchronize(nullptr) : e;  // callers may go on on another stream
 }
 
 template <int B>
