@@ -47,7 +47,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
         return LIB
     os.makedirs(BUILD, exist_ok=True)
     cc = nvcc()
-    flags = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC",
+    # device code uncompressed: nvcc compresses the larger units, and the first
+    # launch from each then unpacks it (11 ms against 1.8 for 8-slot bins)
+    flags = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-no-compress", "-Xcompiler", "-fPIC",
                     "-I" + os.path.join(ROOT, "include"), "-I" + CSRC]
     objs = []
 
