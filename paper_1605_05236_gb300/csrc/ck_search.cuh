@@ -416,122 +416,131 @@ __device__ __forceinline__ void search_begin(const DevTable& t, Ctx& c, Search<B
 
 constexpr int SEARCHING = -1;
 
-// One round: up to spawn_k spawns in candidate order, their bins fetched
+// Rounds of up to spawn_k spawns in candidate order, their bins fetched
 // together (Sec. 5: spawning the k best records at a time lets the fetches
 // overlap); the first of them with room ends the search, the others join as
 // groups.  spawn_k = 1 is the plain search: one spawn, whose count goes up
-// while its bin is viewed.  SEARCHING: another round follows.
-template <int B, int ORDER, bool GHOST, bool NEAR>
-__device__ __forceinline__ int search_round(const DevTable& t, Ctx& c, Search<B, NEAR>& S) {
-  uint32_t rg[8], ry[8];
-  uint8_t rs[8];
-  uint32_t nr = 0, g0 = 0, s0 = 0, y0 = 0;
-  View<B> vy;
-  bool out = false;  // budget spent during the round
-  while (nr < t.spawn_k) {
-    uint32_t s;
-    if (!S.template pop<ORDER>(s)) break;
-    if ((S.meta >> s) & 1u) {  // claimed by another insertion: ignore it (Sec. 8)
-      c.foreign = 1;
-      continue;
-    }
-    const uint64_t rec = ld_slot(t.slots + (uint64_t)S.bin * B + s);
-    if (rec == EMPTY) continue;
-    const uint32_t y = other_bin2(t, rec, S.bin), g = S.cur;
-    if (S.marked(c, y)) continue;
-    const bool spent = c.viewed - c.viewed0 >= S.budget(t, c) || S.ng + nr >= S.max_groups(c);
-    // the spawn counts even where the budget ends the search
-    const bool count = ORDER != P_BFS && spawn_of(S.meta) < 15;
-    const uint32_t nm = S.meta + (1u << SPAWN_SHIFT);
-    uint32_t old = S.meta;
-    if (count) old = cas_acquire_old(t.meta + S.bin, S.meta, nm);
-    if (!spent && t.spawn_k == 1) load_view_fast<B>(t, y, vy);
-    if (count) {
-      if (old == S.meta) {
-        S.meta = nm;
-        S.at(g).meta = nm;
-      } else {
-        S.at(g).stale = 1;
-        uint32_t m = ld_acquire(t.meta + S.bin);
-        for (int k = 0; k < 64 && spawn_of(m) < 15; k++) {  // bounded: a lost count is harmless
-          if (cas_acquire(t.meta + S.bin, m, m + (1u << SPAWN_SHIFT))) break;
-          m = ld_acquire(t.meta + S.bin);
+// while its bin is viewed.  STEP: one round, SEARCHING if another follows (the
+// concurrent kernels); else all of them, as the last thing the first step
+// does, which keeps a thread's search one loop that no other thread's first
+// step holds up.  With a loop of steps around it instead, upserts of absent
+// keys took 6.3 ms against 5.0 (d = 4 sorted search, 2^23 bins from 0.75 to
+// 0.90) and 2.9 against 2.55 (2^21 x 8 sorted search, 0.85 to 0.96), whose
+// spills fell from 776 to 216 bytes.
+template <int B, int ORDER, bool GHOST, bool NEAR, bool STEP>
+__device__ __forceinline__ int search_rounds(const DevTable& t, Ctx& c, Search<B, NEAR>& S) {
+  for (;;) {
+    uint32_t rg[8], ry[8];
+    uint8_t rs[8];
+    uint32_t nr = 0, g0 = 0, s0 = 0, y0 = 0;
+    View<B> vy;
+    bool out = false;  // budget spent during the round
+    while (nr < t.spawn_k) {
+      uint32_t s;
+      if (!S.template pop<ORDER>(s)) break;
+      if ((S.meta >> s) & 1u) {  // claimed by another insertion: ignore it (Sec. 8)
+        c.foreign = 1;
+        continue;
+      }
+      const uint64_t rec = ld_slot(t.slots + (uint64_t)S.bin * B + s);
+      if (rec == EMPTY) continue;
+      const uint32_t y = other_bin2(t, rec, S.bin), g = S.cur;
+      if (S.marked(c, y)) continue;
+      const bool spent = c.viewed - c.viewed0 >= S.budget(t, c) || S.ng + nr >= S.max_groups(c);
+      // the spawn counts even where the budget ends the search
+      const bool count = ORDER != P_BFS && spawn_of(S.meta) < 15;
+      const uint32_t nm = S.meta + (1u << SPAWN_SHIFT);
+      uint32_t old = S.meta;
+      if (count) old = cas_acquire_old(t.meta + S.bin, S.meta, nm);
+      if (!spent && t.spawn_k == 1) load_view_fast<B>(t, y, vy);
+      if (count) {
+        if (old == S.meta) {
+          S.meta = nm;
+          S.at(g).meta = nm;
+        } else {
+          S.at(g).stale = 1;
+          uint32_t m = ld_acquire(t.meta + S.bin);
+          for (int k = 0; k < 64 && spawn_of(m) < 15; k++) {  // bounded: a lost count is harmless
+            if (cas_acquire(t.meta + S.bin, m, m + (1u << SPAWN_SHIFT))) break;
+            m = ld_acquire(t.meta + S.bin);
+          }
         }
       }
-    }
-    if (spent) {
-      out = true;
-      break;
-    }
-    S.mark(c, y);
-    c.viewed++;
-    if (nr == 0) {
-      g0 = g;
-      s0 = s;
-      y0 = y;
-    } else {
-      rg[nr] = g;
-      rs[nr] = (uint8_t)s;
-      ry[nr] = y;
-    }
-    if (t.spawn_k > 1) prefetch_bin<B>(t, y);
-    nr++;
-  }
-  if (nr == 0) return dead_end(c);
-  for (uint32_t i = 0; i < nr; i++) {
-    const uint32_t g = i ? rg[i] : g0, s = i ? rs[i] : s0, y = i ? ry[i] : y0;
-    if (t.spawn_k > 1) load_view_fast<B>(t, y, vy);
-    if (claimed_mask<B>(vy)) c.foreign = 1;
-    int term = lowest(free_mask<B>(vy));
-    bool isdup = false;
-    if (term < 0 && GHOST) {
-      term = lowest(dup_mask<B>(vy));
-      isdup = term >= 0;
-    }
-    if (term < 0) {
-      S.template push<ORDER>(y, vy.m, (g << 3) | s);
-      continue;
-    }
-    // path root -> ... -> (g, s): depth entries in chain order
-    uint32_t depth = 1;
-    for (uint32_t q = g; S.at(q).parent != NO_PARENT; q = S.at(q).parent >> 3) depth++;
-    if ((int)depth + 4 > c.pcap) return ST_LONG;
-    {
-      // entries in chain order; the group index rides in the content word
-      // until the slot is claimed
-      uint32_t q = g, qs = s;
-      for (int e = (int)depth - 1; e >= 0; e--) {
-        set_entry(c, e, pack_entry(S.at(q).bin, (int)qs, K_MOVE, false, 0, 0), q);
-        uint32_t par = S.at(q).parent;
-        if (par != NO_PARENT) { qs = par & 7u; q = par >> 3; }
+      if (spent) {
+        out = true;
+        break;
       }
+      S.mark(c, y);
+      c.viewed++;
+      if (nr == 0) {
+        g0 = g;
+        s0 = s;
+        y0 = y;
+      } else {
+        rg[nr] = g;
+        rs[nr] = (uint8_t)s;
+        ry[nr] = y;
+      }
+      if (t.spawn_k > 1) prefetch_bin<B>(t, y);
+      nr++;
     }
-    // claim the path in chain order; each CAS checks its bin is as viewed,
-    // so the record read after the claim is the one the search saw
-    c.pn = 0;
-    for (uint32_t e = 0; e < depth; e++) {
-      Group gq = S.at((uint32_t)content_at(c, (int)e));
-      uint32_t sl = e_slot(desc_at(c, (int)e));
-      if (gq.stale) return ST_CONFLICT;
-      if (!cas_acquire(t.meta + gq.bin, gq.meta, gq.meta + (1u << sl))) return ST_CONFLICT;
-      c.pn = (int)e + 1;
-      // the record must move into the next bin of the path: it is the one
-      // the search saw unless the bin's word came back to its viewed value
-      const uint64_t r = reread<B>(t, gq.bin, sl);
-      const uint32_t to = e + 1 < depth ? S.at((uint32_t)content_at(c, (int)e + 1)).bin : y;
-      set_content(c, (int)e, r);
-      if (!belongs<B>(t, r, to)) return ST_CONFLICT;
+    if (nr == 0) return dead_end(c);
+    for (uint32_t i = 0; i < nr; i++) {
+      const uint32_t g = i ? rg[i] : g0, s = i ? rs[i] : s0, y = i ? ry[i] : y0;
+      if (t.spawn_k > 1) load_view_fast<B>(t, y, vy);
+      if (claimed_mask<B>(vy)) c.foreign = 1;
+      int term = lowest(free_mask<B>(vy));
+      bool isdup = false;
+      if (term < 0 && GHOST) {
+        term = lowest(dup_mask<B>(vy));
+        isdup = term >= 0;
+      }
+      if (term < 0) {
+        S.template push<ORDER>(y, vy.m, (g << 3) | s);
+        continue;
+      }
+      // path root -> ... -> (g, s): depth entries in chain order
+      uint32_t depth = 1;
+      for (uint32_t q = g; S.at(q).parent != NO_PARENT; q = S.at(q).parent >> 3) depth++;
+      if ((int)depth + 4 > c.pcap) return ST_LONG;
+      {
+        // entries in chain order; the group index rides in the content word
+        // until the slot is claimed
+        uint32_t q = g, qs = s;
+        for (int e = (int)depth - 1; e >= 0; e--) {
+          set_entry(c, e, pack_entry(S.at(q).bin, (int)qs, K_MOVE, false, 0, 0), q);
+          uint32_t par = S.at(q).parent;
+          if (par != NO_PARENT) { qs = par & 7u; q = par >> 3; }
+        }
+      }
+      // claim the path in chain order; each CAS checks its bin is as viewed,
+      // so the record read after the claim is the one the search saw
+      c.pn = 0;
+      for (uint32_t e = 0; e < depth; e++) {
+        Group gq = S.at((uint32_t)content_at(c, (int)e));
+        uint32_t sl = e_slot(desc_at(c, (int)e));
+        if (gq.stale) return ST_CONFLICT;
+        if (!cas_acquire(t.meta + gq.bin, gq.meta, gq.meta + (1u << sl))) return ST_CONFLICT;
+        c.pn = (int)e + 1;
+        // the record must move into the next bin of the path: it is the one
+        // the search saw unless the bin's word came back to its viewed value
+        const uint64_t r = reread<B>(t, gq.bin, sl);
+        const uint32_t to = e + 1 < depth ? S.at((uint32_t)content_at(c, (int)e + 1)).bin : y;
+        set_content(c, (int)e, r);
+        if (!belongs<B>(t, r, to)) return ST_CONFLICT;
+      }
+      c.kicks = depth;
+      if (isdup) return take_dup<B>(t, c, y, vy, term, false);
+      return take_free<B>(t, c, y, vy, term, false);
     }
-    c.kicks = depth;
-    if (isdup) return take_dup<B>(t, c, y, vy, term, false);
-    return take_free<B>(t, c, y, vy, term, false);
+    if (out) return out_of_cap(c);
+    if (STEP) return SEARCHING;
   }
-  return out ? out_of_cap(c) : SEARCHING;
 }
 
 // The first step of a search policy's insertion: room in one of the key's
 // bins (or, with ghosts, a duplicate), or SEARCHING with the search begun.
-template <int B, int ORDER, bool GHOST, bool NEAR>
+template <int B, int ORDER, bool GHOST, bool NEAR, bool STEP>
 __device__ __forceinline__ int search_first(const DevTable& t, Ctx& c, Search<B, NEAR>& S, uint8_t* region) {
   uint32_t b0, b1;
   bins2(t, c.key, b0, b1);
@@ -569,16 +578,15 @@ __device__ __forceinline__ int search_first(const DevTable& t, Ctx& c, Search<B,
     if (f1) return take_free<B>(t, c, b1, v1, lowest(f1), false);
   }
   search_begin<B, ORDER, NEAR>(t, c, S, region, b0, v0.m, b1, v1.m);
-  return SEARCHING;
+  if (STEP) return SEARCHING;
+  return search_rounds<B, ORDER, GHOST, NEAR, false>(t, c, S);
 }
 
 // ORDER: P_BFS, P_SORTED or P_HYBRID
 template <int B, int ORDER, bool GHOST>
 __device__ int insert_search(const DevTable& t, Ctx& c, uint8_t* region) {
   Search<B, false> S;
-  int r = search_first<B, ORDER, GHOST, false>(t, c, S, region);
-  while (r == SEARCHING) r = search_round<B, ORDER, GHOST, false>(t, c, S);
-  return r;
+  return search_first<B, ORDER, GHOST, false, false>(t, c, S, region);
 }
 
 // ------------------------------------------------------------------
@@ -618,8 +626,123 @@ __device__ __forceinline__ void push_dary(DarySearch& S, uint32_t bin, uint32_t 
   vis_insert(S.sp.vis, S.sp.vis_bits, S.gen, bin);
 }
 
-// The first step: placed (a status), or SEARCHING with the search begun.
-template <int ORDER>
+// Rounds of spawn_k tries, as in the two-choice searches: one (STEP) or all.
+template <int ORDER, bool STEP>
+__device__ __forceinline__ int search_rounds_dary(const DevTable& t, Ctx& c, DarySearch& S) {
+  const uint32_t d = t.d;
+  Group* G = S.sp.G;
+  uint64_t* vis = S.sp.vis;
+  const uint32_t vb = S.sp.vis_bits, gen = S.gen;
+  uint32_t &ng = S.ng, &head = S.head;
+  Buckets& bq = S.bq;
+  GroupCache<4>& k = S.k;
+  const SearchSpace& sp = S.sp;
+  for (;;) {
+    uint32_t rg[8], ry[8];
+    uint32_t nr = 0;
+    bool out = false;
+    while (nr < t.spawn_k) {
+      uint32_t g, j, y;
+      if (ORDER == P_BFS) {  // the oldest group, until its hash functions run out
+        if (k.g == head && k.next >= d) head++;
+        if (head == ng) break;  // nothing left to try
+        if (k.g != head) take_group_dary(t, G, head, vis, vb, gen, k);
+        g = head;
+        j = k.next++;
+        if (k.meta & 1u) {  // claimed by another insertion: ignore it (Sec. 8)
+          c.foreign = 1;
+          continue;
+        }
+        // empty, the record's own bin, or a bin already viewed
+        if (!((k.ok >> j) & 1u)) continue;
+        y = pick<4>(k.y, j);
+        if (spawned_to<4>(k, y)) continue;
+      } else {  // the smallest key, oldest first among equals
+        const int bk = bucket_min(ORDER, bq);
+        if (bk < 0) break;
+        g = bq.q[bk];
+        Group gr = G[g];
+        j = gr.next;
+        G[g].next = (uint8_t)(j + 1);
+        if (j + 1 >= d) bucket_pop(bq, G, (uint32_t)bk, g);
+        if (gr.meta & 1u) {
+          c.foreign = 1;
+          continue;
+        }
+        uint64_t rec = ld_slot(t.slots + gr.bin);
+        if (rec == EMPTY) continue;
+        uint32_t rb[4];
+        bins_of(t, key_of(rec), rb);
+        y = rb[j];
+        if (y == gr.bin || vis_has(vis, vb, gen, y)) continue;
+        if (spawn_of(gr.meta) < 15) {
+          uint32_t nm = gr.meta + (1u << SPAWN_SHIFT);
+          if (cas_acquire(t.meta + gr.bin, gr.meta, nm)) {
+            G[g].meta = nm;
+          } else {
+            G[g].stale = 1;
+            uint32_t m = ld_acquire(t.meta + gr.bin);
+            for (int q = 0; q < 64 && spawn_of(m) < 15; q++) {  // bounded: a lost count is harmless
+              if (cas_acquire(t.meta + gr.bin, m, m + (1u << SPAWN_SHIFT))) break;
+              m = ld_acquire(t.meta + gr.bin);
+            }
+          }
+        }
+      }
+      if (c.viewed - c.viewed0 >= sp.budget || ng + nr >= sp.max_groups) { out = true; break; }  // budget spent
+      vis_insert(vis, vb, gen, y);
+      if (ORDER == P_BFS) k.spawned |= 1u << j;
+      c.viewed++;
+      prefetch_bin<1>(t, y);
+      rg[nr] = g;
+      ry[nr] = y;
+      nr++;
+    }
+    if (nr == 0) return dead_end(c);
+    for (uint32_t i = 0; i < nr; i++) {
+      const uint32_t g = rg[i], y = ry[i];
+      View<1> vy;
+      load_view_fast<1>(t, y, vy);
+      if (claimed_mask<1>(vy)) c.foreign = 1;
+      if (!free_mask<1>(vy)) {
+        push_dary<ORDER>(S, y, vy.m, g << 3);
+        continue;
+      }
+      // path: root group -> ... -> group g, one record each, in chain order
+      uint32_t depth = 1;
+      for (uint32_t q = g; G[q].parent != NO_PARENT; q = G[q].parent >> 3) depth++;
+      if ((int)depth + 4 > c.pcap) return ST_LONG;
+      {
+        uint32_t q = g;
+        for (int e = (int)depth - 1; e >= 0; e--) {
+          set_entry(c, e, pack_entry(G[q].bin, 0, K_MOVE, false, 0, 0), q);
+          if (G[q].parent != NO_PARENT) q = G[q].parent >> 3;
+        }
+      }
+      // claim the path in chain order from the metadata words as viewed; the
+      // record read after a claim is the one the search saw
+      c.pn = 0;
+      for (uint32_t e = 0; e < depth; e++) {
+        Group gq = G[(uint32_t)content_at(c, (int)e)];
+        if (gq.stale) return ST_CONFLICT;
+        if (!cas_acquire(t.meta + gq.bin, gq.meta, gq.meta + 1u)) return ST_CONFLICT;
+        c.pn = (int)e + 1;
+        const uint64_t r = reread<1>(t, gq.bin, 0);
+        const uint32_t to = e + 1 < depth ? G[(uint32_t)content_at(c, (int)e + 1)].bin : y;
+        set_content(c, (int)e, r);
+        if (!belongs<1>(t, r, to)) return ST_CONFLICT;
+      }
+      c.kicks = depth;
+      return take_free<1>(t, c, y, vy, 0, false);
+    }
+    if (out) return out_of_cap(c);
+    if (STEP) return SEARCHING;
+  }
+}
+
+// The first step: placed (a status), or the search begun -- SEARCHING (STEP), or
+// its end.
+template <int ORDER, bool STEP>
 __device__ __forceinline__ int search_first_dary(const DevTable& t, Ctx& c, DarySearch& S, uint8_t* region) {
   const uint32_t d = t.d;
   uint32_t b[4];
@@ -641,127 +764,14 @@ __device__ __forceinline__ int search_first_dary(const DevTable& t, Ctx& c, Dary
   S.bq.depth = 0;
   for (uint32_t i = 0; i < d; i++) push_dary<ORDER>(S, b[i], v[i].m, NO_PARENT);
   S.k.g = ~0u;
-  return SEARCHING;
-}
-
-// A round of spawn_k tries, as in the two-choice searches.
-template <int ORDER>
-__device__ __forceinline__ int search_round_dary(const DevTable& t, Ctx& c, DarySearch& S) {
-  const uint32_t d = t.d;
-  Group* G = S.sp.G;
-  uint64_t* vis = S.sp.vis;
-  const uint32_t vb = S.sp.vis_bits, gen = S.gen;
-  uint32_t &ng = S.ng, &head = S.head;
-  Buckets& bq = S.bq;
-  GroupCache<4>& k = S.k;
-  const SearchSpace& sp = S.sp;
-  uint32_t rg[8], ry[8];
-  uint32_t nr = 0;
-  bool out = false;
-  while (nr < t.spawn_k) {
-    uint32_t g, j, y;
-    if (ORDER == P_BFS) {  // the oldest group, until its hash functions run out
-      if (k.g == head && k.next >= d) head++;
-      if (head == ng) break;  // nothing left to try
-      if (k.g != head) take_group_dary(t, G, head, vis, vb, gen, k);
-      g = head;
-      j = k.next++;
-      if (k.meta & 1u) {  // claimed by another insertion: ignore it (Sec. 8)
-        c.foreign = 1;
-        continue;
-      }
-      // empty, the record's own bin, or a bin already viewed
-      if (!((k.ok >> j) & 1u)) continue;
-      y = pick<4>(k.y, j);
-      if (spawned_to<4>(k, y)) continue;
-    } else {  // the smallest key, oldest first among equals
-      const int bk = bucket_min(ORDER, bq);
-      if (bk < 0) break;
-      g = bq.q[bk];
-      Group gr = G[g];
-      j = gr.next;
-      G[g].next = (uint8_t)(j + 1);
-      if (j + 1 >= d) bucket_pop(bq, G, (uint32_t)bk, g);
-      if (gr.meta & 1u) {
-        c.foreign = 1;
-        continue;
-      }
-      uint64_t rec = ld_slot(t.slots + gr.bin);
-      if (rec == EMPTY) continue;
-      uint32_t rb[4];
-      bins_of(t, key_of(rec), rb);
-      y = rb[j];
-      if (y == gr.bin || vis_has(vis, vb, gen, y)) continue;
-      if (spawn_of(gr.meta) < 15) {
-        uint32_t nm = gr.meta + (1u << SPAWN_SHIFT);
-        if (cas_acquire(t.meta + gr.bin, gr.meta, nm)) {
-          G[g].meta = nm;
-        } else {
-          G[g].stale = 1;
-          uint32_t m = ld_acquire(t.meta + gr.bin);
-          for (int q = 0; q < 64 && spawn_of(m) < 15; q++) {  // bounded: a lost count is harmless
-            if (cas_acquire(t.meta + gr.bin, m, m + (1u << SPAWN_SHIFT))) break;
-            m = ld_acquire(t.meta + gr.bin);
-          }
-        }
-      }
-    }
-    if (c.viewed - c.viewed0 >= sp.budget || ng + nr >= sp.max_groups) { out = true; break; }  // budget spent
-    vis_insert(vis, vb, gen, y);
-    if (ORDER == P_BFS) k.spawned |= 1u << j;
-    c.viewed++;
-    prefetch_bin<1>(t, y);
-    rg[nr] = g;
-    ry[nr] = y;
-    nr++;
-  }
-  if (nr == 0) return dead_end(c);
-  for (uint32_t i = 0; i < nr; i++) {
-    const uint32_t g = rg[i], y = ry[i];
-    View<1> vy;
-    load_view_fast<1>(t, y, vy);
-    if (claimed_mask<1>(vy)) c.foreign = 1;
-    if (!free_mask<1>(vy)) {
-      push_dary<ORDER>(S, y, vy.m, g << 3);
-      continue;
-    }
-    // path: root group -> ... -> group g, one record each, in chain order
-    uint32_t depth = 1;
-    for (uint32_t q = g; G[q].parent != NO_PARENT; q = G[q].parent >> 3) depth++;
-    if ((int)depth + 4 > c.pcap) return ST_LONG;
-    {
-      uint32_t q = g;
-      for (int e = (int)depth - 1; e >= 0; e--) {
-        set_entry(c, e, pack_entry(G[q].bin, 0, K_MOVE, false, 0, 0), q);
-        if (G[q].parent != NO_PARENT) q = G[q].parent >> 3;
-      }
-    }
-    // claim the path in chain order from the metadata words as viewed; the
-    // record read after a claim is the one the search saw
-    c.pn = 0;
-    for (uint32_t e = 0; e < depth; e++) {
-      Group gq = G[(uint32_t)content_at(c, (int)e)];
-      if (gq.stale) return ST_CONFLICT;
-      if (!cas_acquire(t.meta + gq.bin, gq.meta, gq.meta + 1u)) return ST_CONFLICT;
-      c.pn = (int)e + 1;
-      const uint64_t r = reread<1>(t, gq.bin, 0);
-      const uint32_t to = e + 1 < depth ? G[(uint32_t)content_at(c, (int)e + 1)].bin : y;
-      set_content(c, (int)e, r);
-      if (!belongs<1>(t, r, to)) return ST_CONFLICT;
-    }
-    c.kicks = depth;
-    return take_free<1>(t, c, y, vy, 0, false);
-  }
-  if (out) return out_of_cap(c);
-  return SEARCHING;
+  if (STEP) return SEARCHING;
+  return search_rounds_dary<ORDER, false>(t, c, S);
 }
 
 template <int ORDER>
 __device__ int insert_search_dary(const DevTable& t, Ctx& c, uint8_t* region) {
   DarySearch S;
-  int r = search_first_dary<ORDER>(t, c, S, region);
-  while (r == SEARCHING) r = search_round_dary<ORDER>(t, c, S);
-  return r;
+  return search_first_dary<ORDER, false>(t, c, S, region);
 }
 
 

@@ -301,8 +301,8 @@ struct Lane {
   static __device__ __forceinline__ int begin(const DevTable& t, Ctx& c, State& w, uint8_t* region) {
     if constexpr (SEARCH) {
       if (!region) return ST_ABORTED;
-      if constexpr (B == 1) return search_first_dary<POL>(t, c, w, region);
-      else return search_first<B, POL, GHOST, NEAR>(t, c, w, region);
+      if constexpr (B == 1) return search_first_dary<POL, true>(t, c, w, region);
+      else return search_first<B, POL, GHOST, NEAR, true>(t, c, w, region);
     } else if constexpr (OWN) {
       return walk_begin<B, POL>(t, c, w);
     } else if constexpr (B == 1) {
@@ -315,8 +315,8 @@ struct Lane {
   }
   static __device__ __forceinline__ int step(const DevTable& t, Ctx& c, State& w) {
     if constexpr (SEARCH) {
-      if constexpr (B == 1) return search_round_dary<POL>(t, c, w);
-      else return search_round<B, POL, GHOST, NEAR>(t, c, w);
+      if constexpr (B == 1) return search_rounds_dary<POL, true>(t, c, w);
+      else return search_rounds<B, POL, GHOST, NEAR, true>(t, c, w);
     } else if constexpr (OWN) {
       return walk_step<B, POL>(t, c, w);
     } else if constexpr (B == 1) {
