@@ -83,8 +83,8 @@ struct Ctx {
   uint64_t* pe;
   int pn;
   int pcap;
-  int long_id;    // scratch plan in use (index in the table's pool), or -1
-  int big_id;     // scratch plan region lent to a search as its larger space, or -1
+  int long_id;    // scratch plan in use (index in the table's pool), or negative
+  int big_id;     // scratch plan region lent to a search as its larger space, or negative
   uint64_t held;  // d-ary walks: the record in hand
 };
 
@@ -143,16 +143,39 @@ __device__ __forceinline__ void release_long(const DevTable& t, int r) {
   atomicExch(t.long_busy + r, 0u);
 }
 
-// The local plan is full: copy the chain into a scratch plan and go on.
-__device__ __forceinline__ bool grow_plan(const DevTable& t, Ctx& c) {
-  if (c.long_id >= 0) return false;
-  int id = acquire_long(t, c.key);
-  if (id < 0) return false;
+// One look for a free scratch plan, without waiting: eight flags from a place
+// that h gives, read together (a pool has at least eight).
+__device__ __forceinline__ int try_long(const DevTable& t, uint32_t h) {
+  const uint32_t start = h % t.n_long;
+  uint32_t busy[8];
+#pragma unroll
+  for (uint32_t u = 0; u < 8; u++) {
+    const uint32_t r = start + u;
+    busy[u] = *(volatile uint32_t*)(t.long_busy + (r < t.n_long ? r : r - t.n_long));
+  }
+#pragma unroll
+  for (uint32_t u = 0; u < 8; u++) {
+    const uint32_t r = start + u < t.n_long ? start + u : start + u - t.n_long;
+    if (busy[u] == 0 && atomicCAS(t.long_busy + r, 0u, 1u) == 0u) return (int)r;
+  }
+  return -1;
+}
+
+// The local plan is full: the chain goes on in scratch plan id ...
+__device__ __forceinline__ void use_plan(const DevTable& t, Ctx& c, int id) {
   uint64_t* le = reinterpret_cast<uint64_t*>(t.long_scratch + (uint64_t)id * LONG_REGION);
   for (int i = 2 * REG_ENTRIES; i < 2 * c.pn; i++) le[i] = c.pe[i];
   c.pe = le;
   c.pcap = LONG_CHAIN;
   c.long_id = id;
+}
+
+// ... which is waited for.
+__device__ __forceinline__ bool grow_plan(const DevTable& t, Ctx& c) {
+  if (c.long_id >= 0) return false;
+  int id = acquire_long(t, c.key);
+  if (id < 0) return false;
+  use_plan(t, c, id);
   return true;
 }
 

@@ -855,14 +855,17 @@ __device__ __forceinline__ void release_slabs(const DevTable& t, const int* slab
   for (int j = 0; j < (int)((blockDim.x + SLAB - 1) / SLAB); j++) atomicExch(t.slab_busy + slabs[j], 0u);
 }
 
-// A larger search space (search_space) for the retries of a key, or -1.
+// A scratch plan that becomes a larger search space (search_space): it held a
+// plan or an earlier search, and its visited set starts without tags.
+__device__ __forceinline__ void clear_big_space(uint8_t* region) {
+  uint64_t* vis = reinterpret_cast<uint64_t*>(region + SEARCH_HDR + BIG_GROUPS * sizeof(Group));
+  for (int i = 0; i < BIG_VISITED; i++) vis[i] = 0;
+}
+
+// A larger search space for the retries of a key, or -1.
 __device__ __forceinline__ int take_big_space(const DevTable& t, uint32_t key) {
   const int id = acquire_long(t, key ^ 0x5bd1e995u);
-  if (id >= 0) {
-    uint64_t* vis = reinterpret_cast<uint64_t*>(t.long_scratch + (uint64_t)id * LONG_REGION + SEARCH_HDR +
-                                                BIG_GROUPS * sizeof(Group));
-    for (int i = 0; i < BIG_VISITED; i++) vis[i] = 0;  // the region held a plan: no stale tags
-  }
+  if (id >= 0) clear_big_space(t.long_scratch + (uint64_t)id * LONG_REGION);
   return id;
 }
 

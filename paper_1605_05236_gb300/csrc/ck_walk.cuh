@@ -346,8 +346,10 @@ __device__ __forceinline__ void walk_keys(Src& src, uint64_t* local_e, uint8_t* 
   using L = Lane<B, POL, GHOST>;
   constexpr bool SEARCH = L::SEARCH;
   // a lane has no key; has one whose next attempt begins; walks; has an
-  // attempt that ended with st; waits before its next attempt
+  // attempt that ended with st; waits, before its next attempt or for a
+  // scratch plan (searches)
   enum Mode { IDLE, READY, WALKING, ENDED, WAITING };
+  constexpr int WANT_BIG = -2;
   int mode = IDLE, st = ST_OK;
   Ctx c;
   c.ghosts_made = c.dup_evict = 0;
@@ -355,7 +357,39 @@ __device__ __forceinline__ void walk_keys(Src& src, uint64_t* local_e, uint8_t* 
   typename L::State w;
   uint32_t fails = 0, aborts = 0, wake = 0;
   for (;;) {
-    if (mode == WAITING && (int)((uint32_t)clock() - wake) >= 0) mode = READY;
+    if (mode == WAITING && (int)((uint32_t)clock() - wake) >= 0) {
+      mode = READY;
+      // A search that ran out of budget (WANT_BIG), or whose path outgrew its
+      // plan, asks the pool for a scratch plan and waits for the next time to
+      // ask beside the other lanes, among them holders of plans (polling in
+      // place held all of them up: BFS, 2^22 x 4 filled to 0.982, 4.3 s and
+      // 56,200 keys FAILED against 2.2 s and 38,900).  It asks for about as long as
+      // acquire_long polls and then goes on without.  A negative long_id or
+      // big_id counts the times.
+      if (SEARCH && (st == ST_LONG || c.big_id <= WANT_BIG)) {
+        const DevTable& t = src.table();
+        const bool plan = st == ST_LONG;
+        int id = plan ? c.long_id : c.big_id;
+        const int got = try_long(t, fmix32(c.key - (uint32_t)id));
+        if (got >= 0) {
+          id = got;
+          if (plan) use_plan(t, c, got);
+          else clear_big_space(t.long_scratch + (uint64_t)got * LONG_REGION);
+        } else if (id > -(int)(256 + 40 * t.n_long)) {
+          id--;
+          wake = (uint32_t)clock() + 2 * backoff_ns(5, c.key - (uint32_t)id);
+          mode = WAITING;
+        } else {
+          id = -1;
+          if (plan) {
+            st = ST_ABORTED;
+            mode = ENDED;
+          }
+        }
+        if (plan) c.long_id = id;
+        else c.big_id = id;
+      }
+    }
     const unsigned walking = __ballot_sync(0xFFFFFFFFu, mode == WALKING);
     const unsigned waiting = __ballot_sync(0xFFFFFFFFu, mode == WAITING);
     const unsigned need = __ballot_sync(0xFFFFFFFFu, mode == ENDED || mode == READY || (mode == IDLE && src.more));
@@ -374,16 +408,17 @@ __device__ __forceinline__ void walk_keys(Src& src, uint64_t* local_e, uint8_t* 
           const bool ran_out = st == ST_FAILED || c.capped;
           const bool longer = SEARCH && st == ST_LONG;  // the path goes on in a scratch plan
           if (longer) {
-            over = c.long_id >= 0 || !grow_plan(src.table(), c);
-            if (over) st = c.long_id >= 0 ? ST_FAILED : ST_ABORTED;
-            else mode = READY;
+            over = c.long_id >= 0;
+            if (over) st = ST_FAILED;
+            wake = (uint32_t)clock();
+            mode = WAITING;
           } else if (SEARCH && st == ST_ABORTED) {  // no search region
             over = true;
           } else if (ran_out) {
             over = ++fails > (st == ST_FAILED ? 6u : 32u);
             if (over) st = ST_FAILED;
             // a search out of budget tries again in a larger space
-            if (SEARCH && !over && c.big_id < 0) c.big_id = take_big_space(src.table(), c.key);
+            if (SEARCH && !over && c.big_id < 0) c.big_id = WANT_BIG;
           } else {
             aborts++;
           }
