@@ -228,7 +228,10 @@ int ck_clear(ck_table *t, void *stream);
 /* Copy the table to host memory (synchronous): slots (n_bins*B uint64) and
  * meta (n_bins uint32: bits 0-7 claim, 8-15 duplicate, 16-19 spawn count,
  * 20-27 hit counter, 28-31 version; d-ary: bit 0 claim, 8-15 rattle
- * counter).  Either pointer may be NULL. */
+ * counter).  Either pointer may be NULL.  The call reads the table and
+ * writes nothing of it (queue-kicking's words, which the device keeps as
+ * hits less occupied slots, are converted in a buffer of at most 16 MiB
+ * that the call allocates and frees). */
 int ck_export(ck_table *t, uint64_t *h_slots, uint32_t *h_meta);
 
 /* Restore a table from a snapshot ck_export wrote (synchronous): slots and
@@ -321,8 +324,10 @@ int ck_multi_create_on(ck_multi **out, void *dev_buf, size_t bytes, const ck_mul
 #define CK_MULTI_CHAIN_CAP 4
 int ck_multi_set_param(ck_multi *m, int key, int64_t value);
 
-/* Insert every table's keys: one persistent launch; blocks take tiles in
- * the order of a list interleaved over the tables.  Asynchronous. */
+/* Insert every table's keys by persistent launches (one for the 4-slot
+ * tables and one for the 8-slot ones; with ghosts one for all), which take
+ * tiles from a list: the tables a group that fits L2 at a time, the tiles
+ * of a group interleaved over its tables.  Asynchronous. */
 int ck_multi_insert(ck_multi *m, const uint32_t *d_keys, const uint32_t *d_vals, uint8_t *d_status,
                     void *stream);
 
@@ -347,9 +352,9 @@ int ck_multi_clear(ck_multi *m, void *stream);
 void ck_multi_destroy(ck_multi *m);
 
 /* A batched fill captured once and replayed as a CUDA graph: launching the
- * thousands of operations of a fill (a clear is three copies per table;
- * the per-table path launches one kernel per table) costs the host more
- * than the GPU spends on them, and a graph replays them with one call.
+ * thousands of operations of a fill (the per-table path launches one kernel
+ * per table) costs the host more than the GPU spends on them, and a graph
+ * replays them with one call; a clear is one launch.
  * ck_multi_capture records, on `stream` (NULL: a stream of the library's
  * own), an optional clear of every table (CK_MULTI_CAPTURE_CLEAR) followed
  * by ck_multi_insert -- or ck_multi_insert_per_table with

@@ -28,9 +28,12 @@
 // field (the release also folds in the duplicate/rattle update of the slot),
 // and the hit counter of queue-kicking moves on every kick-out -- unless
 // the word came back to the value seen (the 4-bit version wraps after 16
-// releases).  The writes themselves are therefore 64-bit compare-and-swaps
-// from the records the plan saw, undone if one fails, which closes that
-// gap.
+// releases).  So every move is checked once more: a walk reads the claimed slot
+// again with its next step and gives up if it no longer holds the record the
+// plan moves, a search checks the records it reads under its claims, and the
+// free slot or duplicate that ends a chain, ghost pairs, deletes and overwrites
+// are written by 64-bit compare-and-swaps from the record seen.  The other
+// writes of a chain, to slots claimed and checked, are plain stores.
 #pragma once
 #include <cstdint>
 #include <cuda/atomic>
@@ -241,14 +244,17 @@ __device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p) {
   return v;
 }
 
-// A read of a bin's slots that saw no claim bit in the bin's metadata word,
-// and finds the word unchanged when it is read again after the slots, saw
-// no key move: every move (a chain step, a delete) happens under a claim,
-// and every release advances the bin's version.  The one write without a
-// claim, a new key taking a free slot, adds a key and moves none.  This is
-// how a miss is proven while insertions run (a key moving between its own
-// bins is written to the new bin before it leaves the old one, but two
-// separate reads can still fall on either side of the move).
+// How a miss is proven while insertions run: the metadata words of all of the
+// key's bins are read, then the bins' slots, then the words again; if no word
+// showed a claim and none changed, the key did not move meanwhile.  A key moves
+// (a chain step, a delete) only while the slot it leaves is claimed, and the
+// release of that claim advances its bin's version.  The slot it moves to need
+// not be claimed -- a new key takes a free slot without a claim, and so does the
+// record a walk ends with (ck_walk.cuh) -- so the second bin's word need not
+// show the move: callers must have read every word before any slot
+// (read_words).  With words and slots read bin by bin, the key could be missed
+// in its second bin, read before it arrived, and in its first, whose word was
+// read after it had left.
 __device__ __forceinline__ bool unchanged_since(const uint32_t* meta, const uint32_t* bins, const uint32_t* seen,
                                                 uint32_t nb, uint32_t claim_bits) {
   fence_acquire();

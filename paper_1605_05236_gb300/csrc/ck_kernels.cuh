@@ -22,9 +22,9 @@ __device__ __forceinline__ int attempt_insert(const DevTable& t, Ctx& c, uint8_t
 }
 
 // One insertion with bounded retries after claim conflicts.  A chain that
-// outgrows the local plan continues in a scratch plan.  retry_failed: a
-// random walk that failed in concurrent mode is tried again with new draws
-// (up to 3 times): its path depended on the timing of other insertions.
+// outgrows the local plan continues in a scratch plan.  retry_failed: in
+// concurrent mode an attempt that ran out is made again (six times, 32 while
+// it meets other insertions' claims): its path depended on their timing.
 template <int B, int POL, bool GHOST>
 __device__ __forceinline__ int insert_one(const DevTable& t, Ctx& c, uint8_t* region, uint32_t& aborts,
                                           uint64_t* local_e, int local_cap, bool retry_failed = false) {

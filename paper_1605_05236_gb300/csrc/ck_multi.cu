@@ -2,16 +2,18 @@
 // of uneven sizes filled in one persistent launch.
 //
 // Each table is a full table (slots, metadata, counters) of its own and is
-// filled with exactly the per-insertion code of the single-table path
-// (insert_one: the kick-out policies of Sec. 3-7 with claim flags and
-// back-to-front chains, Sec. 8), so a key set gives the same key->value map
-// per table either way.  What the batched form changes is scheduling: the
-// keys of all tables are cut into tiles, a tile list is built once, and a
-// persistent grid pulls tiles from one global counter and keys within a
-// tile from a shared-memory counter.  Small tables no longer leave the GPU
-// idle and 4096 launches become one.  The reference path,
-// ck_multi_insert_per_table, launches the single-table kernel once per
-// table.
+// filled with the per-insertion code of the single-table path (the kick-out
+// policies of Sec. 3-7 with claim flags and back-to-front chains, Sec. 8), so
+// a key set gives the same key->value map per table either way.  What the
+// batched form changes is scheduling.  The keys of all tables are cut into
+// tiles, listed a group of tables that fits L2 at a time.  Walks
+// (k_multi_walk: queue-kicking and random kicking): each warp takes pieces of
+// 512 keys from the list, and its lanes walk in tables of their own, one launch
+// for the 4-slot tables and one for the 8-slot ones.  With ghosts
+// (k_multi_insert): each block takes a tile, and its threads the tile's keys.
+// Small tables no longer leave the GPU idle and 4096 launches become one or
+// two.  The reference path, ck_multi_insert_per_table, launches the
+// single-table kernel once per table.
 #include <cuda_runtime.h>
 
 #include <cstring>

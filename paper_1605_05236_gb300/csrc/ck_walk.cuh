@@ -270,8 +270,8 @@ __device__ __forceinline__ bool walk_commit(const DevTable& t, Ctx& c) {
 // 7.59, 7.37 and 7.16 (commits loading one entry at a time: 6.86 for 1/2 with
 // four at a time), from as many on 6.44, from twice as many on 6.33.
 //
-// 80 registers (3 blocks of 256 threads on an SM): 6.43 ms against 6.61 at
-// 64, which spill more.  One block waits for the launch before, which is
+// 80 registers (3 blocks of 256 threads on an SM; 4-slot queue-kicking spills
+// nothing): 6.43 ms against 6.61 at 64, which spill.  One block waits for the launch before, which is
 // enough to keep this one from completing first: blocks that are done make
 // room for the next launch's (6.43 against 6.46 with every block waiting).
 constexpr int WAITERS = 2;
