@@ -175,11 +175,18 @@ __device__ __forceinline__ uint64_t next_draw(Txn& x) {
   return splitmix64_at(x.rng);
 }
 
-// A random wait of less than 128 ns << k (at most 0.52 ms), different for
-// every worker and attempt; it draws nothing from the worker's sequence.
-__device__ void random_wait(const Txn& x, uint32_t k) {
+// A random wait of less than span ns (at most MAX_WAIT_NS), different for every
+// worker, attempt and k; it draws nothing from the worker's sequence.
+constexpr uint64_t MAX_WAIT_NS = 16ull * 1000 * 1000;
+__device__ void random_wait(const Txn& x, uint32_t k, uint64_t span) {
+  if (span > MAX_WAIT_NS) span = MAX_WAIT_NS;
   const uint64_t r = splitmix64_at(x.rng ^ ((uint64_t)x.epoch << 40) ^ k);
-  __nanosleep((uint32_t)r & ((128u << (k < 12 ? k : 12)) - 1));
+  const uint64_t until = now_ns() + (uint64_t)((double)(r >> 11) * 0x1p-53 * (double)span);
+  for (int n = 0; n < 4096; n++) {
+    const uint64_t now = now_ns();
+    if (now >= until) return;
+    __nanosleep((uint32_t)min(until - now, (uint64_t)16000));
+  }
 }
 
 // ---- the attempt's hash set of slots and bins in its read/write sets ----
@@ -795,14 +802,16 @@ __device__ bool lock_ws(const TxDev& t, Txn& x) {
 // holding locks could deadlock).  Two workers that each read a bin the other
 // writes set each other off: both wait for the other to unlock and then lock
 // again together, and with write sets of nearly one size they would stay in
-// step for every pass of every attempt.  A random wait before locking again,
-// up to about the time a pass takes once a few were in vain, separates them.
+// step for every pass of every attempt.  A random wait before locking again
+// separates them once it is longer than a pass holds its locks, so it is
+// measured by the pass: less than 1/32 of it at first, doubling to four times.
 __device__ bool stage2(const TxDev& t, Txn& x) {
   const bool local = t.flags & CK_TXF_LOCAL_RETRY;
   sort_lock_order(x);
   int passes = 0;
   uint32_t relocks = 0;
   while (passes < STAGE2_PASSES) {
+    const uint64_t begun = now_ns();
     if (!lock_ws(t, x)) return false;
     bool relock = false;
     while (!relock) {
@@ -873,7 +882,8 @@ __device__ bool stage2(const TxDev& t, Txn& x) {
       e.ver = w & ~3ull;
       atomicAdd(t.stats + TXS_LOCAL_RETRIES, 1ull);
     }
-    random_wait(x, 3 + ++relocks);
+    relocks++;
+    random_wait(x, relocks, ((now_ns() - begun) >> 6) << (relocks < 8 ? relocks : 8));
   }
   x.cause = TXS_ABORT_RS;
   return false;
@@ -1039,6 +1049,7 @@ __global__ void __launch_bounds__(32 * WORKERS_PER_BLOCK) k_txn_run(
     while (rc == 1 && a < ATTEMPTS_MAX && now_ns() - start < TIME_BUDGET_NS) {
       a++;
       tid = last;
+      const uint64_t begun = now_ns();
       rc = attempt(t, x, op + base, key + base, val + base, L, status ? status + out : nullptr,
                    value ? value + out : nullptr, tid, pos);
       if (rc == 1) {
@@ -1048,7 +1059,8 @@ __global__ void __launch_bounds__(32 * WORKERS_PER_BLOCK) k_txn_run(
         // eligible slot on every attempt: give those up
         if (x.cause == TXS_ABORT_OVERFLOW && ++overflows == OVERFLOWS_MAX) rc = 2;
         else if (x.cause == TXS_ABORT_CHAIN && ++chain_aborts == CHAIN_ABORTS_MAX) rc = 2;
-        else if (a > 16) random_wait(x, a - 16);  // attempts that keep meeting each other drift apart
+        else if (a > 16)  // attempts that keep meeting each other drift apart
+          random_wait(x, a, ((now_ns() - begun) >> 6) << (a < 24 ? a - 16 : 8));
       }
     }
     atomicAdd(t.stats + TXS_ATTEMPTS, (unsigned long long)a);

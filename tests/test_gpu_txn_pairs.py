@@ -48,8 +48,8 @@ def test_pairs_in_step_commit_at_once(flags, ins):
         tab.reset()
         out = tab.run(*dev, W, 1, L, flags)
         s = tab.stats()
-        assert s["failed"] == 0 and s["commits"] == W, s
-        assert s["attempts"] == W, s
+        assert s["failed"] == 0 and s["commits"] == W, str(s)
+        assert s["attempts"] == W, str(s)
         assert bool((out["status"] == 0).all())
         slots = tab.export(0)
         stored = np.sort((slots[slots != np.uint64(0xFFFFFFFFFFFFFFFF)] >> np.uint64(32)).astype(np.uint32))
